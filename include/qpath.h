@@ -93,15 +93,17 @@ typedef struct {
 
 /* qp_build_qubo flags */
 enum { QP_DENSE = 1, QP_STRUCTURED = 2, QP_DIST_I16 = 4 };
-/* qp_anneal_opts.kernel.  STRUCTURED uses the row-parallel kernel for fields
- * of up to 512 cells and the general one above; STRUCTURED_ROWS forces the
- * row-parallel kernel (up to 512 cells), STRUCTURED_FLAT the general structured
- * kernel (up to 4096 cells), STRUCTURED_GROUP the grouped kernel that anneals 4
- * replicas per warp up to 64 cells and 2 up to 128 (faster than the
- * row-parallel kernel at low temperature, slower at high temperature).  Above
- * 256 cells the row-parallel kernel keeps each replica's spins in global
- * memory (more replicas resident per SM); STRUCTURED_ROWS_SHARED forces the
- * variant with the spins in shared memory.  All give the same results. */
+/* qp_anneal_opts.kernel.  STRUCTURED (AUTO's choice for a handle with a
+ * structured form) is the event-driven kernel, for fields of any size: it
+ * passes over the proposals that cannot be accepted in groups, by bounds that
+ * hold for the current state.  The others evaluate every proposal:
+ * STRUCTURED_ROWS forces the row-parallel kernel (up to 512 cells),
+ * STRUCTURED_FLAT the general structured kernel (up to 4096 cells),
+ * STRUCTURED_GROUP the grouped kernel that anneals 4 replicas per warp up to
+ * 64 cells and 2 up to 128.  Above 256 cells the row-parallel kernel keeps each
+ * replica's spins in global memory (more replicas resident per SM);
+ * STRUCTURED_ROWS_SHARED forces the variant with the spins in shared memory.
+ * All give the same results. */
 enum {
   QP_KERNEL_AUTO = 0,
   QP_KERNEL_DENSE = 1,
@@ -112,8 +114,8 @@ enum {
   QP_KERNEL_STRUCTURED_ROWS_SHARED = 6
 };
 
-/* qp_anneal_opts.flags.  QP_ANNEAL_SKIP_SETTLED lets the row-parallel kernel
- * (fields of up to 512 cells, also in qp_batch_*) skip a sweep whose outcome
+/* qp_anneal_opts.flags.  QP_ANNEAL_SKIP_SETTLED lets the event-driven kernel
+ * and the row-parallel one (also in qp_batch_*) skip a sweep whose outcome
  * is already known: once a sweep of a replica met no proposal with dE < len
  * (none accepted outright, none needing a draw), its state cannot change in
  * any later sweep whose table is no longer (len non-increasing, as on a
@@ -123,8 +125,8 @@ enum { QP_ANNEAL_SKIP_SETTLED = 1 };
 
 typedef struct {
   int32_t kernel;            /* QP_KERNEL_*; AUTO = structured when built     */
-  int32_t replicas_per_cta;  /* warps (= replicas) per CTA; 0 = chosen to keep
-                                the most chains resident at once (occupancy) */
+  int32_t replicas_per_cta;  /* warps (= replicas) per CTA; 0 = chosen from the
+                                number of replicas and the occupancy        */
   int32_t replica_offset;    /* global index of replica 0 (its RNG stream)    */
   int64_t *accepts_out;      /* optional [R]: accepted flips per replica      */
   int32_t flags;             /* QP_ANNEAL_* bits                              */
@@ -379,8 +381,7 @@ qp_status qp_anneal_timed(qp_handle *h, int32_t replicas, const qp_schedule *sch
  * chain; best_out G*M (NULL allowed) the best feasible E of each chain at
  * any sweep end; levels_out G*M int32 (NULL allowed) each chain's final
  * level; swaps_out G*(M-1) int64 (NULL allowed) accepted trades of each
- * pair of levels.  Fields of up to 512 cells use the row kernel, larger ones
- * the flat kernel.  Asynchronous on cuda_stream when every output is device
+ * pair of levels.  The sweeps run on the event-driven kernel.  Asynchronous on cuda_stream when every output is device
  * memory; calls on one handle must not overlap (they share its buffers).
  * QP_ERANGE if two levels are so close that the exchange temperature
  * exceeds 1e8. */

@@ -76,8 +76,7 @@ extern "C" qp_status qp_batch_create(qp_handle *const *hs, int32_t count, int32_
     const qp_handle *h = hs[f];
     StructArgs &a = fa[f];
     a = StructArgs{};
-    a.C = h->C; a.Cp = h->Cp; a.start = h->start; a.A = h->A; a.B = h->B;
-    a.d = h->d_dev.p;
+    fill_field_args(h, a);
     a.R = R; a.rep_offset = 0;
     a.sweep_begin = sc->sweep_begin; a.sweep_end = sc->sweep_end;
     const uint64_t sf = seed + (uint64_t)f;

@@ -345,7 +345,29 @@ static qp_status build_field_qubo(const qp_field *f, int32_t A, int32_t B, int32
   QP_CU(cudaMemcpy(h->d32_dev.p, h->d.data(), (size_t)C * C * 4, cudaMemcpyHostToDevice));
   {
     const size_t es = h->d_i16 ? 2 : 4;
-    std::vector<uint8_t> pad((size_t)C * h->Cp * es, 0);
+    // after the matrix: the cells' grid coordinates and d by grid difference
+    const int r0 = *std::min_element(cr.begin(), cr.end()), c0 = *std::min_element(cc.begin(), cc.end());
+    const int rows = *std::max_element(cr.begin(), cr.end()) - r0 + 1, cols = *std::max_element(cc.begin(), cc.end()) - c0 + 1;
+    while ((1 << h->tab_sh) < cols) ++h->tab_sh;
+    if (rows <= 256 && cols <= 256 && (size_t)(rows << h->tab_sh) * es <= 32 * 1024) h->tab_n = rows << h->tab_sh;
+    h->xy_at = (size_t)C * h->Cp * es;
+    h->tab_at = h->xy_at + (size_t)h->Cp * 2;
+    std::vector<uint8_t> pad(h->tab_at + (size_t)h->tab_n * es, 0);
+    if (h->tab_n) {
+      for (int i = 0; i < C; ++i) {
+        const uint16_t v = (uint16_t)((cr[i] - r0) << 8 | (cc[i] - c0));
+        std::memcpy(pad.data() + h->xy_at + 2 * (size_t)i, &v, 2);
+      }
+      for (int dr = 0; dr < rows; ++dr)
+        for (int dc = 0; dc < cols; ++dc) {
+          const int32_t v = (int32_t)std::min<int64_t>(round_scaled_sqrt((int64_t)dr * dr + (int64_t)dc * dc, scale),
+                                                       h->d_i16 ? INT16_MAX : INT32_MAX);
+          const int16_t v16 = (int16_t)v;
+          uint8_t *at = pad.data() + h->tab_at + (((size_t)dr << h->tab_sh) + dc) * es;
+          if (h->d_i16) std::memcpy(at, &v16, 2);
+          else std::memcpy(at, &v, 4);
+        }
+    }
     for (int i = 0; i < C; ++i)
       for (int j = 0; j < C; ++j) {
         const int32_t v = h->d[(size_t)i * C + j];
@@ -480,7 +502,7 @@ extern "C" qp_status qp_device_checks(int32_t *enabled, uint32_t *first_failure)
   *enabled = qp::chk::enabled();
   uint32_t w = 0;
   bool read_failed = false;
-  for (uint32_t (*take)() : {qp::chk::rows, qp::chk::kernels, qp::chk::group, qp::chk::repair}) {
+  for (uint32_t (*take)() : {qp::chk::rows, qp::chk::kernels, qp::chk::group, qp::chk::events, qp::chk::repair}) {
     const uint32_t v = take();
     if (v == 0xFFFFFFFFu) {  // the record could not be read from the device
       read_failed = true;
@@ -511,6 +533,23 @@ extern "C" qp_status qp_thresholds(const qp_schedule *sc, int32_t sweep, uint32_
 // --------------------------------------------------------------------------- anneal
 namespace qp {
 namespace host {
+
+void fill_field_args(const qp_handle *h, StructArgs &a) {
+  a.C = h->C; a.Cp = h->Cp; a.start = h->start; a.A = h->A; a.B = h->B;
+  a.d = h->d_dev.p;
+  a.xy = reinterpret_cast<const uint16_t *>(h->d_dev.as<uint8_t>() + h->xy_at);
+  a.tab = h->d_dev.as<uint8_t>() + h->tab_at;
+  a.tab_sh = h->tab_sh; a.tab_n = h->tab_n;
+}
+
+qp_status launch_structured_events(qp_handle *h, StructArgs &a, int W, cudaStream_t st, LaunchInfo *info) {
+  if (const size_t words = events_state_words(h->C)) {
+    QP_TRY(h->gstate.ensure((size_t)a.R * words * 4));
+    a.gstate = h->gstate.as<uint32_t>();
+  }
+  QP_CU(launch_events(a, h->d_i16, W, st, info));
+  return QP_OK;
+}
 
 // The structured sweep of a.R replicas: the row kernel when allowed and the
 // field fits it, else the flat kernel (spins in global memory when a
@@ -615,8 +654,7 @@ extern "C" qp_status qp_anneal_ex(qp_handle *h, int32_t R, const qp_schedule *sc
   if (structured) {
     int W = o.replicas_per_cta ? o.replicas_per_cta : 4;
     StructArgs a{};
-    a.C = h->C; a.Cp = h->Cp; a.start = h->start; a.A = h->A; a.B = h->B;
-    a.d = h->d_dev.p;
+    fill_field_args(h, a);
     a.R = R; a.rep_offset = o.replica_offset;
     a.sweep_begin = sc->sweep_begin; a.sweep_end = sc->sweep_end;
     a.key0 = key0; a.key1 = key1;
@@ -629,6 +667,10 @@ extern "C" qp_status qp_anneal_ex(qp_handle *h, int32_t R, const qp_schedule *sc
       while (Wg > 1 && !group_supported(h->C, h->d_i16, Wg)) --Wg;
       if (!group_supported(h->C, h->d_i16, Wg)) return fail(QP_ERANGE, "grouped kernel: no launch fits");
       QP_CU(launch_group(a, h->d_i16, Wg, st, &info));
+      goto launched;
+    }
+    if (kernel == QP_KERNEL_STRUCTURED) {
+      QP_TRY(launch_structured_events(h, a, o.replicas_per_cta, st, &info));
       goto launched;
     }
     // replicas per CTA as asked, else chosen for the most resident chains

@@ -120,9 +120,11 @@ struct qp_handle {
   int64_t n = 0, c0 = 0;
   std::vector<int32_t> d;  // C x C (host)
   // device data
-  qp::host::DevBuf d_dev;            // C x Cp, int16 or int32
+  qp::host::DevBuf d_dev;            // C x Cp, int16 or int32; then the cells' coordinates and the distance table
   bool d_i16 = false;
   int32_t Cp = 0;
+  size_t xy_at = 0, tab_at = 0;      // byte offsets of both in d_dev
+  int32_t tab_sh = 0, tab_n = 0;     // tab_n = 0: the grid is too large for a table
   qp::host::DevBuf d32_dev;          // C x C int32 (decode, dense build)
   qp::host::DevBuf S_dev;            // n x np, int16 or int32
   bool has_dense = false, S_i16 = false;
@@ -139,10 +141,14 @@ struct qp_handle {
 
 namespace qp {
 namespace host {
+// The field's part of a structured launch's arguments.
+void fill_field_args(const qp_handle *h, StructArgs &a);
 // The structured sweep of a.R replicas: the row kernel when allowed and the
 // field fits it, else the flat kernel.
 // W = replicas per CTA, 0 = chosen from the occupancy (row kernel) or 4 (flat kernel)
 qp_status launch_structured_auto(qp_handle *h, StructArgs &a, int W, bool allow_rows, cudaStream_t st,
                                  LaunchInfo *info, bool rows_shared_spins = false);
+// The event-driven sweep of a.R replicas.
+qp_status launch_structured_events(qp_handle *h, StructArgs &a, int W, cudaStream_t st, LaunchInfo *info);
 }  // namespace host
 }  // namespace qp

@@ -49,6 +49,12 @@ struct StructArgs {
   const int32_t *level;
   // QP_ANNEAL_SKIP_SETTLED: skip sweeps that provably change nothing
   int32_t skip_settled;
+  // d as a function of the cells' grid differences: xy[i] = row << 8 | column
+  // (from the field's first row and column with a cell), tab[(|dr| << tab_sh)
+  // + |dc|] in d's type; tab_n = 0 when the grid is too large for it.
+  const uint16_t *xy;
+  const void *tab;
+  int32_t tab_sh, tab_n;
 };
 
 // Arguments of the dense sweep (one warp = one replica).
@@ -103,6 +109,11 @@ cudaError_t launch_rows_g(const StructArgs &a, bool d_i16, int warps_per_cta, in
                           long long *carry, int *err, cudaStream_t st, LaunchInfo *info);
 cudaError_t launch_rows(const StructArgs &a, bool d_i16, int warps_per_cta, cudaStream_t st,
                         LaunchInfo *info);
+// Event-driven structured kernel (qp_sweep_events.cu), any field: words of one
+// replica's bitsets in a.gstate (0: in shared memory) and the launch
+// (warps_per_cta 0 = chosen from the replica count).
+size_t events_state_words(int C);
+cudaError_t launch_events(const StructArgs &a, bool d_i16, int warps_per_cta, cudaStream_t st, LaunchInfo *info);
 // Batched persistent launch (qp_sweep_rows.cu): fields[] per field, units[]
 // = (field, replica) in processing order, counter = the work-queue head (zeroed
 // before each launch).  All fields must use int16 distances.
@@ -194,6 +205,7 @@ namespace chk {
 uint32_t kernels();
 uint32_t rows();
 uint32_t group();
+uint32_t events();
 uint32_t repair();
 int32_t enabled();
 }  // namespace chk

@@ -131,8 +131,7 @@ extern "C" qp_status qp_anneal_pt(qp_handle *h, int32_t G, const qp_pt_schedule 
   }
   uint8_t *cur = h->pt_states[0].as<uint8_t>(), *nxt = h->pt_states[1].as<uint8_t>();
   StructArgs a{};
-  a.C = h->C; a.Cp = h->Cp; a.start = h->start; a.A = h->A; a.B = h->B;
-  a.d = h->d_dev.p;
+  fill_field_args(h, a);
   a.R = R; a.rep_offset = 0;
   a.key0 = (uint32_t)seed; a.key1 = (uint32_t)(seed >> 32);
   a.thr = lt.thr; a.thr_off = lt.off; a.thr_len = lt.len; a.thr_c = lt.c;
@@ -150,7 +149,7 @@ extern "C" qp_status qp_anneal_pt(qp_handle *h, int32_t G, const qp_pt_schedule 
     a.sweep_end = (e + 1) * I;
     a.init = e == 0 ? init_d : cur;
     a.states_out = nxt;
-    QP_TRY(launch_structured_auto(h, a, 0, true, st, &info));
+    QP_TRY(launch_structured_events(h, a, 0, st, &info));
     x.phase = e & 1;
     x.round = e;
     QP_CU(launch_pt_exchange(x, st));

@@ -1,0 +1,720 @@
+// Event-driven structured sweep (sm_103a): the same sequential chain as the
+// row kernels, with the proposals that cannot be accepted passed over in
+// groups by bounds that hold for the current state.
+//
+// With r the sum of row t and c the sum of column i (both including x_{t,i})
+// and f = sum of d over the cells of rows t-1 and t+1, Eq. 6 gives
+//   x = 0:  dE = B f + 2A (r + c - 1),      x = 1:  dE = 2A (3 - r - c) - B f.
+// So a cell proposed into a row and a column that hold one between them at
+// least twice (r + c >= 2) costs dE >= 2A.  Such a proposal is accepted only
+// if its draw u is below thr[2A], and never when the table ends at or before
+// 2A: a test that does not look at the state.  What is left in a row with
+// r >= 1 are few columns: the row's own cells (x = 1), the empty columns
+// (c = 0) and the columns whose draw passed the test ("survivors").  At
+// T = 1000 that is 1 in 170 draws on a 10x10 field and 1 in 400,000 on a
+// 24x24 one; sweeps whose table ends at 2A have none and draw nothing.
+// A row without cells (r = 0) has no such bound: all its columns are evaluated.
+//
+// One warp anneals one replica.  A sweep goes through windows of 32 rows:
+//   draws   (only when len > 2A) every Philox block of the window, one per
+//           lane and step, each word compared with thr[2A]; the rows that have
+//           a survivor are kept as a mask.
+//   check   lane j looks at row t0 + j as the state stands: rows that do not
+//           hold exactly one cell, that have a survivor, or whose cell or an
+//           empty column would be accepted are events.  The first event row
+//           is found by one ballot; every row before it is final.
+//   event   the row evaluated exactly, 128 columns at a time (a lane takes the
+//           four columns of one Philox block), the first accepted proposal
+//           applied and the rest re-evaluated, in proposal order.
+// After an event the check resumes at the next row.  A sweep most of whose
+// rows are events goes from row to row without draws and checks of its own.
+// Every decision is the sequential chain's: the same words of the generator
+// against the same tables.
+//
+// What bounds it: the latency of one chain (a check is ~150 dependent cycles,
+// an event ~1500), and in hot sweeps of large fields the Philox multiplies.
+// Against the row kernels, which evaluate every column of every row (one GB300;
+// microseconds per sweep of all chains): 92 cells, 1024 chains: 161 -> 97 at
+// T = 1000 (1.2 flips a row), 72 -> 20 at T = 436, 20.9 -> 1.8 below T = 115;
+// 491 cells, 4096 chains x 1000 sweeps: 899 -> 109 ms; 893 cells, 512 chains x
+// 40 sweeps (the general kernel): 272 -> 25.9 ms.  It is also the faster one far
+// above the temperatures of a useful schedule (T = 1e6, a third of the cells
+// set: 1.5 to 2.2 times), so every structured launch uses it.
+#include <algorithm>
+#include <climits>
+
+#include "qp_device.cuh"
+#include "qp_internal.h"
+
+namespace qp {
+namespace {
+
+using namespace dev;
+
+__device__ __forceinline__ int sel4(const int (&v)[4], int j) {
+  return j == 0 ? v[0] : (j == 1 ? v[1] : (j == 2 ? v[2] : v[3]));
+}
+
+constexpr int kZCheck = 4;    // most empty columns the check looks at; above, rows are processed one by one
+constexpr int kRowCells = 3;  // cells of a row kept in its record
+constexpr int kPad = 8;       // entries before and after the arrays read by four columns at a time
+
+__host__ __device__ constexpr size_t align16e(size_t x) { return (x + 15) & ~size_t(15); }
+
+// A row's record: its number of cells and, when there are at most three, the
+// cells themselves; of a row with more, one of its cells (c0).  The bits hold
+// every row.
+struct Row {
+  int n, c0, c1, c2;
+};
+__device__ __forceinline__ Row unpack_row(uint2 q) {
+  return Row{(int)(q.x & 0xFFFFu), (int)(q.x >> 16), (int)(q.y & 0xFFFFu), (int)(q.y >> 16)};
+}
+__device__ __forceinline__ uint2 pack_row(int n, int c0, int c1, int c2) {
+  return make_uint2((uint32_t)n | ((uint32_t)c0 << 16), (uint32_t)c1 | ((uint32_t)c2 << 16));
+}
+
+// d_{h,i}: from the matrix in global memory (DM = 0) or in shared memory
+// (DM = 1), or from the field's table over (|row difference|, |column
+// difference|) in shared memory (DM = 2: 24x24 cells take 1.5 KB instead of
+// the matrix's 482 KB).
+template <typename DT, int DM>
+struct Dist {
+  const DT *m;
+  int Cp, C;
+  const uint16_t *xy;  // row << 8 | column of every cell
+  int sh, tab_n;
+  __device__ __forceinline__ int lookup(uint32_t a, uint32_t b) const {
+    const uint32_t ad = __vabsdiffu4(a, b);
+    return (int)m[QP_IX((int)(((ad >> 8) << sh) + (ad & 0xFFu)), tab_n, 2)];
+  }
+  __device__ __forceinline__ int operator()(int h, int i) const {
+    if (DM == 2) return lookup(xy[QP_IX(h, C, 2)], xy[QP_IX(i, C, 2)]);
+    const int k = QP_IX(h * Cp + i, C * Cp, 2);
+    return DM == 1 ? (int)m[k] : (int)__ldg(m + k);
+  }
+  // f[j] += d_{h,i+j}, -4 < i <= C; columns outside the field give anything.
+  // xi: the columns' coordinates (DM = 2).
+  __device__ __forceinline__ void add4(int h, int i, const uint32_t (&xi)[4], int (&f)[4]) const {
+    if (DM == 2) {
+      const uint32_t a = xy[QP_IX(h, C, 2)];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) f[j] += lookup(a, xi[j]);
+    } else if (DM == 1) {
+      const DT *p = m + QP_IX(h, C, 2) * Cp + i;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) f[j] += (int)p[j];
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) f[j] += (int)__ldg(m + min(max(h * Cp + i + j, 0), C * Cp - 1));
+    }
+  }
+};
+
+// SB: the spins' bitsets are in shared memory (up to 256 cells, 8 KB a
+// replica); else in global memory (L2, flipped by atomics, read past L1).
+template <bool SB>
+__device__ __forceinline__ uint32_t bits_word(const uint32_t *p) {
+  if (SB) return *p;
+  return __ldcg(p);
+}
+
+// Sum of d over the cells of row u (whose record is q), for this lane's column i.
+template <typename DT, int DM, bool SB>
+__device__ __forceinline__ int row_sum_d(const Row &q, int u, const uint32_t *bits, int Cw, int C,
+                                         const Dist<DT, DM> &D, int i) {
+  int f = 0;
+  if (q.n <= kRowCells) {
+    if (q.n > 0) f = D(q.c0, i);
+    if (q.n > 1) f += D(q.c1, i);
+    if (q.n > 2) f += D(q.c2, i);
+  } else {
+    for (int w = 0; w < Cw; ++w) {
+      uint32_t wd = bits_word<SB>(bits + QP_IX(u * Cw + w, C * Cw, 3));
+      while (wd) {
+        f += D((w << 5) + __ffs(wd) - 1, i);
+        wd &= wd - 1;
+      }
+    }
+  }
+  return f;
+}
+
+// Row t's record from its bits (r cells); of a row with more than three, one
+// of its cells.
+template <bool SB>
+__device__ __forceinline__ uint2 record_from_bits(const uint32_t *bits, int Cw, int C, int t, int r, int lane) {
+  int c[3] = {0, 0, 0}, k = 0;
+  const int want = r <= kRowCells ? r : 1;
+  for (int w0 = 0; w0 < Cw && k < want; w0 += 32) {
+    const uint32_t word = w0 + lane < Cw ? bits_word<SB>(bits + QP_IX(t * Cw + w0 + lane, C * Cw, 3)) : 0u;
+    for (uint32_t b = __ballot_sync(kFull, word != 0); b && k < want; b &= b - 1) {
+      const int w = __ffs(b) - 1;
+      for (uint32_t wd = __shfl_sync(kFull, word, w); wd && k < want; wd &= wd - 1) {
+        const int i = ((w0 + w) << 5) + __ffs(wd) - 1;
+        if (k == 0) c[0] = i;
+        else if (k == 1) c[1] = i;
+        else c[2] = i;
+        ++k;
+      }
+    }
+  }
+  return pack_row(r, c[0], c[1], c[2]);
+}
+
+// The sweeps of one replica.  rec: C + 1 row records (the last stays empty),
+// cc: column sums with kPad entries on both sides, bits: C x Cw words.
+template <typename DT, int DM, bool SB, typename KEY>
+__device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uint2 *rec, uint16_t *cc, uint32_t *bits,
+                                               const Dist<DT, DM> &D, int lane, const KEY &key) {
+  const int C = a.C, s0 = a.start, B = a.B, twoA = 2 * a.A;
+  const int Cw = (C + 31) >> 5;
+  const int n = C * C;
+  const uint32_t rg = (uint32_t)(a.rep_offset + rep);
+  const uint32_t magic = (uint32_t)((0x100000000ull + (uint32_t)C - 1) / (uint32_t)C);  // x / C = umulhi(x, magic), x < 2^18
+
+  // ---- initial state: given or all zero; row 0 and column s clamped (x_{0,s} = 1)
+  for (int i = lane; i < C + 2 * kPad; i += 32) cc[i - kPad] = 0;
+  for (int e = lane; e < C * Cw; e += 32) bits[e] = 0;
+  for (int t = lane; t <= C; t += 32) rec[t] = make_uint2(0, 0);
+  __syncwarp();
+  if (lane == 0) {
+    bits[s0 >> 5] = 1u << (s0 & 31);
+    rec[0] = pack_row(1, s0, 0, 0);
+    cc[s0] = 1;
+  }
+  __syncwarp();
+  if (a.init) {
+    // the bytes that are set, found 16 at a time
+    const uint8_t *x = a.init + (size_t)rep * n;
+    auto set = [&](int k) {
+      const int t = k / C, i = k - t * C;
+      if (t == 0 || i == s0) return;
+      atomicOr(bits + QP_IX(t * Cw + (i >> 5), C * Cw, 3), 1u << (i & 31));
+      const int at = (int)(atomicAdd(&rec[t].x, 1u) & 0xFFFFu);
+      if (at == 0) atomicOr(&rec[t].x, (uint32_t)i << 16);
+      else if (at < kRowCells) atomicOr(&rec[t].y, (uint32_t)i << (at == 1 ? 0 : 16));
+      uint32_t *cw = reinterpret_cast<uint32_t *>(cc - kPad) + ((i + kPad) >> 1);
+      atomicAdd(cw, (i & 1) ? 0x10000u : 1u);
+    };
+    const int head = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(x) & 15)) & 15));
+    const int nv = (n - head) / 16;
+    if (lane < head && x[lane]) set(lane);
+    for (int v0 = 0; v0 < nv; v0 += 128) {
+      uint4 q[4];
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        const int v = v0 + 32 * g + lane;
+        q[g] = v < nv ? __ldg(reinterpret_cast<const uint4 *>(x + head) + v) : make_uint4(0, 0, 0, 0);
+      }
+#pragma unroll
+      for (int g = 0; g < 4; ++g) {
+        if ((q[g].x | q[g].y | q[g].z | q[g].w) == 0) continue;
+        const int k0 = head + 16 * (v0 + 32 * g + lane);
+        for (int b = 0; b < 16; ++b)
+          if ((word_of(q[g], b >> 2) >> (8 * (b & 3))) & 0xFFu) set(k0 + b);
+      }
+    }
+    for (int k = head + 16 * nv + lane; k < n; k += 32)
+      if (x[k]) set(k);
+    __syncwarp();
+  }
+  // ---- energy (Eqs. 3-6), violation count, empty columns
+  long long E;
+  int viol, nz;
+  {
+    long long hd = 0, pen = 0;
+    int v = 0, z = 0;
+    for (int t = lane; t < C; t += 32) {
+      const Row q = unpack_row(rec[t]);
+      pen += (long long)(1 - q.n) * (1 - q.n);
+      v += q.n != 1;
+      if (a.init && t + 1 < C && q.n > 0) {
+        const Row p = unpack_row(rec[t + 1]);
+        if (q.n <= kRowCells) {
+          hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c0);
+          if (q.n > 1) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c1);
+          if (q.n > 2) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c2);
+        } else {
+          for (int w = 0; w < Cw; ++w) {
+            uint32_t wd = bits_word<SB>(bits + t * Cw + w);
+            while (wd) {
+              hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, (w << 5) + __ffs(wd) - 1);
+              wd &= wd - 1;
+            }
+          }
+        }
+      }
+    }
+    for (int i = lane; i < C; i += 32) {
+      const int c = cc[i];
+      pen += (long long)(1 - c) * (1 - c);
+      v += c != 1;
+      z += c == 0;
+    }
+    E = (long long)B * warp_sum64(hd) + (long long)a.A * warp_sum64(pen);
+    viol = __reduce_add_sync(kFull, v);
+    nz = __reduce_add_sync(kFull, z);
+  }
+  long long best = LLONG_MAX, acc = 0;
+  int zreg = 0;          // lane q < nz: an empty column (when zok)
+  bool zok = nz == 0;
+  int rows_flipped = 2 * viol;  // rows the last sweep changed; at first, a guess from the state
+
+  // ---- sweeps.  The table's place, length and log2(e)/T of a sweep are
+  // loaded two sweeps ahead, thr[2A] one ahead, so no sweep waits for them.
+  const int lev = a.level ? __ldg(a.level + rep) : -1;
+  const int last = a.sweep_end - 1;
+  auto row_of = [&](int s) { return lev >= 0 ? lev : min(s, last); };
+  long long off1 = 0, off2 = 0;
+  int len1 = 0, len2 = 0;
+  float c1 = 0.0f, c2 = 0.0f;
+  uint32_t q1 = 0;
+  if (a.sweep_begin < a.sweep_end) {
+    const int u1 = row_of(a.sweep_begin), u2 = row_of(a.sweep_begin + 1);
+    off1 = a.thr_off[u1]; len1 = a.thr_len[u1]; c1 = a.thr_c[u1];
+    off2 = a.thr_off[u2]; len2 = a.thr_len[u2]; c2 = a.thr_c[u2];
+    if (len1 > twoA) q1 = __ldg(a.thr + off1 + twoA);
+  }
+  bool settled = false;
+  int settled_len = 0;
+  for (int s = a.sweep_begin; s < a.sweep_end; ++s) {
+    const uint32_t *thr = a.thr + off1;
+    const int len = len1;
+    const float cT = c1;
+    const uint32_t Q2 = q1;  // 0 when len <= 2A
+    off1 = off2; len1 = len2; c1 = c2;
+    q1 = len1 > twoA ? __ldg(a.thr + off1 + twoA) : 0u;
+    {
+      const int u2 = row_of(s + 2);
+      off2 = a.thr_off[u2]; len2 = a.thr_len[u2]; c2 = a.thr_c[u2];
+    }
+    if (settled && len <= settled_len) continue;
+    const bool hot = Q2 != 0;
+    const float Tl = 1.0f / cT;                // T ln 2
+    const float margin = Tl * (1.0f / 512.0f);  // of the estimate below
+    const int band = (int)(2.0f * margin) + 2;
+    // row by row when half the rows are events anyway: rows changed in the last sweep, rows with survivors
+    const float lambda = (float)Q2 * 2.3283064365386963e-10f * (float)C;
+    const bool rowwise = (float)rows_flipped + 0.5f * lambda * (float)C > 0.5f * (float)C;
+    rows_flipped = 0;
+    bool hit = hot;  // a proposal with dE < len was met
+    for (int t0 = 1; t0 < C; t0 += 32) {
+      const int t1 = min(C, t0 + 32);
+      // -- draws of the window: the rows with survivors
+      uint32_t smask = 0;
+      if (hot && !rowwise) {
+        const uint32_t k0 = (uint32_t)(t0 * C), nk = (uint32_t)((t1 - t0) * C);
+        const uint32_t mend = (k0 + nk - 1) >> 2;
+        auto mark = [&](const uint4 &u, uint32_t m) {
+          const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const uint32_t rel = 4 * m + j - k0;
+            if (w[j] < Q2 && rel < nk) smask |= 1u << __umulhi(rel, magic);
+          }
+        };
+        for (uint32_t mb = k0 >> 2; mb <= mend; mb += 64) {
+          const uint32_t ma = mb + lane, mc = ma + 32;
+          const uint4 ua = philox4x32_10(make_uint4(ma, (uint32_t)s, rg, kRngTag), key);
+          const uint4 ub = philox4x32_10(make_uint4(mc, (uint32_t)s, rg, kRngTag), key);
+          const uint32_t la = min(min(ua.x, ua.y), min(ua.z, ua.w)), lb = min(min(ub.x, ub.y), min(ub.z, ub.w));
+          if (min(la, lb) < Q2) {
+            mark(ua, ma);
+            mark(ub, mc);
+          }
+        }
+        smask = __reduce_or_sync(kFull, smask);
+      }
+      // -- the window's rows
+      bool have_uh = false;
+      uint32_t uh = 0;  // the draw of the cell of row t0 + lane
+      for (int t = t0; t < t1; ++t) {
+        if (!rowwise && nz <= kZCheck) {
+          if (!zok) {  // list the empty columns
+            int k = 0;
+            for (int i0 = 0; i0 < C; i0 += 32) {
+              uint32_t b = __ballot_sync(kFull, i0 + lane < C && cc[i0 + lane] == 0);
+              while (b) {
+                if (lane == k) zreg = i0 + __ffs(b) - 1;
+                b &= b - 1;
+                ++k;
+              }
+            }
+            zok = true;
+          }
+          // the check: lane = row
+          const int tl = t0 + lane;
+          const bool in = tl >= t && tl < t1;
+          const int tr = min(tl, C - 1);
+          const Row p0 = unpack_row(rec[tr - 1]), p1 = unpack_row(rec[tr]), p2 = unpack_row(rec[tr + 1]);
+          bool ev = p1.n != 1 || p0.n > 1 || p2.n > 1 || ((smask >> lane) & 1u);
+          const int h = p1.c0;
+          int dE = len;
+          if (in && !ev) {
+            int f = 0;
+            if (p0.n) f = D(p0.c0, h);
+            if (p2.n) f += D(p2.c0, h);
+            dE = twoA * (2 - (int)cc[h]) - B * f;
+          }
+          bool need = dE < len;
+          if (__any_sync(kFull, need)) {
+            hit = true;
+            if (!have_uh) {
+              const uint32_t k = (uint32_t)(tr * C + h);
+              const uint4 u = philox4x32_10(make_uint4(k >> 2, (uint32_t)s, rg, kRngTag), key);
+              uh = word_of(u, k & 3);
+              have_uh = true;
+            }
+            if (need) ev = dE <= 0 || accept_draw(uh, dE, cT, thr, len);
+          }
+          for (int q = 0; q < nz; ++q) {
+            const int z = __shfl_sync(kFull, zreg, q);
+            dE = len;
+            if (in && !ev) {
+              int f = 0;
+              if (p0.n) f = D(p0.c0, z);
+              if (p2.n) f += D(p2.c0, z);
+              dE = B * f;
+            }
+            need = dE < len;
+            if (__any_sync(kFull, need)) {
+              hit = true;
+              const uint32_t k = (uint32_t)(tr * C + z);
+              const uint4 u = philox4x32_10(make_uint4(k >> 2, (uint32_t)s, rg, kRngTag), key);
+              if (need) ev = dE <= 0 || accept_draw(word_of(u, k & 3), dE, cT, thr, len);
+            }
+          }
+          const uint32_t bal = __ballot_sync(kFull, in && ev);
+          if (bal == 0) break;  // nothing happens in the rest of the window
+          t = t0 + __ffs(bal) - 1;
+        }
+        // -- event row t
+        hit = true;
+        const Row p0 = unpack_row(rec[t - 1]), p1 = unpack_row(rec[t]), p2 = unpack_row(rec[t + 1]);
+        const int tC = t * C;
+        int r = p1.n, l0 = p1.c0, l1 = p1.c1, l2 = p1.c2;
+        bool lost = p1.n > kRowCells, flipped = false;
+        const bool many = p0.n > 1 || p1.n > 1 || p2.n > 1;
+        const int h1 = p1.n > 0 ? p1.c0 : -8;
+        const uint32_t m1 = (uint32_t)(tC + C - 1) >> 2;
+        for (uint32_t mb = (uint32_t)tC >> 2; mb <= m1; mb += 32) {
+          const uint32_t m = mb + lane;
+          const uint4 u4 = philox4x32_10(make_uint4(m, (uint32_t)s, rg, kRngTag), key);
+          const int i0 = (int)(4 * m) - tC;  // the lane's columns i0 .. i0 + 3, -4 < i0
+          const int ic = min(i0, C);
+          int f[4] = {0, 0, 0, 0}, c[4];
+          uint32_t xi[4] = {0, 0, 0, 0};
+          if (DM == 2) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) xi[j] = D.xy[ic + j];
+          }
+#pragma unroll
+          for (int j = 0; j < 4; ++j) c[j] = cc[ic + j];
+          if (p0.n > 0) D.add4(p0.c0, ic, xi, f);
+          if (p2.n > 0) D.add4(p2.c0, ic, xi, f);
+          int xm = 0;  // x of the lane's columns
+#pragma unroll
+          for (int j = 0; j < 4; ++j) xm |= (int)(i0 + j == h1) << j;
+          if (many) {  // rows of several cells
+            if (p1.n > kRowCells) {
+              xm = 0;
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const int i = i0 + j;
+                if (i >= 0 && i < C)
+                  xm |= (int)((bits_word<SB>(bits + QP_IX(t * Cw + (i >> 5), C * Cw, 3)) >> (i & 31)) & 1u) << j;
+              }
+            } else if (p1.n > 1) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j)
+                xm |= (int)(i0 + j == p1.c1 || (p1.n > 2 && i0 + j == p1.c2)) << j;
+            }
+#pragma unroll 1
+            for (int side = -1; side <= 1; side += 2) {
+              const Row &p = side < 0 ? p0 : p2;
+              if (p.n > kRowCells) {  // the cells from the row's bits, but the one already added
+                for (int w0 = 0; w0 < Cw; w0 += 32) {
+                  uint32_t word = w0 + lane < Cw ? bits_word<SB>(bits + QP_IX((t + side) * Cw + w0 + lane, C * Cw, 3)) : 0u;
+                  if ((p.c0 >> 5) == w0 + lane) word &= ~(1u << (p.c0 & 31));
+                  for (uint32_t b = __ballot_sync(kFull, word != 0); b; b &= b - 1) {
+                    const int w = __ffs(b) - 1;
+                    for (uint32_t wd = __shfl_sync(kFull, word, w); wd; wd &= wd - 1)
+                      D.add4(((w0 + w) << 5) + __ffs(wd) - 1, ic, xi, f);
+                  }
+                }
+              } else if (p.n > 1) {
+                D.add4(p.c1, ic, xi, f);
+                if (p.n > 2) D.add4(p.c2, ic, xi, f);
+              }
+            }
+          }
+          // dE of the columns, and the largest dE their draws can accept:
+          // u < floor(2^32 exp(-dE/T)) iff dE <= T ln(2^32 / (u + 1)), here
+          // with a margin above the estimate's error (100 times it), so that a
+          // dE above the bound is rejected for certain, and one more than
+          // `band` below it accepted; between them the table decides.
+          int dE[4], top[4];
+          const uint32_t u[4] = {u4.x, u4.y, u4.z, u4.w};
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int bf = B * f[j];
+            dE[j] = ((xm >> j) & 1) ? twoA * (3 - c[j] - r) - bf : twoA * (c[j] + r - 1) + bf;
+            float lg;
+            asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(__uint2float_rn(u[j]) + 1.0f));
+            const int i = i0 + j;
+            top[j] = (unsigned)i < (unsigned)C && i != s0 ? (int)(fmaf(32.0f - lg, Tl, margin)) : INT_MIN;
+          }
+          while (true) {
+            if (!__any_sync(kFull, dE[0] <= top[0] || dE[1] <= top[1] || dE[2] <= top[2] || dE[3] <= top[3])) break;
+            // the first proposal that may be accepted
+            const int jl = dE[0] <= top[0] ? 0 : (dE[1] <= top[1] ? 1 : (dE[2] <= top[2] ? 2 : 3));
+            const int dl = sel4(dE, jl), tl = sel4(top, jl);
+            const int L = __ffs(__ballot_sync(kFull, dl <= tl)) - 1;
+            const int pk0 = jl | ((xm >> jl) & 1) << 2 | sel4(c, jl) << 3;
+            bool ok = true;
+            if (lane == L && dl >= tl - band) {
+              const uint32_t uj = jl == 0 ? u[0] : (jl == 1 ? u[1] : (jl == 2 ? u[2] : u[3]));
+              ok = dl <= 0 || (dl < len && uj < __ldg(thr + QP_IX(dl, len, 1)));
+            }
+            const int de = __shfl_sync(kFull, dl, L);
+            const int pk = __shfl_sync(kFull, ok ? pk0 : -1, L);
+            if (pk < 0) {  // rejected by the table
+              if (lane == L) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                  if (j == jl) top[j] = INT_MIN;
+              }
+              continue;
+            }
+            const int jm = pk & 3, cm = pk >> 3, dlt = 1 - 2 * ((pk >> 2) & 1);
+            const int im = (int)(4 * (mb + L)) - tC + jm;
+            E += de;
+            ++acc;
+            viol += (cm + dlt != 1) - (cm != 1);
+            if (lane == 0) {
+              cc[im] = (uint16_t)(cm + dlt);
+              uint32_t *wp = bits + QP_IX(t * Cw + (im >> 5), C * Cw, 3);
+              if (SB) *wp ^= 1u << (im & 31);
+              else atomicXor(wp, 1u << (im & 31));
+            }
+            // every proposal up to it is decided; the row's sum moved for the rest
+            const int step = dlt * twoA;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              dE[j] += ((xm >> j) & 1) ? -step : step;
+              if (i0 + j <= im) top[j] = INT_MIN;
+            }
+            if (dlt > 0) {
+              if (cm == 0) {  // no longer empty
+                if (zok) {
+                  const int p = __ffs(__ballot_sync(kFull, lane < nz && zreg == im)) - 1;
+                  const int tail = __shfl_sync(kFull, zreg, nz - 1);
+                  if (lane == p) zreg = tail;
+                }
+                --nz;
+              }
+              if (r == 0) l0 = im;
+              else if (r == 1) l1 = im;
+              else if (r == 2) l2 = im;
+              else lost = true;
+            } else {
+              if (cm == 1) {  // now empty
+                if (nz >= 32) zok = false;
+                else if (lane == nz) zreg = im;
+                ++nz;
+              }
+              if (l0 == im) {
+                l0 = l1;
+                l1 = l2;
+              } else if (l1 == im) {
+                l1 = l2;
+              }
+            }
+            r += dlt;
+            flipped = true;
+          }
+        }
+        if (flipped) {
+          ++rows_flipped;
+          viol += (r != 1) - (p1.n != 1);
+          __syncwarp();
+          uint2 q = pack_row(r, l0, l1, l2);
+          if (lost) q = record_from_bits<SB>(bits, Cw, C, t, r, lane);
+          if (lane == 0) rec[t] = q;
+          __syncwarp();
+        }
+      }
+    }
+    if (viol == 0 && E < best) best = E;
+    settled = a.skip_settled && !hit;
+    settled_len = len;
+  }
+
+  // ---- outputs: zeros in 16-byte stores, then the cells
+  uint8_t *out = a.states_out + (size_t)rep * n;
+  const int head = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(out) & 15)) & 15));
+  const int nv = (n - head) / 16;
+  if (lane < head) out[lane] = 0;
+  for (int v = lane; v < nv; v += 32) reinterpret_cast<uint4 *>(out + head)[v] = make_uint4(0, 0, 0, 0);
+  for (int e = head + 16 * nv + lane; e < n; e += 32) out[e] = 0;
+  __syncwarp();
+  for (int t = lane; t < C; t += 32) {
+    const Row q = unpack_row(rec[t]);
+    uint8_t *o = out + (size_t)t * C;
+    if (q.n <= kRowCells) {
+      if (q.n > 0) o[q.c0] = 1;
+      if (q.n > 1) o[q.c1] = 1;
+      if (q.n > 2) o[q.c2] = 1;
+    } else {
+      for (int w = 0; w < Cw; ++w) {
+        uint32_t wd = bits_word<SB>(bits + t * Cw + w);
+        while (wd) {
+          o[(w << 5) + __ffs(wd) - 1] = 1;
+          wd &= wd - 1;
+        }
+      }
+    }
+  }
+  if (lane == 0) {
+    a.E_out[rep] = E;
+    if (a.best_out) a.best_out[rep] = best;
+    if (a.acc_out) a.acc_out[rep] = acc;
+  }
+}
+
+// Shared memory of one replica.
+__host__ __device__ inline size_t events_warp_bytes(int C, bool bits_smem) {
+  const int Cw = (C + 31) >> 5;
+  return align16e(8 * ((size_t)C + 1)) + align16e(2 * ((size_t)C + 2 * kPad)) +
+         (bits_smem ? align16e(4 * (size_t)C * Cw) : 0);
+}
+
+// Shared memory of the distances: the matrix (DM = 1) or the coordinates and the table (DM = 2).
+__host__ __device__ inline size_t events_dist_bytes(int C, int Cp, size_t es, int dm, int tab_n) {
+  if (dm == 1) return align16e(((size_t)C * Cp + 2 * kPad) * es);
+  if (dm == 2) return align16e(2 * ((size_t)C + 2 * kPad)) + align16e((size_t)tab_n * es);
+  return 0;
+}
+
+template <typename DT, int DM>
+__device__ __forceinline__ Dist<DT, DM> stage_dist(const StructArgs &a, unsigned char *p, int tid, int nthreads) {
+  Dist<DT, DM> D{static_cast<const DT *>(a.d), a.Cp, a.C, nullptr, a.tab_sh, a.tab_n};
+  if (DM == 1) {
+    const int nv = (int)((size_t)a.C * a.Cp * sizeof(DT) / 16);
+    const int4 *src = static_cast<const int4 *>(a.d);
+    DT *m = reinterpret_cast<DT *>(p) + kPad;
+    for (int v = tid; v < nv; v += nthreads) reinterpret_cast<int4 *>(m)[v] = __ldg(src + v);
+    D.m = m;
+  } else if (DM == 2) {
+    uint16_t *xy = reinterpret_cast<uint16_t *>(p) + kPad;
+    DT *tab = reinterpret_cast<DT *>(p + align16e(2 * ((size_t)a.C + 2 * kPad)));
+    for (int i = tid - kPad; i < a.C + kPad; i += nthreads) xy[i] = i >= 0 && i < a.C ? __ldg(a.xy + i) : 0;
+    for (int i = tid; i < a.tab_n; i += nthreads) tab[i] = __ldg(static_cast<const DT *>(a.tab) + i);
+    D.xy = xy;
+    D.m = tab;
+  }
+  return D;
+}
+
+template <typename DT, int DM, bool SB>
+__global__ void __launch_bounds__(kMaxWarpsPerCta * 32) k_sweep_events(const StructArgs a, const RoundKeys rk) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+  const Dist<DT, DM> D = stage_dist<DT, DM>(a, smem, threadIdx.x, blockDim.x);
+  __syncthreads();
+  const int rep = blockIdx.x * W + warp;
+  if (rep >= a.R) return;  // no CTA-wide barrier after this point
+  const size_t per = events_warp_bytes(a.C, SB);
+  unsigned char *p = smem + events_dist_bytes(a.C, a.Cp, sizeof(DT), DM, a.tab_n) + warp * per;
+  uint2 *rec = reinterpret_cast<uint2 *>(p);
+  p += align16e(8 * ((size_t)a.C + 1));
+  uint16_t *cc = reinterpret_cast<uint16_t *>(p) + kPad;
+  p += align16e(2 * ((size_t)a.C + 2 * kPad));
+  uint32_t *bits = SB ? reinterpret_cast<uint32_t *>(p) : a.gstate + (size_t)rep * a.nw_pad;
+  events_replica<DT, DM, SB>(a, rep, rec, cc, bits, D, lane, rk);
+}
+
+constexpr size_t kSmemLimitEvents = 227 * 1024;
+constexpr size_t kBitsSmem = 8 * 1024;       // most bytes of a replica's bitsets kept in shared memory
+constexpr size_t kMatrixSmem = 40 * 1024;    // largest distance matrix staged in shared memory
+
+struct EventsShape {
+  int dm;
+  bool sb;
+  size_t dist, per;
+};
+
+EventsShape events_shape(const StructArgs &a, bool d_i16) {
+  const size_t es = d_i16 ? 2 : 4;
+  const int Cw = (a.C + 31) / 32;
+  EventsShape s;
+  s.sb = 4 * (size_t)a.C * Cw <= kBitsSmem;
+  s.dm = (size_t)a.C * a.Cp * es <= kMatrixSmem ? 1 : (a.tab_n > 0 ? 2 : 0);
+  s.dist = events_dist_bytes(a.C, a.Cp, es, s.dm, a.tab_n);
+  s.per = events_warp_bytes(a.C, s.sb);
+  return s;
+}
+
+template <typename DT, int DM, bool SB>
+cudaError_t launch_e(const StructArgs &a, const RoundKeys &rk, int W, size_t smem, cudaStream_t st) {
+  auto k = k_sweep_events<DT, DM, SB>;
+  std::lock_guard<std::mutex> lk(launch_mutex());
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  k<<<(a.R + W - 1) / W, W * 32, smem, st>>>(a, rk);
+  return cudaGetLastError();
+}
+
+template <typename DT>
+cudaError_t launch_e2(const StructArgs &a, const RoundKeys &rk, const EventsShape &s, int W, size_t smem,
+                      cudaStream_t st) {
+  if (s.dm == 1) return s.sb ? launch_e<DT, 1, true>(a, rk, W, smem, st) : launch_e<DT, 1, false>(a, rk, W, smem, st);
+  if (s.dm == 2) return s.sb ? launch_e<DT, 2, true>(a, rk, W, smem, st) : launch_e<DT, 2, false>(a, rk, W, smem, st);
+  return s.sb ? launch_e<DT, 0, true>(a, rk, W, smem, st) : launch_e<DT, 0, false>(a, rk, W, smem, st);
+}
+
+}  // namespace
+
+size_t events_state_words(int C) {
+  const int Cw = (C + 31) / 32;
+  const size_t words = ((size_t)C * Cw + 3) / 4 * 4;
+  return 4 * (size_t)C * Cw <= kBitsSmem ? 0 : words;
+}
+
+cudaError_t launch_events(const StructArgs &a_in, bool d_i16, int W, cudaStream_t st, LaunchInfo *info) {
+  StructArgs a = a_in;
+  a.nw_pad = (int32_t)events_state_words(a.C);
+  const EventsShape s = events_shape(a, d_i16);
+  if (!s.sb && a.gstate == nullptr) return cudaErrorInvalidValue;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  // one chain per scheduler first: a chain's latency is its time, so few
+  // chains spread over the SMs, many share the staged distances
+  if (W <= 0) W = std::max(1, std::min(8, (a.R + sms - 1) / sms));
+  while (W > 1 && s.dist + W * s.per > kSmemLimitEvents) --W;
+  const size_t smem = s.dist + W * s.per;
+  if (smem > kSmemLimitEvents) return cudaErrorInvalidValue;
+  if (info) {
+    info->warps_per_cta = W;
+    info->blocks = (a.R + W - 1) / W;
+    info->smem = smem;
+    info->variant = s.dm == 1 ? "events,d:smem" : (s.dm == 2 ? "events,d:table" : "events,d:global");
+  }
+  RoundKeys rk;
+  for (int i = 0; i < 10; ++i) {
+    rk.k[2 * i] = a.key0 + (uint32_t)i * 0x9E3779B9u;
+    rk.k[2 * i + 1] = a.key1 + (uint32_t)i * 0xBB67AE85u;
+  }
+  return d_i16 ? launch_e2<int16_t>(a, rk, s, W, smem, st) : launch_e2<int32_t>(a, rk, s, W, smem, st);
+}
+
+}  // namespace qp
+
+namespace qp {
+namespace chk {
+QP_CHECK_ACCESSOR(events)
+}  // namespace chk
+}  // namespace qp
