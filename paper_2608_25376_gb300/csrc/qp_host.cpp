@@ -345,12 +345,15 @@ static qp_status build_field_qubo(const qp_field *f, int32_t A, int32_t B, int32
   QP_CU(cudaMemcpy(h->d32_dev.p, h->d.data(), (size_t)C * C * 4, cudaMemcpyHostToDevice));
   {
     const size_t es = h->d_i16 ? 2 : 4;
-    // after the matrix: the cells' grid coordinates and d by grid difference
+    // The matrix with 16 bytes before it and a row of zeros after it (the
+    // event-driven sweep reads four columns at a time around a row's ends, and
+    // an empty row's distances), the cells' grid coordinates, and d by grid
+    // difference.
     const int r0 = *std::min_element(cr.begin(), cr.end()), c0 = *std::min_element(cc.begin(), cc.end());
     const int rows = *std::max_element(cr.begin(), cr.end()) - r0 + 1, cols = *std::max_element(cc.begin(), cc.end()) - c0 + 1;
     while ((1 << h->tab_sh) < cols) ++h->tab_sh;
     if (rows <= 256 && cols <= 256 && (size_t)(rows << h->tab_sh) * es <= 32 * 1024) h->tab_n = rows << h->tab_sh;
-    h->xy_at = (size_t)C * h->Cp * es;
+    h->xy_at = 16 + ((size_t)C + 1) * h->Cp * es;
     h->tab_at = h->xy_at + (size_t)h->Cp * 2;
     std::vector<uint8_t> pad(h->tab_at + (size_t)h->tab_n * es, 0);
     if (h->tab_n) {
@@ -371,8 +374,8 @@ static qp_status build_field_qubo(const qp_field *f, int32_t A, int32_t B, int32
     for (int i = 0; i < C; ++i)
       for (int j = 0; j < C; ++j) {
         const int32_t v = h->d[(size_t)i * C + j];
-        if (h->d_i16) reinterpret_cast<int16_t *>(pad.data())[(size_t)i * h->Cp + j] = (int16_t)v;
-        else reinterpret_cast<int32_t *>(pad.data())[(size_t)i * h->Cp + j] = v;
+        if (h->d_i16) reinterpret_cast<int16_t *>(pad.data() + 16)[(size_t)i * h->Cp + j] = (int16_t)v;
+        else reinterpret_cast<int32_t *>(pad.data() + 16)[(size_t)i * h->Cp + j] = v;
       }
     QP_TRY(h->d_dev.ensure(pad.size()));
     QP_CU(cudaMemcpy(h->d_dev.p, pad.data(), pad.size(), cudaMemcpyHostToDevice));
@@ -536,7 +539,7 @@ namespace host {
 
 void fill_field_args(const qp_handle *h, StructArgs &a) {
   a.C = h->C; a.Cp = h->Cp; a.start = h->start; a.A = h->A; a.B = h->B;
-  a.d = h->d_dev.p;
+  a.d = h->d_matrix();
   a.xy = reinterpret_cast<const uint16_t *>(h->d_dev.as<uint8_t>() + h->xy_at);
   a.tab = h->d_dev.as<uint8_t>() + h->tab_at;
   a.tab_sh = h->tab_sh; a.tab_n = h->tab_n;
@@ -810,7 +813,7 @@ bool handle_struct_view(const qp_handle *h, StructView *out) {
   out->start = h->start;
   out->A = h->A;
   out->B = h->B;
-  out->d = h->d_dev.p;
+  out->d = h->d_matrix();
   out->d_i16 = h->d_i16;
   out->max_d = h->max_d;
   out->d32 = h->d32_dev.as<int32_t>();

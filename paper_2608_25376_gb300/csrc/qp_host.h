@@ -120,10 +120,12 @@ struct qp_handle {
   int64_t n = 0, c0 = 0;
   std::vector<int32_t> d;  // C x C (host)
   // device data
-  qp::host::DevBuf d_dev;            // C x Cp, int16 or int32; then the cells' coordinates and the distance table
+  qp::host::DevBuf d_dev;            // 16 bytes, C x Cp (int16 or int32), a row of zeros, the cells'
+                                     // coordinates, the distance table
   bool d_i16 = false;
   int32_t Cp = 0;
-  size_t xy_at = 0, tab_at = 0;      // byte offsets of both in d_dev
+  const void *d_matrix() const { return d_dev.as<uint8_t>() + 16; }
+  size_t xy_at = 0, tab_at = 0;      // byte offsets of the last two
   int32_t tab_sh = 0, tab_n = 0;     // tab_n = 0: the grid is too large for a table
   qp::host::DevBuf d32_dev;          // C x C int32 (decode, dense build)
   qp::host::DevBuf S_dev;            // n x np, int16 or int32

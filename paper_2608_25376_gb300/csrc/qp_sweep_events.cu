@@ -32,16 +32,18 @@
 // against the same tables.
 //
 // What bounds it: the latency of one chain (a check is ~150 dependent cycles,
-// an event ~1500), and in hot sweeps of large fields the Philox multiplies.
+// an event ~1500), and in hot sweeps of large fields the Philox multiplies
+// (88 cycles of a scheduler per warp-wide block, whatever the occupancy).
 // Against the row kernels, which evaluate every column of every row (one GB300;
-// microseconds per sweep of all chains): 92 cells, 1024 chains: 161 -> 97 at
-// T = 1000 (1.2 flips a row), 72 -> 20 at T = 436, 20.9 -> 1.8 below T = 115;
-// 491 cells, 4096 chains x 1000 sweeps: 899 -> 109 ms; 893 cells, 512 chains x
+// microseconds per sweep of all chains): 92 cells, 1024 chains: 161 -> 84 at
+// T = 1000 (1.2 flips a row), 72 -> 20 at T = 436, 20.9 -> 0.5 below T = 115;
+// 491 cells, 4096 chains x 1000 sweeps: 899 -> 101 ms; 893 cells, 512 chains x
 // 40 sweeps (the general kernel): 272 -> 25.9 ms.  It is also the faster one far
 // above the temperatures of a useful schedule (T = 1e6, a third of the cells
 // set: 1.5 to 2.2 times), so every structured launch uses it.
 #include <algorithm>
 #include <climits>
+#include <type_traits>
 
 #include "qp_device.cuh"
 #include "qp_internal.h"
@@ -62,8 +64,9 @@ constexpr int kPad = 8;       // entries before and after the arrays read by fou
 __host__ __device__ constexpr size_t align16e(size_t x) { return (x + 15) & ~size_t(15); }
 
 // A row's record: its number of cells and, when there are at most three, the
-// cells themselves; of a row with more, one of its cells (c0).  The bits hold
-// every row.
+// cells themselves (c0 = C in an empty row); of a row with more, one of its
+// cells (c0), and the row's bits hold them all.  The bits of other rows are
+// not kept.
 struct Row {
   int n, c0, c1, c2;
 };
@@ -75,7 +78,7 @@ __device__ __forceinline__ uint2 pack_row(int n, int c0, int c1, int c2) {
 }
 
 // d_{h,i}: from the matrix in global memory (DM = 0) or in shared memory
-// (DM = 1), or from the field's table over (|row difference|, |column
+// (DM = 1), with a row of zeros after it and readable entries around it, or from the field's table over (|row difference|, |column
 // difference|) in shared memory (DM = 2: 24x24 cells take 1.5 KB instead of
 // the matrix's 482 KB).
 template <typename DT, int DM>
@@ -88,25 +91,32 @@ struct Dist {
     const uint32_t ad = __vabsdiffu4(a, b);
     return (int)m[QP_IX((int)(((ad >> 8) << sh) + (ad & 0xFFu)), tab_n, 2)];
   }
+  // A cell as hx keeps it (its coordinates when they are all a distance needs,
+  // which spares the gather of them), and the distance of two of those.
+  __device__ __forceinline__ uint32_t code(int h) const { return DM == 2 ? (uint32_t)xy[QP_IX(h, C, 2)] : (uint32_t)h; }
+  __device__ __forceinline__ int near(uint32_t a, uint32_t b) const {
+    if (DM == 2) return lookup(a, b);
+    const int k = QP_IX((int)a * Cp + (int)b, (C + 1) * Cp, 2);
+    return DM == 1 ? (int)m[k] : (int)__ldg(m + k);
+  }
+  // h = C (an empty row's record): 0
   __device__ __forceinline__ int operator()(int h, int i) const {
-    if (DM == 2) return lookup(xy[QP_IX(h, C, 2)], xy[QP_IX(i, C, 2)]);
-    const int k = QP_IX(h * Cp + i, C * Cp, 2);
+    if (DM == 2) return h < C ? lookup(xy[QP_IX(h, C, 2)], xy[QP_IX(i, C, 2)]) : 0;
+    const int k = QP_IX(h * Cp + i, (C + 1) * Cp, 2);
     return DM == 1 ? (int)m[k] : (int)__ldg(m + k);
   }
   // f[j] += d_{h,i+j}, -4 < i <= C; columns outside the field give anything.
   // xi: the columns' coordinates (DM = 2).
   __device__ __forceinline__ void add4(int h, int i, const uint32_t (&xi)[4], int (&f)[4]) const {
     if (DM == 2) {
+      if (h >= C) return;
       const uint32_t a = xy[QP_IX(h, C, 2)];
 #pragma unroll
       for (int j = 0; j < 4; ++j) f[j] += lookup(a, xi[j]);
-    } else if (DM == 1) {
-      const DT *p = m + QP_IX(h, C, 2) * Cp + i;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) f[j] += (int)p[j];
     } else {
+      const DT *p = m + QP_IX(h, C + 1, 2) * Cp + i;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) f[j] += (int)__ldg(m + min(max(h * Cp + i + j, 0), C * Cp - 1));
+      for (int j = 0; j < 4; ++j) f[j] += DM == 1 ? (int)p[j] : (int)__ldg(p + j);
     }
   }
 };
@@ -144,7 +154,7 @@ __device__ __forceinline__ int row_sum_d(const Row &q, int u, const uint32_t *bi
 // of its cells.
 template <bool SB>
 __device__ __forceinline__ uint2 record_from_bits(const uint32_t *bits, int Cw, int C, int t, int r, int lane) {
-  int c[3] = {0, 0, 0}, k = 0;
+  int c[3] = {C, 0, 0}, k = 0;
   const int want = r <= kRowCells ? r : 1;
   for (int w0 = 0; w0 < Cw && k < want; w0 += 32) {
     const uint32_t word = w0 + lane < Cw ? bits_word<SB>(bits + QP_IX(t * Cw + w0 + lane, C * Cw, 3)) : 0u;
@@ -163,10 +173,11 @@ __device__ __forceinline__ uint2 record_from_bits(const uint32_t *bits, int Cw, 
 }
 
 // The sweeps of one replica.  rec: C + 1 row records (the last stays empty),
-// cc: column sums with kPad entries on both sides, bits: C x Cw words.
+// hx: what D.near needs of the cell of a row that holds one, cc:
+// column sums with kPad entries on both sides, bits: C x Cw words.
 template <typename DT, int DM, bool SB, typename KEY>
-__device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uint2 *rec, uint16_t *cc, uint32_t *bits,
-                                               const Dist<DT, DM> &D, int lane, const KEY &key) {
+__device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uint2 *rec, uint16_t *hx, uint16_t *cc,
+                                               uint32_t *bits, const Dist<DT, DM> &D, int lane, const KEY &key) {
   const int C = a.C, s0 = a.start, B = a.B, twoA = 2 * a.A;
   const int Cw = (C + 31) >> 5;
   const int n = C * C;
@@ -175,11 +186,11 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
 
   // ---- initial state: given or all zero; row 0 and column s clamped (x_{0,s} = 1)
   for (int i = lane; i < C + 2 * kPad; i += 32) cc[i - kPad] = 0;
-  for (int e = lane; e < C * Cw; e += 32) bits[e] = 0;
-  for (int t = lane; t <= C; t += 32) rec[t] = make_uint2(0, 0);
+  if (a.init)
+    for (int e = lane; e < C * Cw; e += 32) bits[e] = 0;
+  for (int t = lane; t <= C; t += 32) rec[t] = a.init ? make_uint2(0, 0) : pack_row(0, C, 0, 0);
   __syncwarp();
   if (lane == 0) {
-    bits[s0 >> 5] = 1u << (s0 & 31);
     rec[0] = pack_row(1, s0, 0, 0);
     cc[s0] = 1;
   }
@@ -218,6 +229,9 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
     for (int k = head + 16 * nv + lane; k < n; k += 32)
       if (x[k]) set(k);
     __syncwarp();
+    for (int t = lane; t <= C; t += 32)
+      if ((rec[t].x & 0xFFFFu) == 0) rec[t] = pack_row(0, C, 0, 0);
+    __syncwarp();
   }
   // ---- energy (Eqs. 3-6), violation count, empty columns
   long long E;
@@ -252,297 +266,341 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
       v += c != 1;
       z += c == 0;
     }
+    for (int t = lane; t < C; t += 32) {
+      const int h = (int)(rec[t].x >> 16);
+      hx[t] = (uint16_t)D.code(min(h, C - 1));
+    }
+    __syncwarp();
     E = (long long)B * warp_sum64(hd) + (long long)a.A * warp_sum64(pen);
     viol = __reduce_add_sync(kFull, v);
     nz = __reduce_add_sync(kFull, z);
   }
   long long best = LLONG_MAX, acc = 0;
   int zreg = 0;          // lane q < nz: an empty column (when zok)
-  bool zok = nz == 0;
+  bool zok = false;
   int rows_flipped = 2 * viol;  // rows the last sweep changed; at first, a guess from the state
-
-  // ---- sweeps.  The table's place, length and log2(e)/T of a sweep are
-  // loaded two sweeps ahead, thr[2A] one ahead, so no sweep waits for them.
-  const int lev = a.level ? __ldg(a.level + rep) : -1;
-  const int last = a.sweep_end - 1;
-  auto row_of = [&](int s) { return lev >= 0 ? lev : min(s, last); };
-  long long off1 = 0, off2 = 0;
-  int len1 = 0, len2 = 0;
-  float c1 = 0.0f, c2 = 0.0f;
-  uint32_t q1 = 0;
-  if (a.sweep_begin < a.sweep_end) {
-    const int u1 = row_of(a.sweep_begin), u2 = row_of(a.sweep_begin + 1);
-    off1 = a.thr_off[u1]; len1 = a.thr_len[u1]; c1 = a.thr_c[u1];
-    off2 = a.thr_off[u2]; len2 = a.thr_len[u2]; c2 = a.thr_c[u2];
-    if (len1 > twoA) q1 = __ldg(a.thr + off1 + twoA);
+  // the lane's valid columns (in the field, not s) of a row's first chunk, by t C mod 4: bit 4 (tC mod 4) + j
+  uint32_t vfirst = 0;
+#pragma unroll
+  for (int e = 0; e < 16; ++e) {
+    const int i = 4 * lane - (e >> 2) + (e & 3);
+    vfirst |= (uint32_t)(i >= 0 && i < C && i != s0) << e;
   }
+
+  // ---- sweeps.  Lane l holds the table's place and length, T ln 2 and thr[2A]
+  // of sweep s0 + l, loaded 32 sweeps at a time (a cold sweep is shorter than
+  // one load).
+  const int lev = a.level ? __ldg(a.level + rep) : -1;
+  long long off_l = 0;
+  int len_l = 0;
+  float cT_l = 0.0f, Tl_l = 0.0f;
+  uint32_t q2_l = 0;  // thr[2A], 0 when the table ends before it
   bool settled = false;
   int settled_len = 0;
   for (int s = a.sweep_begin; s < a.sweep_end; ++s) {
-    const uint32_t *thr = a.thr + off1;
-    const int len = len1;
-    const float cT = c1;
-    const uint32_t Q2 = q1;  // 0 when len <= 2A
-    off1 = off2; len1 = len2; c1 = c2;
-    q1 = len1 > twoA ? __ldg(a.thr + off1 + twoA) : 0u;
-    {
-      const int u2 = row_of(s + 2);
-      off2 = a.thr_off[u2]; len2 = a.thr_len[u2]; c2 = a.thr_c[u2];
+    const int sl = (s - a.sweep_begin) & 31;
+    if (sl == 0) {
+      const int ts = lev >= 0 ? lev : min(s + lane, a.sweep_end - 1);
+      off_l = __ldg(reinterpret_cast<const long long *>(a.thr_off) + ts);
+      len_l = __ldg(a.thr_len + ts);
+      cT_l = __ldg(a.thr_c + ts);
+      Tl_l = 1.0f / cT_l;
+      q2_l = len_l > twoA ? __ldg(a.thr + off_l + twoA) : 0u;
     }
+    const uint32_t *thr = a.thr + __shfl_sync(kFull, off_l, sl);
+    const int len = __shfl_sync(kFull, len_l, sl);
+    const float cT = __shfl_sync(kFull, cT_l, sl), Tl = __shfl_sync(kFull, Tl_l, sl);
+    const uint32_t Q2 = __shfl_sync(kFull, q2_l, sl);
     if (settled && len <= settled_len) continue;
     const bool hot = Q2 != 0;
-    const float Tl = 1.0f / cT;                // T ln 2
     const float margin = Tl * (1.0f / 512.0f);  // of the estimate below
+    const float top0 = fmaf(32.0f, Tl, margin);
     const int band = (int)(2.0f * margin) + 2;
-    // row by row when half the rows are events anyway: rows changed in the last sweep, rows with survivors
-    const float lambda = (float)Q2 * 2.3283064365386963e-10f * (float)C;
-    const bool rowwise = (float)rows_flipped + 0.5f * lambda * (float)C > 0.5f * (float)C;
-    rows_flipped = 0;
     bool hit = hot;  // a proposal with dE < len was met
-    for (int t0 = 1; t0 < C; t0 += 32) {
-      const int t1 = min(C, t0 + 32);
-      // -- draws of the window: the rows with survivors
-      uint32_t smask = 0;
-      if (hot && !rowwise) {
-        const uint32_t k0 = (uint32_t)(t0 * C), nk = (uint32_t)((t1 - t0) * C);
-        const uint32_t mend = (k0 + nk - 1) >> 2;
-        auto mark = [&](const uint4 &u, uint32_t m) {
-          const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+
+    // The draws of the lane's four columns of row t, block m (first: in the
+    // row's first 128 columns), and the largest
+    // dE each can accept: u < floor(2^32 exp(-dE/T)) iff dE <= T ln(2^32 /
+    // (u + 1)), here with a margin above the estimate's error (100 times it), so
+    // that a dE above the bound is rejected for certain, and one more than
+    // `band` below it accepted; between them the table decides.
+    auto draws = [&](int tC, uint32_t m, uint32_t (&u)[4], int (&top)[4], auto first) {
+      const uint4 u4 = philox4x32_10(make_uint4(m, (uint32_t)s, rg, kRngTag), key);
+      u[0] = u4.x; u[1] = u4.y; u[2] = u4.z; u[3] = u4.w;
+      uint32_t v = vfirst >> (4 * (tC & 3));
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const uint32_t rel = 4 * m + j - k0;
-            if (w[j] < Q2 && rel < nk) smask |= 1u << __umulhi(rel, magic);
-          }
-        };
-        for (uint32_t mb = k0 >> 2; mb <= mend; mb += 64) {
-          const uint32_t ma = mb + lane, mc = ma + 32;
-          const uint4 ua = philox4x32_10(make_uint4(ma, (uint32_t)s, rg, kRngTag), key);
-          const uint4 ub = philox4x32_10(make_uint4(mc, (uint32_t)s, rg, kRngTag), key);
-          const uint32_t la = min(min(ua.x, ua.y), min(ua.z, ua.w)), lb = min(min(ub.x, ub.y), min(ub.z, ub.w));
-          if (min(la, lb) < Q2) {
-            mark(ua, ma);
-            mark(ub, mc);
-          }
-        }
-        smask = __reduce_or_sync(kFull, smask);
+      for (int j = 0; j < 4; ++j) {
+        float lg;
+        asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(__uint2float_rn(u[j]) + 1.0f));
+        const int i = (int)(4 * m) - tC + j;
+        const bool valid = decltype(first)::value ? (v >> j) & 1u : (unsigned)i < (unsigned)C && i != s0;
+        top[j] = valid ? (int)fmaf(-lg, Tl, top0) : INT_MIN;
       }
-      // -- the window's rows
-      bool have_uh = false;
-      uint32_t uh = 0;  // the draw of the cell of row t0 + lane
-      for (int t = t0; t < t1; ++t) {
-        if (!rowwise && nz <= kZCheck) {
-          if (!zok) {  // list the empty columns
-            int k = 0;
-            for (int i0 = 0; i0 < C; i0 += 32) {
-              uint32_t b = __ballot_sync(kFull, i0 + lane < C && cc[i0 + lane] == 0);
-              while (b) {
-                if (lane == k) zreg = i0 + __ffs(b) - 1;
-                b &= b - 1;
-                ++k;
-              }
-            }
-            zok = true;
-          }
-          // the check: lane = row
-          const int tl = t0 + lane;
-          const bool in = tl >= t && tl < t1;
-          const int tr = min(tl, C - 1);
-          const Row p0 = unpack_row(rec[tr - 1]), p1 = unpack_row(rec[tr]), p2 = unpack_row(rec[tr + 1]);
-          bool ev = p1.n != 1 || p0.n > 1 || p2.n > 1 || ((smask >> lane) & 1u);
-          const int h = p1.c0;
-          int dE = len;
-          if (in && !ev) {
-            int f = 0;
-            if (p0.n) f = D(p0.c0, h);
-            if (p2.n) f += D(p2.c0, h);
-            dE = twoA * (2 - (int)cc[h]) - B * f;
-          }
-          bool need = dE < len;
-          if (__any_sync(kFull, need)) {
-            hit = true;
-            if (!have_uh) {
-              const uint32_t k = (uint32_t)(tr * C + h);
-              const uint4 u = philox4x32_10(make_uint4(k >> 2, (uint32_t)s, rg, kRngTag), key);
-              uh = word_of(u, k & 3);
-              have_uh = true;
-            }
-            if (need) ev = dE <= 0 || accept_draw(uh, dE, cT, thr, len);
-          }
-          for (int q = 0; q < nz; ++q) {
-            const int z = __shfl_sync(kFull, zreg, q);
-            dE = len;
-            if (in && !ev) {
-              int f = 0;
-              if (p0.n) f = D(p0.c0, z);
-              if (p2.n) f += D(p2.c0, z);
-              dE = B * f;
-            }
-            need = dE < len;
-            if (__any_sync(kFull, need)) {
-              hit = true;
-              const uint32_t k = (uint32_t)(tr * C + z);
-              const uint4 u = philox4x32_10(make_uint4(k >> 2, (uint32_t)s, rg, kRngTag), key);
-              if (need) ev = dE <= 0 || accept_draw(word_of(u, k & 3), dE, cT, thr, len);
-            }
-          }
-          const uint32_t bal = __ballot_sync(kFull, in && ev);
-          if (bal == 0) break;  // nothing happens in the rest of the window
-          t = t0 + __ffs(bal) - 1;
+    };
+
+    // Row t, exactly.  pre (PRE, rows of one block): the next row's draws are
+    // computed beside this row's evaluation, of which they are independent (u
+    // and top hold this row's on entry, the next one's on return).
+    uint32_t u[4];
+    int top[4];
+    auto event_row = [&](int t, auto pre) {
+      constexpr bool PRE = decltype(pre)::value;
+      const Row p0 = unpack_row(rec[t - 1]), p1 = unpack_row(rec[t]), p2 = unpack_row(rec[t + 1]);
+      const int tC = t * C;
+      int r = p1.n, l0 = p1.c0, l1 = p1.c1, l2 = p1.c2;
+      bool lost = p1.n > kRowCells, flipped = false;
+      const uint32_t m1 = (uint32_t)(tC + C - 1) >> 2;
+            for (uint32_t mb = (uint32_t)tC >> 2; mb <= m1; mb += 32) {
+        uint32_t un[4];
+        int topn[4];
+        if (PRE) draws(tC + C, ((uint32_t)(tC + C) >> 2) + lane, un, topn, pre);
+        else draws(tC, mb + lane, u, top, pre);
+        const int i0 = (int)(4 * (mb + lane)) - tC;  // the lane's columns i0 .. i0 + 3, -4 < i0
+        const int ic = min(i0, C);
+        int f[4] = {0, 0, 0, 0}, c[4];
+        uint32_t xi[4] = {0, 0, 0, 0};
+        if (DM == 2) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) xi[j] = D.xy[ic + j];
         }
-        // -- event row t
-        hit = true;
-        const Row p0 = unpack_row(rec[t - 1]), p1 = unpack_row(rec[t]), p2 = unpack_row(rec[t + 1]);
-        const int tC = t * C;
-        int r = p1.n, l0 = p1.c0, l1 = p1.c1, l2 = p1.c2;
-        bool lost = p1.n > kRowCells, flipped = false;
-        const bool many = p0.n > 1 || p1.n > 1 || p2.n > 1;
-        const int h1 = p1.n > 0 ? p1.c0 : -8;
-        const uint32_t m1 = (uint32_t)(tC + C - 1) >> 2;
-        for (uint32_t mb = (uint32_t)tC >> 2; mb <= m1; mb += 32) {
-          const uint32_t m = mb + lane;
-          const uint4 u4 = philox4x32_10(make_uint4(m, (uint32_t)s, rg, kRngTag), key);
-          const int i0 = (int)(4 * m) - tC;  // the lane's columns i0 .. i0 + 3, -4 < i0
-          const int ic = min(i0, C);
-          int f[4] = {0, 0, 0, 0}, c[4];
-          uint32_t xi[4] = {0, 0, 0, 0};
-          if (DM == 2) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) xi[j] = D.xy[ic + j];
+        for (int j = 0; j < 4; ++j) c[j] = cc[ic + j];
+        D.add4(p0.c0, ic, xi, f);
+        D.add4(p2.c0, ic, xi, f);
+        int xm = 0;  // x of the lane's columns
+#pragma unroll
+        for (int j = 0; j < 4; ++j) xm |= (int)(i0 + j == p1.c0) << j;
+        if (p0.n > 1 || p1.n > 1 || p2.n > 1) {  // rows of several cells
+          if (p1.n > kRowCells) {
+            xm = 0;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int i = i0 + j;
+              if (i >= 0 && i < C)
+                xm |= (int)((bits_word<SB>(bits + QP_IX(t * Cw + (i >> 5), C * Cw, 3)) >> (i & 31)) & 1u) << j;
+            }
+          } else if (p1.n > 1) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              xm |= (int)(i0 + j == p1.c1 || (p1.n > 2 && i0 + j == p1.c2)) << j;
           }
-#pragma unroll
-          for (int j = 0; j < 4; ++j) c[j] = cc[ic + j];
-          if (p0.n > 0) D.add4(p0.c0, ic, xi, f);
-          if (p2.n > 0) D.add4(p2.c0, ic, xi, f);
-          int xm = 0;  // x of the lane's columns
-#pragma unroll
-          for (int j = 0; j < 4; ++j) xm |= (int)(i0 + j == h1) << j;
-          if (many) {  // rows of several cells
-            if (p1.n > kRowCells) {
-              xm = 0;
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const int i = i0 + j;
-                if (i >= 0 && i < C)
-                  xm |= (int)((bits_word<SB>(bits + QP_IX(t * Cw + (i >> 5), C * Cw, 3)) >> (i & 31)) & 1u) << j;
+#pragma unroll 1
+          for (int side = -1; side <= 1; side += 2) {
+            const Row &p = side < 0 ? p0 : p2;
+            if (p.n > kRowCells) {  // the cells from the row's bits, but the one already added
+              for (int w0 = 0; w0 < Cw; w0 += 32) {
+                uint32_t word = w0 + lane < Cw ? bits_word<SB>(bits + QP_IX((t + side) * Cw + w0 + lane, C * Cw, 3)) : 0u;
+                if ((p.c0 >> 5) == w0 + lane) word &= ~(1u << (p.c0 & 31));
+                for (uint32_t b = __ballot_sync(kFull, word != 0); b; b &= b - 1) {
+                  const int w = __ffs(b) - 1;
+                  for (uint32_t wd = __shfl_sync(kFull, word, w); wd; wd &= wd - 1)
+                    D.add4(((w0 + w) << 5) + __ffs(wd) - 1, ic, xi, f);
+                }
               }
-            } else if (p1.n > 1) {
+            } else if (p.n > 1) {
+              D.add4(p.c1, ic, xi, f);
+              if (p.n > 2) D.add4(p.c2, ic, xi, f);
+            }
+          }
+        }
+        // dE of x = 0, and 4A less it for x = 1
+        int dE[4], step[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const int v = twoA * (c[j] + r - 1) + B * f[j];
+          const bool x = (xm >> j) & 1;
+          dE[j] = x ? 2 * twoA - v : v;
+          step[j] = x ? -twoA : twoA;
+        }
+        while (true) {
+          if (!__any_sync(kFull, dE[0] <= top[0] || dE[1] <= top[1] || dE[2] <= top[2] || dE[3] <= top[3])) break;
+          // the first proposal that may be accepted
+          const int jl = dE[0] <= top[0] ? 0 : (dE[1] <= top[1] ? 1 : (dE[2] <= top[2] ? 2 : 3));
+          const int dl = sel4(dE, jl), tl = sel4(top, jl);
+          const int L = __ffs(__ballot_sync(kFull, dl <= tl)) - 1;
+          int pk0 = jl | (sel4(step, jl) < 0) << 2 | sel4(c, jl) << 3;
+          if (lane == L && dl >= tl - band) {
+            const uint32_t uj = jl == 0 ? u[0] : (jl == 1 ? u[1] : (jl == 2 ? u[2] : u[3]));
+            if (!(dl <= 0 || (dl < len && uj < __ldg(thr + QP_IX(dl, len, 1))))) pk0 = -1;
+          }
+          const int de = __shfl_sync(kFull, dl, L);
+          const int pk = __shfl_sync(kFull, pk0, L);
+          if (pk < 0) {  // rejected by the table
+            if (lane == L) {
 #pragma unroll
               for (int j = 0; j < 4; ++j)
-                xm |= (int)(i0 + j == p1.c1 || (p1.n > 2 && i0 + j == p1.c2)) << j;
+                if (j == jl) top[j] = INT_MIN;
             }
-#pragma unroll 1
-            for (int side = -1; side <= 1; side += 2) {
-              const Row &p = side < 0 ? p0 : p2;
-              if (p.n > kRowCells) {  // the cells from the row's bits, but the one already added
-                for (int w0 = 0; w0 < Cw; w0 += 32) {
-                  uint32_t word = w0 + lane < Cw ? bits_word<SB>(bits + QP_IX((t + side) * Cw + w0 + lane, C * Cw, 3)) : 0u;
-                  if ((p.c0 >> 5) == w0 + lane) word &= ~(1u << (p.c0 & 31));
-                  for (uint32_t b = __ballot_sync(kFull, word != 0); b; b &= b - 1) {
-                    const int w = __ffs(b) - 1;
-                    for (uint32_t wd = __shfl_sync(kFull, word, w); wd; wd &= wd - 1)
-                      D.add4(((w0 + w) << 5) + __ffs(wd) - 1, ic, xi, f);
-                  }
-                }
-              } else if (p.n > 1) {
-                D.add4(p.c1, ic, xi, f);
-                if (p.n > 2) D.add4(p.c2, ic, xi, f);
-              }
-            }
+            continue;
           }
-          // dE of the columns, and the largest dE their draws can accept:
-          // u < floor(2^32 exp(-dE/T)) iff dE <= T ln(2^32 / (u + 1)), here
-          // with a margin above the estimate's error (100 times it), so that a
-          // dE above the bound is rejected for certain, and one more than
-          // `band` below it accepted; between them the table decides.
-          int dE[4], top[4];
-          const uint32_t u[4] = {u4.x, u4.y, u4.z, u4.w};
+          const int cm = pk >> 3, dlt = 1 - 2 * ((pk >> 2) & 1);
+          const int im = (int)(4 * (mb + L)) - tC + (pk & 3);
+          E += de;
+          ++acc;
+          viol += (cm + dlt != 1) - (cm != 1);
+          nz += (cm + dlt == 0) - (cm == 0);
+          if (lane == 0) cc[im] = (uint16_t)(cm + dlt);
+          // every proposal up to it is decided; the row's sum moved for the rest
 #pragma unroll
           for (int j = 0; j < 4; ++j) {
-            const int bf = B * f[j];
-            dE[j] = ((xm >> j) & 1) ? twoA * (3 - c[j] - r) - bf : twoA * (c[j] + r - 1) + bf;
-            float lg;
-            asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(lg) : "f"(__uint2float_rn(u[j]) + 1.0f));
-            const int i = i0 + j;
-            top[j] = (unsigned)i < (unsigned)C && i != s0 ? (int)(fmaf(32.0f - lg, Tl, margin)) : INT_MIN;
+            dE[j] += dlt * step[j];
+            if (i0 + j <= im) top[j] = INT_MIN;
           }
-          while (true) {
-            if (!__any_sync(kFull, dE[0] <= top[0] || dE[1] <= top[1] || dE[2] <= top[2] || dE[3] <= top[3])) break;
-            // the first proposal that may be accepted
-            const int jl = dE[0] <= top[0] ? 0 : (dE[1] <= top[1] ? 1 : (dE[2] <= top[2] ? 2 : 3));
-            const int dl = sel4(dE, jl), tl = sel4(top, jl);
-            const int L = __ffs(__ballot_sync(kFull, dl <= tl)) - 1;
-            const int pk0 = jl | ((xm >> jl) & 1) << 2 | sel4(c, jl) << 3;
-            bool ok = true;
-            if (lane == L && dl >= tl - band) {
-              const uint32_t uj = jl == 0 ? u[0] : (jl == 1 ? u[1] : (jl == 2 ? u[2] : u[3]));
-              ok = dl <= 0 || (dl < len && uj < __ldg(thr + QP_IX(dl, len, 1)));
+          if (lost || (dlt > 0 && r >= kRowCells)) {  // a row of more than three cells: its bits
+            if (!lost) {
+              for (int w = lane; w < Cw; w += 32)
+                bits[QP_IX(t * Cw + w, C * Cw, 3)] = ((l0 >> 5) == w ? 1u << (l0 & 31) : 0u) |
+                                                     ((l1 >> 5) == w ? 1u << (l1 & 31) : 0u) |
+                                                     ((l2 >> 5) == w ? 1u << (l2 & 31) : 0u);
+              lost = true;
+              __syncwarp();
             }
-            const int de = __shfl_sync(kFull, dl, L);
-            const int pk = __shfl_sync(kFull, ok ? pk0 : -1, L);
-            if (pk < 0) {  // rejected by the table
-              if (lane == L) {
-#pragma unroll
-                for (int j = 0; j < 4; ++j)
-                  if (j == jl) top[j] = INT_MIN;
-              }
-              continue;
-            }
-            const int jm = pk & 3, cm = pk >> 3, dlt = 1 - 2 * ((pk >> 2) & 1);
-            const int im = (int)(4 * (mb + L)) - tC + jm;
-            E += de;
-            ++acc;
-            viol += (cm + dlt != 1) - (cm != 1);
             if (lane == 0) {
-              cc[im] = (uint16_t)(cm + dlt);
               uint32_t *wp = bits + QP_IX(t * Cw + (im >> 5), C * Cw, 3);
               if (SB) *wp ^= 1u << (im & 31);
               else atomicXor(wp, 1u << (im & 31));
             }
-            // every proposal up to it is decided; the row's sum moved for the rest
-            const int step = dlt * twoA;
+          } else if (dlt > 0) {
+            l2 = l1;
+            l1 = l0;
+            l0 = im;
+          } else {
+            const bool first = l0 == im, second = l1 == im;
+            l0 = first ? l1 : l0;
+            l1 = first || second ? l2 : l1;
+          }
+          r += dlt;
+          flipped = true;
+        }
+        if (PRE) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              dE[j] += ((xm >> j) & 1) ? -step : step;
-              if (i0 + j <= im) top[j] = INT_MIN;
-            }
-            if (dlt > 0) {
-              if (cm == 0) {  // no longer empty
-                if (zok) {
-                  const int p = __ffs(__ballot_sync(kFull, lane < nz && zreg == im)) - 1;
-                  const int tail = __shfl_sync(kFull, zreg, nz - 1);
-                  if (lane == p) zreg = tail;
-                }
-                --nz;
-              }
-              if (r == 0) l0 = im;
-              else if (r == 1) l1 = im;
-              else if (r == 2) l2 = im;
-              else lost = true;
-            } else {
-              if (cm == 1) {  // now empty
-                if (nz >= 32) zok = false;
-                else if (lane == nz) zreg = im;
-                ++nz;
-              }
-              if (l0 == im) {
-                l0 = l1;
-                l1 = l2;
-              } else if (l1 == im) {
-                l1 = l2;
-              }
-            }
-            r += dlt;
-            flipped = true;
+          for (int j = 0; j < 4; ++j) {
+            u[j] = un[j];
+            top[j] = topn[j];
           }
         }
-        if (flipped) {
-          ++rows_flipped;
-          viol += (r != 1) - (p1.n != 1);
-          __syncwarp();
-          uint2 q = pack_row(r, l0, l1, l2);
-          if (lost) q = record_from_bits<SB>(bits, Cw, C, t, r, lane);
-          if (lane == 0) rec[t] = q;
-          __syncwarp();
+      }
+      if (flipped) {
+        ++rows_flipped;
+        zok = false;
+        viol += (r != 1) - (p1.n != 1);
+        __syncwarp();
+        uint2 q = pack_row(r, r > 0 ? l0 : C, l1, l2);
+        if (lost) q = record_from_bits<SB>(bits, Cw, C, t, r, lane);
+        if (lane == 0) {
+          rec[t] = q;
+          if (r == 1) hx[t] = (uint16_t)D.code((int)(q.x >> 16));
+        }
+        __syncwarp();
+      }
+    };
+
+    // A cold sweep over a permutation (every row and column holds one cell):
+    // only removing a row's own cell can cost less than 2A.  32 rows at a time
+    // and one vote for the sweep.
+    bool quiet = false;
+    if (!hot && viol == 0) {
+      bool any = false;
+#pragma unroll 4
+      for (int t = 1 + lane; t < C; t += 32) {
+        const uint32_t h = hx[t];
+        const int f = D.near(hx[t - 1], h) + (t + 1 < C ? D.near(hx[t + 1], h) : 0);
+        any |= twoA - B * f < len;
+      }
+      quiet = !__any_sync(kFull, any);
+    }
+    // row by row when half the rows are events anyway: rows changed in the last sweep, rows with survivors
+    const float lambda = (float)Q2 * 2.3283064365386963e-10f * (float)C;
+    const bool rowwise = (float)rows_flipped + 0.5f * lambda * (float)C > 0.5f * (float)C;
+    rows_flipped = 0;
+    if (quiet) {
+    } else if (rowwise && C <= 125) {  // a row is one block of 128 columns, whatever t C mod 4
+      hit = true;
+      draws(C, ((uint32_t)C >> 2) + lane, u, top, std::true_type());
+      for (int t = 1; t < C; ++t) event_row(t, std::true_type());
+    } else {
+      for (int t0 = 1; t0 < C; t0 += 32) {
+        const int t1 = min(C, t0 + 32);
+        // -- draws of the window: the rows with survivors
+        uint32_t smask = 0;
+        if (hot && !rowwise) {
+          const uint32_t k0 = (uint32_t)(t0 * C), nk = (uint32_t)((t1 - t0) * C);
+          const uint32_t mend = (k0 + nk - 1) >> 2;
+          auto mark = [&](const uint4 &w4, uint32_t m) {
+            const uint32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const uint32_t rel = 4 * m + j - k0;
+              if (w[j] < Q2 && rel < nk) smask |= 1u << __umulhi(rel, magic);
+            }
+          };
+          for (uint32_t mb = k0 >> 2; mb <= mend; mb += 64) {
+            const uint32_t ma = mb + lane, mc = ma + 32;
+            const uint4 ua = philox4x32_10(make_uint4(ma, (uint32_t)s, rg, kRngTag), key);
+            const uint4 ub = philox4x32_10(make_uint4(mc, (uint32_t)s, rg, kRngTag), key);
+            const uint32_t la = min(min(ua.x, ua.y), min(ua.z, ua.w)), lb = min(min(ub.x, ub.y), min(ub.z, ub.w));
+            if (min(la, lb) < Q2) {
+              mark(ua, ma);
+              mark(ub, mc);
+            }
+          }
+          smask = __reduce_or_sync(kFull, smask);
+        }
+        // -- the window's rows
+        bool have_uh = false;
+        uint32_t uh = 0;  // the draw of the cell of row t0 + lane
+        for (int t = t0; t < t1; ++t) {
+          if (!rowwise && nz <= kZCheck) {
+            if (!zok) {  // list the empty columns
+              int k = 0;
+              for (int i0 = 0; i0 < C && k < nz; i0 += 32) {
+                uint32_t b = __ballot_sync(kFull, i0 + lane < C && cc[i0 + lane] == 0);
+                while (b) {
+                  if (lane == k) zreg = i0 + __ffs(b) - 1;
+                  b &= b - 1;
+                  ++k;
+                }
+              }
+              zok = true;
+            }
+            // the check: lane = row
+            const int tl = t0 + lane;
+            const bool in = tl >= t && tl < t1;
+            const int tr = min(tl, C - 1);
+            const Row p0 = unpack_row(rec[tr - 1]), p1 = unpack_row(rec[tr]), p2 = unpack_row(rec[tr + 1]);
+            bool ev = p1.n != 1 || p0.n > 1 || p2.n > 1 || ((smask >> lane) & 1u);
+            const int h = p1.c0;
+            int dE = len;
+            if (in && !ev) dE = twoA * (2 - (int)cc[h]) - B * (D(p0.c0, h) + D(p2.c0, h));
+            bool need = dE < len;
+            if (__any_sync(kFull, need)) {
+              hit = true;
+              if (!have_uh) {
+                const uint32_t k = (uint32_t)(tr * C + h);
+                const uint4 u4 = philox4x32_10(make_uint4(k >> 2, (uint32_t)s, rg, kRngTag), key);
+                uh = word_of(u4, k & 3);
+                have_uh = true;
+              }
+              if (need) ev = dE <= 0 || accept_draw(uh, dE, cT, thr, len);
+            }
+            for (int q = 0; q < nz; ++q) {
+              const int z = __shfl_sync(kFull, zreg, q);
+              dE = len;
+              if (in && !ev) dE = B * (D(p0.c0, z) + D(p2.c0, z));
+              need = dE < len;
+              if (__any_sync(kFull, need)) {
+                hit = true;
+                const uint32_t k = (uint32_t)(tr * C + z);
+                const uint4 u4 = philox4x32_10(make_uint4(k >> 2, (uint32_t)s, rg, kRngTag), key);
+                if (need) ev = dE <= 0 || accept_draw(word_of(u4, k & 3), dE, cT, thr, len);
+              }
+            }
+            const uint32_t bal = __ballot_sync(kFull, in && ev);
+            if (bal == 0) break;  // nothing happens in the rest of the window
+            t = t0 + __ffs(bal) - 1;
+          }
+          hit = true;
+          event_row(t, std::false_type());
         }
       }
     }
@@ -586,13 +644,13 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
 // Shared memory of one replica.
 __host__ __device__ inline size_t events_warp_bytes(int C, bool bits_smem) {
   const int Cw = (C + 31) >> 5;
-  return align16e(8 * ((size_t)C + 1)) + align16e(2 * ((size_t)C + 2 * kPad)) +
+  return align16e(8 * ((size_t)C + 1)) + align16e(2 * ((size_t)C + 1)) + align16e(2 * ((size_t)C + 2 * kPad)) +
          (bits_smem ? align16e(4 * (size_t)C * Cw) : 0);
 }
 
 // Shared memory of the distances: the matrix (DM = 1) or the coordinates and the table (DM = 2).
 __host__ __device__ inline size_t events_dist_bytes(int C, int Cp, size_t es, int dm, int tab_n) {
-  if (dm == 1) return align16e(((size_t)C * Cp + 2 * kPad) * es);
+  if (dm == 1) return align16e((((size_t)C + 1) * Cp + 2 * kPad) * es);
   if (dm == 2) return align16e(2 * ((size_t)C + 2 * kPad)) + align16e((size_t)tab_n * es);
   return 0;
 }
@@ -605,6 +663,7 @@ __device__ __forceinline__ Dist<DT, DM> stage_dist(const StructArgs &a, unsigned
     const int4 *src = static_cast<const int4 *>(a.d);
     DT *m = reinterpret_cast<DT *>(p) + kPad;
     for (int v = tid; v < nv; v += nthreads) reinterpret_cast<int4 *>(m)[v] = __ldg(src + v);
+    for (int i = tid; i < a.Cp; i += nthreads) m[a.C * a.Cp + i] = 0;
     D.m = m;
   } else if (DM == 2) {
     uint16_t *xy = reinterpret_cast<uint16_t *>(p) + kPad;
@@ -617,6 +676,24 @@ __device__ __forceinline__ Dist<DT, DM> stage_dist(const StructArgs &a, unsigned
   return D;
 }
 
+// A warp's arrays of one replica in shared memory (events_warp_bytes(C, SB)).
+struct WarpArea {
+  uint2 *rec;
+  uint16_t *hx, *cc;
+  uint32_t *bits;  // with SB
+};
+__device__ __forceinline__ WarpArea warp_area(unsigned char *p, int C) {
+  WarpArea w;
+  w.rec = reinterpret_cast<uint2 *>(p);
+  p += align16e(8 * ((size_t)C + 1));
+  w.hx = reinterpret_cast<uint16_t *>(p);
+  p += align16e(2 * ((size_t)C + 1));
+  w.cc = reinterpret_cast<uint16_t *>(p) + kPad;
+  p += align16e(2 * ((size_t)C + 2 * kPad));
+  w.bits = reinterpret_cast<uint32_t *>(p);
+  return w;
+}
+
 template <typename DT, int DM, bool SB>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * 32) k_sweep_events(const StructArgs a, const RoundKeys rk) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -625,14 +702,9 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * 32) k_sweep_events(const Str
   __syncthreads();
   const int rep = blockIdx.x * W + warp;
   if (rep >= a.R) return;  // no CTA-wide barrier after this point
-  const size_t per = events_warp_bytes(a.C, SB);
-  unsigned char *p = smem + events_dist_bytes(a.C, a.Cp, sizeof(DT), DM, a.tab_n) + warp * per;
-  uint2 *rec = reinterpret_cast<uint2 *>(p);
-  p += align16e(8 * ((size_t)a.C + 1));
-  uint16_t *cc = reinterpret_cast<uint16_t *>(p) + kPad;
-  p += align16e(2 * ((size_t)a.C + 2 * kPad));
-  uint32_t *bits = SB ? reinterpret_cast<uint32_t *>(p) : a.gstate + (size_t)rep * a.nw_pad;
-  events_replica<DT, DM, SB>(a, rep, rec, cc, bits, D, lane, rk);
+  const WarpArea w = warp_area(smem + events_dist_bytes(a.C, a.Cp, sizeof(DT), DM, a.tab_n) +
+                                   warp * events_warp_bytes(a.C, SB), a.C);
+  events_replica<DT, DM, SB>(a, rep, w.rec, w.hx, w.cc, SB ? w.bits : a.gstate + (size_t)rep * a.nw_pad, D, lane, rk);
 }
 
 constexpr size_t kSmemLimitEvents = 227 * 1024;
