@@ -22,8 +22,8 @@ using namespace qp::host;
 struct qp_batch {
   int dev = 0;
   int count = 0, R = 0, Cmax = 0, W = 0, blocks = 0, n_units = 0;
-  bool staged = false;
   DevBuf fields, units, counter;
+  DevBuf gstate;  // bitsets of the grid's warps, when they do not live in shared memory
   std::shared_ptr<const void> sched_keep;  // the schedule's tables, referenced by the captured graph
   cudaStream_t cap = nullptr;
   cudaGraph_t graph = nullptr;
@@ -65,7 +65,7 @@ extern "C" qp_status qp_batch_create(qp_handle *const *hs, int32_t count, int32_
   }
   if (o.flags & ~(QP_ANNEAL_SKIP_SETTLED | QP_BATCH_D_SHARED)) return fail(QP_EINVAL, "unknown batch flags");
   const bool staged = (o.flags & QP_BATCH_D_SHARED) != 0;
-  auto fits = [&](int w) { return staged ? batch_staged_supported(Cmax, w) : batch_supported(Cmax, w); };
+  auto fits = [&](int w) { return batch_supported(Cmax, w, staged); };
   int W = o.replicas_per_cta > 0 ? o.replicas_per_cta : 4;
   while (W > 1 && !fits(W)) --W;
   if (!fits(W)) return fail(QP_ERANGE, "largest field (%d cells) too large for the batch kernel", Cmax);
@@ -104,12 +104,13 @@ extern "C" qp_status qp_batch_create(qp_handle *const *hs, int32_t count, int32_
   QP_CU(cudaMemcpy(b->fields.p, fa.data(), fa.size() * sizeof(StructArgs), cudaMemcpyHostToDevice));
   QP_CU(cudaMemcpy(b->units.p, units.data(), units.size() * sizeof(int2), cudaMemcpyHostToDevice));
   int per_sm = 0, sms = 0;
-  QP_CU(staged ? batch_staged_prepare(Cmax, W, &per_sm) : batch_prepare(Cmax, W, &per_sm));
+  size_t gwords = 0;
+  QP_CU(events_batch_prepare(Cmax, W, staged, &per_sm, &gwords));
   QP_CU(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, b->dev));
   if (per_sm < 1) return fail(QP_ERANGE, "batch kernel does not fit on an SM");
   const int want = o.ctas > 0 ? o.ctas : per_sm * sms;
   b->blocks = std::min(want, staged ? (int)units.size() : (int)((units.size() + W - 1) / W));
-  b->staged = staged;
+  if (gwords) QP_TRY(b->gstate.ensure((size_t)b->blocks * W * gwords * 4));
   b->count = count; b->R = R; b->Cmax = Cmax; b->W = W; b->n_units = (int)units.size();
   // one graph: reset the queue head, run the persistent kernel
   QP_CU(cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking));
@@ -117,10 +118,8 @@ extern "C" qp_status qp_batch_create(qp_handle *const *hs, int32_t count, int32_
   cudaError_t e1 = cudaMemsetAsync(b->counter.p, 0, sizeof(int), b->cap);
   cudaError_t e2 = e1;
   if (e1 == cudaSuccess)
-    e2 = staged ? launch_batch_staged(b->fields.as<StructArgs>(), b->units.as<int2>(), b->n_units,
-                                      b->counter.as<int>(), Cmax, W, b->blocks, b->cap)
-                : launch_batch(b->fields.as<StructArgs>(), b->units.as<int2>(), b->n_units, b->counter.as<int>(),
-                               Cmax, W, b->blocks, b->cap);
+    e2 = launch_events_batch(b->fields.as<StructArgs>(), b->units.as<int2>(), b->n_units, b->counter.as<int>(), Cmax, W,
+                             staged, b->blocks, b->gstate.as<uint32_t>(), b->cap);
   cudaError_t e3 = cudaStreamEndCapture(b->cap, &b->graph);
   if (e2 != cudaSuccess) return fail(QP_ECUDA, "capturing the batch graph: %s", cudaGetErrorString(e2));
   if (e3 != cudaSuccess) return fail(QP_ECUDA, "capturing the batch graph: %s", cudaGetErrorString(e3));

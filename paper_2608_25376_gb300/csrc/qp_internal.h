@@ -114,19 +114,16 @@ cudaError_t launch_rows(const StructArgs &a, bool d_i16, int warps_per_cta, cuda
 // (warps_per_cta 0 = chosen from the replica count).
 size_t events_state_words(int C);
 cudaError_t launch_events(const StructArgs &a, bool d_i16, int warps_per_cta, cudaStream_t st, LaunchInfo *info);
-// Batched persistent launch (qp_sweep_rows.cu): fields[] per field, units[]
+// Batched persistent launch (qp_sweep_events.cu): fields[] per field, units[]
 // = (field, replica) in processing order, counter = the work-queue head (zeroed
-// before each launch).  All fields must use int16 distances.
-bool batch_supported(int Cmax, int warps_per_cta);
-cudaError_t batch_prepare(int Cmax, int warps_per_cta, int *blocks_per_sm);
-cudaError_t launch_batch(const StructArgs *fields, const int2 *units, int n_units, int *counter, int Cmax,
-                         int warps_per_cta, int blocks, cudaStream_t st);
-// The batched launch with each field's d staged in shared memory (units of W
-// replicas of one field per CTA).
-bool batch_staged_supported(int Cmax, int warps_per_cta);
-cudaError_t batch_staged_prepare(int Cmax, int warps_per_cta, int *blocks_per_sm);
-cudaError_t launch_batch_staged(const StructArgs *fields, const int2 *units, int n_units, int *counter, int Cmax,
-                                int warps_per_cta, int blocks, cudaStream_t st);
+// before each launch).  All fields must use int16 distances.  staged: a unit is
+// W replicas of one field, whose d the CTA stages in shared memory.
+// batch_supported: the shapes the batch entry points take.  gstate: blocks x W
+// x gstate_words words (none when 0).
+bool batch_supported(int Cmax, int warps_per_cta, bool staged);
+cudaError_t events_batch_prepare(int Cmax, int W, bool staged, int *blocks_per_sm, size_t *gstate_words);
+cudaError_t launch_events_batch(const StructArgs *fields, const int2 *units, int n_units, int *counter, int Cmax, int W,
+                                bool staged, int blocks, uint32_t *gstate, cudaStream_t st);
 // Grouped structured kernel (qp_sweep_group.cu): 4 replicas per warp for
 // C <= 64, 2 for C <= 128.
 int group_size_for(int C);

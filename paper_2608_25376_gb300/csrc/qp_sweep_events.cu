@@ -707,6 +707,65 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * 32) k_sweep_events(const Str
   events_replica<DT, DM, SB>(a, rep, w.rec, w.hx, w.cc, SB ? w.bits : a.gstate + (size_t)rep * a.nw_pad, D, lane, rk);
 }
 
+// Many fields in one persistent launch: a warp takes (field, replica) units
+// from a counter, largest fields first, and reads the field's matrix through
+// L1 (consecutive units are replicas of the same field).  No warp waits on
+// another.  per: shared memory of a warp, sized for the largest field;
+// gbits: one replica's bitsets per warp of the grid (without SB).  256 fields
+// of 10-169 cells x 128 replicas x 2000 sweeps: 198 ms (the row kernel's batch:
+// 1190), 182 with the matrix staged in shared memory by 8 warps (1054).  At 128
+// registers and 16 warps per SM: 96 registers (20 warps) 273, 168 (12 warps) 216.
+template <bool SB>
+__global__ void __launch_bounds__(kMaxWarpsPerCta * 32)
+    k_events_batch(const StructArgs *fields, const int2 *units, int n_units, int *counter, size_t per, uint32_t *gbits,
+                   int gwords) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+  while (true) {
+    int u = 0;
+    if (lane == 0) u = atomicAdd(counter, 1);
+    u = __shfl_sync(kFull, u, 0);
+    if (u >= n_units) break;
+    const int2 unit = units[u];
+    const StructArgs &a = fields[unit.x];
+    const Dist<int16_t, 0> D{static_cast<const int16_t *>(a.d), a.Cp, a.C, nullptr, 0, 0};
+    const WarpArea w = warp_area(smem + warp * per, a.C);
+    events_replica<int16_t, 0, SB>(a, unit.y, w.rec, w.hx, w.cc,
+                                   SB ? w.bits : gbits + (size_t)(blockIdx.x * W + warp) * gwords, D, lane,
+                                   PhiloxKey{a.key0, a.key1});
+    __syncwarp();
+  }
+}
+
+// The same with units of W replicas of one field per CTA, whose matrix the CTA
+// stages in shared memory.
+template <bool SB>
+__global__ void __launch_bounds__(kMaxWarpsPerCta * 32)
+    k_events_batch_staged(const StructArgs *fields, const int2 *units, int n_units, int *counter, size_t dist,
+                          size_t per, uint32_t *gbits, int gwords) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ int s_unit;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
+  while (true) {
+    if (threadIdx.x == 0) s_unit = atomicAdd(counter, 1);
+    __syncthreads();
+    const int u = s_unit;
+    if (u >= n_units) break;  // the same u in every thread
+    const int2 unit = units[u];
+    const StructArgs &a = fields[unit.x];
+    const Dist<int16_t, 1> D = stage_dist<int16_t, 1>(a, smem, threadIdx.x, blockDim.x);
+    __syncthreads();
+    const int rep = unit.y + warp;
+    if (rep < a.R) {
+      const WarpArea w = warp_area(smem + dist + warp * per, a.C);
+      events_replica<int16_t, 1, SB>(a, rep, w.rec, w.hx, w.cc,
+                                     SB ? w.bits : gbits + (size_t)(blockIdx.x * W + warp) * gwords, D, lane,
+                                     PhiloxKey{a.key0, a.key1});
+    }
+    __syncthreads();  // every warp is done with the matrix and s_unit before the next unit
+  }
+}
+
 constexpr size_t kSmemLimitEvents = 227 * 1024;
 constexpr size_t kBitsSmem = 8 * 1024;       // most bytes of a replica's bitsets kept in shared memory
 constexpr size_t kMatrixSmem = 40 * 1024;    // largest distance matrix staged in shared memory
@@ -781,6 +840,73 @@ cudaError_t launch_events(const StructArgs &a_in, bool d_i16, int W, cudaStream_
     rk.k[2 * i + 1] = a.key1 + (uint32_t)i * 0xBB67AE85u;
   }
   return d_i16 ? launch_e2<int16_t>(a, rk, s, W, smem, st) : launch_e2<int32_t>(a, rk, s, W, smem, st);
+}
+
+namespace {
+
+// The batched launch's shared memory: bitsets in shared memory when a replica's
+// are small and the CTA's fit.
+struct BatchShape {
+  bool sb;
+  size_t dist, per, smem;
+};
+BatchShape batch_shape(int Cmax, int W, bool staged) {
+  BatchShape b;
+  b.dist = staged ? events_dist_bytes(Cmax, (Cmax + 7) / 8 * 8, 2, 1, 0) : 0;
+  b.sb = 4 * (size_t)Cmax * ((Cmax + 31) / 32) <= kBitsSmem;
+  b.per = events_warp_bytes(Cmax, b.sb);
+  if (b.sb && b.dist + W * b.per > kSmemLimitEvents) {
+    b.sb = false;
+    b.per = events_warp_bytes(Cmax, false);
+  }
+  b.smem = b.dist + W * b.per;
+  return b;
+}
+
+template <typename K>
+cudaError_t prepare_batch(K k, int W, size_t smem, int *blocks_per_sm) {
+  std::lock_guard<std::mutex> lk(launch_mutex());
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, W * 32, smem);
+}
+
+}  // namespace
+
+// Up to 512 cells, 16 replicas per CTA (8 above 256 cells) whose bitsets and
+// one 2-byte entry per row fit 227 KB beside the staged matrix: the entry
+// points' limits, which all fit the kernel's own layout too.
+bool batch_supported(int Cmax, int W, bool staged) {
+  if (Cmax < 2 || Cmax > 512 || W < 1 || W > (Cmax <= 256 ? kMaxWarpsPerCta : 8)) return false;
+  const size_t bits = ((size_t)Cmax * ((Cmax + 31) / 32) + 3) / 4 * 16;
+  const size_t d = staged ? align16e((size_t)Cmax * ((Cmax + 7) / 8 * 8) * 2) : 0;
+  return d + W * (bits + align16e(2 * (size_t)Cmax)) <= kSmemLimitEvents;
+}
+
+cudaError_t events_batch_prepare(int Cmax, int W, bool staged, int *blocks_per_sm, size_t *gstate_words) {
+  const BatchShape b = batch_shape(Cmax, W, staged);
+  *gstate_words = b.sb ? 0 : ((size_t)Cmax * ((Cmax + 31) / 32) + 3) / 4 * 4;
+  if (b.smem > kSmemLimitEvents) return cudaErrorInvalidValue;
+  if (staged)
+    return b.sb ? prepare_batch(k_events_batch_staged<true>, W, b.smem, blocks_per_sm)
+                : prepare_batch(k_events_batch_staged<false>, W, b.smem, blocks_per_sm);
+  return b.sb ? prepare_batch(k_events_batch<true>, W, b.smem, blocks_per_sm)
+              : prepare_batch(k_events_batch<false>, W, b.smem, blocks_per_sm);
+}
+
+cudaError_t launch_events_batch(const StructArgs *fields, const int2 *units, int n_units, int *counter, int Cmax, int W,
+                                bool staged, int blocks, uint32_t *gstate, cudaStream_t st) {
+  const BatchShape b = batch_shape(Cmax, W, staged);
+  if (b.smem > kSmemLimitEvents || blocks < 1 || (!b.sb && gstate == nullptr)) return cudaErrorInvalidValue;
+  const int gwords = (Cmax * ((Cmax + 31) / 32) + 3) / 4 * 4;
+  if (staged) {
+    if (b.sb) k_events_batch_staged<true><<<blocks, W * 32, b.smem, st>>>(fields, units, n_units, counter, b.dist, b.per, gstate, gwords);
+    else k_events_batch_staged<false><<<blocks, W * 32, b.smem, st>>>(fields, units, n_units, counter, b.dist, b.per, gstate, gwords);
+  } else {
+    if (b.sb) k_events_batch<true><<<blocks, W * 32, b.smem, st>>>(fields, units, n_units, counter, b.per, gstate, gwords);
+    else k_events_batch<false><<<blocks, W * 32, b.smem, st>>>(fields, units, n_units, counter, b.per, gstate, gwords);
+  }
+  return cudaGetLastError();
 }
 
 }  // namespace qp

@@ -44,8 +44,7 @@ using namespace dev;
 #include "qp_rows.cuh"
 
 // One replica of a field through the sweeps [sweep_begin, sweep_end): the
-// whole chain of the row kernel, shared by the single-field launch and the
-// batched persistent launch.  st: the replica's C x Cw row bitsets; hot1: its
+// whole chain of the row kernel.  st: the replica's C x Cw row bitsets; hot1: its
 // per-row single-cell cache (C entries); d: the distance matrix (global or
 // shared memory, per DMODE).
 template <typename DT, int NCH, int DMODE, int LA>
@@ -661,70 +660,7 @@ __global__ void __launch_bounds__(rows_max_warps<NCH>() * 32) k_sweep_rows(const
   rows_replica<DT, NCH, DMODE, DMODE == 0 ? 2 : 1>(a, r, st, hot1, d, lane);
 }
 
-// Batched persistent sweep: many fields of uneven size in one launch.  Each
-// warp takes (field, replica) units from a global counter until none are left
-// and runs the same chain as k_sweep_rows for that replica; units are ordered
-// largest field first so the tail is made of short units.  Taking a unit is
-// one atomicAdd: no warp ever waits on another.  The distance matrices are
-// read from L2 (all fields of a batch together are a few MB).
-template <int NCH>
-__global__ void __launch_bounds__(rows_max_warps<NCH>() * 32)
-    k_sweep_batch(const StructArgs *fields, const int2 *units, int n_units, int *counter, int nw_pad_max,
-                  int Cmax) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const size_t per_warp = 4 * (size_t)nw_pad_max + align16r(2 * (size_t)Cmax);
-  uint32_t *st = reinterpret_cast<uint32_t *>(smem + warp * per_warp);
-  int16_t *hot1 = reinterpret_cast<int16_t *>(smem + warp * per_warp + 4 * (size_t)nw_pad_max);
-  while (true) {
-    int u = 0;
-    if (lane == 0) u = atomicAdd(counter, 1);
-    u = __shfl_sync(kFull, u, 0);
-    if (u >= n_units) break;
-    const int2 unit = units[u];
-    const StructArgs a = fields[unit.x];
-    rows_replica<int16_t, NCH, 0, 1>(a, unit.y, st, hot1, a.d, lane);
-    __syncwarp();
-  }
-}
-
 constexpr size_t kSmemLimitRows = 227 * 1024;
-
-// The batched launch with each field's distance matrix staged in shared
-// memory: a CTA takes a unit of W replicas of one field (W = its warps), copies
-// the field's int16 d into shared memory, runs one replica per warp against it
-// and, once every warp is done, takes the next unit.  The autotuner times it
-// against k_sweep_batch (d read from L2, units of one replica per warp).
-template <int NCH>
-__global__ void __launch_bounds__(rows_max_warps<NCH>() * 32)
-    k_sweep_batch_staged(const StructArgs *fields, const int2 *units, int n_units, int *counter, int nw_pad_max,
-                         int Cmax, int Cpmax) {
-  extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ int s_unit;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int16_t *dsm = reinterpret_cast<int16_t *>(smem);
-  const size_t dbytes = align16r((size_t)Cmax * Cpmax * 2);
-  const size_t per_warp = 4 * (size_t)nw_pad_max + align16r(2 * (size_t)Cmax);
-  uint32_t *st = reinterpret_cast<uint32_t *>(smem + dbytes + warp * per_warp);
-  int16_t *hot1 = reinterpret_cast<int16_t *>(smem + dbytes + warp * per_warp + 4 * (size_t)nw_pad_max);
-  while (true) {
-    if (threadIdx.x == 0) s_unit = atomicAdd(counter, 1);
-    __syncthreads();
-    const int u = s_unit;
-    if (u >= n_units) break;  // the same u in every thread
-    const int2 unit = units[u];
-    const StructArgs a = fields[unit.x];
-    const int nv = (int)((size_t)a.C * a.Cp * 2 / 16);  // Cp is a multiple of 8
-    const int4 *src = static_cast<const int4 *>(a.d);
-    for (int v = threadIdx.x; v < nv; v += blockDim.x) reinterpret_cast<int4 *>(dsm)[v] = __ldg(src + v);
-    __syncthreads();
-    const int r = unit.y + warp;
-    if (r < a.R) rows_replica<int16_t, NCH, 1, 1>(a, r, st, hot1, dsm, lane);
-    __syncthreads();  // every warp is done with d and s_unit before the next unit
-  }
-}
-
-
 
 template <typename DT, int NCH, int DMODE>
 cudaError_t launch_r(const StructArgs &a, int W, size_t smem, cudaStream_t st) {
@@ -763,85 +699,6 @@ size_t rows_smem(int C, bool d_i16, int W, int dmode) {
 bool rows_supported(int C, bool d_i16, int W) {
   const int wmax = C <= 256 ? kMaxWarpsPerCta : 8;
   return C <= 512 && W >= 1 && W <= wmax && rows_smem(C, d_i16, W, 0) <= kSmemLimitRows;
-}
-
-size_t batch_smem(int Cmax, int W) {
-  return (size_t)W * (4 * rows_state_words(Cmax) + align16r(2 * (size_t)Cmax));
-}
-
-bool batch_supported(int Cmax, int W) {
-  const int wmax = Cmax <= 256 ? kMaxWarpsPerCta : 8;
-  return Cmax >= 2 && Cmax <= 512 && W >= 1 && W <= wmax && batch_smem(Cmax, W) <= kSmemLimitRows;
-}
-
-template <int NCH>
-static cudaError_t prep_batch(int W, size_t smem, int *blocks_per_sm) {
-  auto k = k_sweep_batch<NCH>;
-  std::lock_guard<std::mutex> lk(launch_mutex());
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, W * 32, smem);
-}
-
-cudaError_t batch_prepare(int Cmax, int W, int *blocks_per_sm) {
-  if (!batch_supported(Cmax, W)) return cudaErrorInvalidValue;
-  const size_t smem = batch_smem(Cmax, W);
-  if (Cmax <= 128) return prep_batch<1>(W, smem, blocks_per_sm);
-  if (Cmax <= 256) return prep_batch<2>(W, smem, blocks_per_sm);
-  return prep_batch<4>(W, smem, blocks_per_sm);
-}
-
-size_t batch_staged_smem(int Cmax, int W) {
-  const int Cpmax = (Cmax + 7) / 8 * 8;
-  return align16r((size_t)Cmax * Cpmax * 2) + batch_smem(Cmax, W);
-}
-
-bool batch_staged_supported(int Cmax, int W) {
-  const int wmax = Cmax <= 256 ? kMaxWarpsPerCta : 8;
-  return Cmax >= 2 && Cmax <= 512 && W >= 1 && W <= wmax && batch_staged_smem(Cmax, W) <= kSmemLimitRows;
-}
-
-template <int NCH>
-static cudaError_t prep_batch_staged(int W, size_t smem, int *blocks_per_sm) {
-  auto k = k_sweep_batch_staged<NCH>;
-  std::lock_guard<std::mutex> lk(launch_mutex());
-  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, k, W * 32, smem);
-}
-
-cudaError_t batch_staged_prepare(int Cmax, int W, int *blocks_per_sm) {
-  if (!batch_staged_supported(Cmax, W)) return cudaErrorInvalidValue;
-  const size_t smem = batch_staged_smem(Cmax, W);
-  if (Cmax <= 128) return prep_batch_staged<1>(W, smem, blocks_per_sm);
-  if (Cmax <= 256) return prep_batch_staged<2>(W, smem, blocks_per_sm);
-  return prep_batch_staged<4>(W, smem, blocks_per_sm);
-}
-
-cudaError_t launch_batch_staged(const StructArgs *fields, const int2 *units, int n_units, int *counter, int Cmax,
-                                int W, int blocks, cudaStream_t st) {
-  if (!batch_staged_supported(Cmax, W) || blocks < 1) return cudaErrorInvalidValue;
-  const size_t smem = batch_staged_smem(Cmax, W);
-  const int nwp = (int)rows_state_words(Cmax);
-  const int Cpmax = (Cmax + 7) / 8 * 8;
-  if (Cmax <= 128)
-    k_sweep_batch_staged<1><<<blocks, W * 32, smem, st>>>(fields, units, n_units, counter, nwp, Cmax, Cpmax);
-  else if (Cmax <= 256)
-    k_sweep_batch_staged<2><<<blocks, W * 32, smem, st>>>(fields, units, n_units, counter, nwp, Cmax, Cpmax);
-  else
-    k_sweep_batch_staged<4><<<blocks, W * 32, smem, st>>>(fields, units, n_units, counter, nwp, Cmax, Cpmax);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_batch(const StructArgs *fields, const int2 *units, int n_units, int *counter, int Cmax,
-                         int W, int blocks, cudaStream_t st) {
-  if (!batch_supported(Cmax, W) || blocks < 1) return cudaErrorInvalidValue;
-  const size_t smem = batch_smem(Cmax, W);
-  const int nwp = (int)rows_state_words(Cmax);
-  if (Cmax <= 128) k_sweep_batch<1><<<blocks, W * 32, smem, st>>>(fields, units, n_units, counter, nwp, Cmax);
-  else if (Cmax <= 256) k_sweep_batch<2><<<blocks, W * 32, smem, st>>>(fields, units, n_units, counter, nwp, Cmax);
-  else k_sweep_batch<4><<<blocks, W * 32, smem, st>>>(fields, units, n_units, counter, nwp, Cmax);
-  return cudaGetLastError();
 }
 
 namespace {
