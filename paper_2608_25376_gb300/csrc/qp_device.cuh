@@ -89,6 +89,21 @@ __device__ __forceinline__ uint32_t word_of(const uint4 &u, int j) {
   return j == 0 ? u.x : (j == 1 ? u.y : (j == 2 ? u.z : u.w));
 }
 
+// f(k0 + b) for every byte b of q that is not zero.
+template <typename F>
+__device__ __forceinline__ void each_set_byte(const uint4 &q, int k0, F &&f) {
+  if ((q.x | q.y | q.z | q.w) == 0) return;
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    uint32_t w = g == 0 ? q.x : (g == 1 ? q.y : (g == 2 ? q.z : q.w));
+    while (w) {
+      const int b = (__ffs(w) - 1) >> 3;
+      w &= ~(0xFFu << (8 * b));
+      f(k0 + 4 * g + b);
+    }
+  }
+}
+
 __device__ __forceinline__ long long warp_sum64(long long v) {
 #pragma unroll
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
