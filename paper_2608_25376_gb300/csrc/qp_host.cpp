@@ -818,6 +818,12 @@ bool handle_struct_view(const qp_handle *h, StructView *out) {
   out->max_d = h->max_d;
   out->d32 = h->d32_dev.as<int32_t>();
   out->weighted = h->weighted;
+  StructArgs a{};
+  fill_field_args(h, a);
+  out->xy = a.xy;
+  out->tab = a.tab;
+  out->tab_sh = a.tab_sh;
+  out->tab_n = a.tab_n;
   return true;
 }
 

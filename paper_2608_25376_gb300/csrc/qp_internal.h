@@ -169,6 +169,9 @@ struct StructView {
   bool d_i16;
   const int32_t *d32;  // C x C int32 on the device
   bool weighted;       // leg weights on the distance term (the structured kernels do not apply them)
+  const uint16_t *xy;  // coordinates and distance table (StructArgs)
+  const void *tab;
+  int32_t tab_sh, tab_n;
 };
 bool handle_struct_view(const qp_handle *h, StructView *out);  // false for a generic QUBO
 // false if not cached on this device; *keep (may be NULL) holds the tables alive
