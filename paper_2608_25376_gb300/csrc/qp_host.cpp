@@ -318,7 +318,7 @@ static qp_status build_field_qubo(const qp_field *f, int32_t A, int32_t B, int32
   h->C = C;
   h->n = (int64_t)C * C;
   h->d.resize((size_t)C * C);
-  int64_t maxd = 0;
+  int64_t maxd = 0, mind = INT32_MAX;
   for (int i = 0; i < C; ++i)
     for (int j = 0; j < C; ++j) {
       const int64_t dr = cr[i] - cr[j], dc = cc[i] - cc[j];
@@ -326,8 +326,10 @@ static qp_status build_field_qubo(const qp_field *f, int32_t A, int32_t B, int32
       if (v > INT32_MAX) return fail(QP_ERANGE, "distance beyond int32");
       h->d[(size_t)i * C + j] = (int32_t)v;
       maxd = std::max(maxd, v);
+      if (i != j) mind = std::min(mind, v);
     }
   h->max_d = (int32_t)maxd;
+  h->min_d = (int32_t)mind;
   const int64_t Aeff = A > 0 ? A : 2 * maxd * (w ? std::max<int64_t>(1, maxw) : 1);
   if (Aeff > INT32_MAX / 4) return fail(QP_ERANGE, "penalty A beyond int32/4");
   h->A = (int32_t)Aeff;
@@ -543,6 +545,12 @@ void fill_field_args(const qp_handle *h, StructArgs &a) {
   a.xy = reinterpret_cast<const uint16_t *>(h->d_dev.as<uint8_t>() + h->xy_at);
   a.tab = h->d_dev.as<uint8_t>() + h->tab_at;
   a.tab_sh = h->tab_sh; a.tab_n = h->tab_n;
+}
+
+RepairField repair_field(const qp_handle *h) {
+  StructArgs a{};
+  fill_field_args(h, a);
+  return RepairField{h->C, h->start, h->d32_dev.as<int32_t>(), a.xy, a.tab, a.tab_sh, a.tab_n, h->d_i16, h->min_d};
 }
 
 qp_status launch_structured_events(qp_handle *h, StructArgs &a, int W, cudaStream_t st, LaunchInfo *info) {

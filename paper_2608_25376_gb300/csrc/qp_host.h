@@ -116,7 +116,7 @@ struct qp_handle {
   int dev = 0;
   bool path = false;       // built from a field (structured terms available)
   bool weighted = false;   // per-leg weights on the distance term: the dense form only
-  int32_t C = 0, start = 0, A = 0, B = 0, max_d = 0;
+  int32_t C = 0, start = 0, A = 0, B = 0, max_d = 0, min_d = 0;  // min_d: of two different cells
   int64_t n = 0, c0 = 0;
   std::vector<int32_t> d;  // C x C (host)
   // device data
@@ -145,6 +145,7 @@ namespace qp {
 namespace host {
 // The field's part of a structured launch's arguments.
 void fill_field_args(const qp_handle *h, StructArgs &a);
+RepairField repair_field(const qp_handle *h);
 // The structured sweep of a.R replicas: the row kernel when allowed and the
 // field fits it, else the flat kernel.
 // W = replicas per CTA, 0 = chosen from the occupancy (row kernel) or 4 (flat kernel)

@@ -141,10 +141,18 @@ cudaError_t launch_decode(const uint8_t *states, int32_t R, int32_t C, const int
 // Read-only views used by the allocation-free entry point (qp_noalloc.cu);
 // none of these allocate.
 // Repair of R states into paths (greedy fix + 2-opt), one warp per replica.
+struct RepairField {
+  int32_t C, start;
+  const int32_t *d32;  // C x C
+  const uint16_t *xy;  // coordinates and distance table (StructArgs)
+  const void *tab;
+  int32_t tab_sh, tab_n;
+  bool d_i16;          // the table's type
+  int32_t min_d;       // smallest distance of two cells
+};
 size_t repair_smem_per_warp(int32_t C);
-cudaError_t launch_repair(const uint8_t *states, int32_t R, int32_t C, int32_t start, const int32_t *d32,
-                          int32_t max_passes, int32_t *paths, int64_t *lengths, int32_t *status,
-                          cudaStream_t st);
+cudaError_t launch_repair(const uint8_t *states, int32_t R, const RepairField &f, int32_t max_passes, int32_t *paths,
+                          int64_t *lengths, int32_t *status, cudaStream_t st);
 
 // Replica exchange round (qp_pt.cu).
 struct PtArgs {

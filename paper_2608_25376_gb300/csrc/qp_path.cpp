@@ -48,7 +48,7 @@ extern "C" qp_status qp_repair_batch(const qp_handle *hc, int32_t R, const uint8
   if (ph) { QP_TRY(h->p_stage.ensure((size_t)R * h->C * 4)); pd = h->p_stage.as<int32_t>(); }
   if (lh) { QP_TRY(h->l_stage.ensure((size_t)R * 8)); ld = h->l_stage.as<int64_t>(); }
   if (!status_out || rh) { QP_TRY(h->r_stage.ensure((size_t)R * 4)); rd = h->r_stage.as<int32_t>(); }
-  QP_CU(launch_repair(sd, R, h->C, h->start, h->d32_dev.as<int32_t>(), max_passes, pd, ld, rd, st));
+  QP_CU(launch_repair(sd, R, repair_field(h), max_passes, pd, ld, rd, st));
   if (ph) QP_CU(cudaMemcpyAsync(paths_out, pd, (size_t)R * h->C * 4, cudaMemcpyDeviceToHost, st));
   if (lh) QP_CU(cudaMemcpyAsync(lengths_out, ld, (size_t)R * 8, cudaMemcpyDeviceToHost, st));
   if (rh) QP_CU(cudaMemcpyAsync(status_out, rd, (size_t)R * 4, cudaMemcpyDeviceToHost, st));
@@ -125,7 +125,7 @@ extern "C" qp_status qp_anneal_timed(qp_handle *h, int32_t R, const qp_schedule 
   // Repair the R final states in `S`, fold them into `best` (shortest path,
   // ties to the smaller replica index) and keep the winner's path and state.
   auto harvest = [&](const uint8_t *S, int32_t offset) -> qp_status {
-    QP_CU(launch_repair(S, R, C, h->start, h->d32_dev.as<int32_t>(), max_passes, Pd, Ld, Sd, st));
+    QP_CU(launch_repair(S, R, repair_field(h), max_passes, Pd, Ld, Sd, st));
     QP_CU(cudaMemcpyAsync(len.data(), Ld, (size_t)R * 8, cudaMemcpyDeviceToHost, st));
     QP_CU(cudaMemcpyAsync(stat.data(), Sd, (size_t)R * 4, cudaMemcpyDeviceToHost, st));
     QP_CU(cudaMemcpyAsync(en.data(), E, (size_t)R * 8, cudaMemcpyDeviceToHost, st));
