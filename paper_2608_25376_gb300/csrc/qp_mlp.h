@@ -34,12 +34,24 @@ struct GemmArgs {
   int *err;  // set to 1 if a bounded wait gave up
 };
 
-cudaError_t gemm(const GemmArgs &g, int splits, cudaStream_t st);
+constexpr int kMaxGroup = 4;
+// `count` products in one launch, each in the same number of K-splits (their
+// tiles run side by side: one product of the weight gradients fills a fifth of
+// the SMs).
+cudaError_t gemm(const GemmArgs *g, int count, int splits, cudaStream_t st);
 // The number of K-splits gemm() launches for K and the requested splits.
 int gemm_splits(int K, int splits);
-// out[i] = sum over z = 0 .. splits-1, in that order, of ws[z * n + i]: the
-// split-K partials of a kEpiPartialF32 gemm, added the same way on every run.
-cudaError_t sum_splits(const float *ws, int splits, int n, float *out, cudaStream_t st);
+// out[i] = sum over z = 0 .. splits-1, in that order, of ws[z * n + i]: split-K
+// partials, or slabs of column sums, added the same way on every run.  Every job
+// runs in the same launch, and v's ordered sum into v_sum beside them (v may
+// be null): thread j of 256 adds v[j], v[j + 256], ...; then the 256 in order.
+struct SumJob {
+  const float *ws;
+  int splits, n;
+  float *out;
+};
+constexpr int kMaxSums = 8;
+cudaError_t sum_jobs(const SumJob *jobs, int count, const float *v, int nv, float *v_sum, cudaStream_t st);
 
 // The network's whole forward pass in one launch, one CTA per 128-row tile:
 // x0 bf16 [Mp x 16] (Mp a multiple of 128), weights w[l] bf16 [256 x K_l]
@@ -50,22 +62,57 @@ struct FwdArgs {
   const float *bias[4];
   __nv_bfloat16 *h[3];
   float *z;
+  float *z2;  // a second copy of the first rows2 rows of z (null: none; 16-byte aligned)
+  int rows2;
   int Mp;
   int *err;  // set to 1 if a bounded wait gave up
 };
 cudaError_t forward(const FwdArgs &g, const __nv_bfloat16 *const w[4], cudaStream_t st);
-// loss_rows[m] = -log p[label] of row m (0 for a padding row); loss_sum[0]
-// = their sum, added in a fixed order.
-cudaError_t softmax_ce(const float *Z, int ldz, const int32_t *label, const int32_t *steps, int M, float inv_rows,
-                       __nv_bfloat16 *dZ, int ldd, float *loss_rows, float *loss_sum, cudaStream_t st);
-// out[n] = sum_m Y[m][n], in a fixed order: per slab of rows into partial
-// (kColsumSlabs x N floats), then the slabs in order.
+// From the logits to the gradients at the hidden activations, in two launches:
+// dz bf16 [Mp x 256] = the softmax cross-entropy's
+// gradient times inv_rows, loss_rows[m] = -log p[label] of row m (0 for a
+// padding row, label < 0), dh[l] bf16 [Mp x 256] = relu'(h[l]) * dY W of the layer
+// above.  wt[l]: the transposed weights of layer l (0-based; wt[0] is not read).
+struct BwdArgs {
+  const float *z;
+  const int32_t *label, *steps;
+  float inv_rows;
+  const __nv_bfloat16 *h[3];
+  __nv_bfloat16 *dz, *dh[3];
+  float *loss_rows;
+  int Mp;
+  int *err;  // set to 1 if a bounded wait gave up
+};
+cudaError_t backward(const BwdArgs &g, const __nv_bfloat16 *const wt[4], cudaStream_t st);
+// Column sums of `count` bf16 matrices Y[k] [M x 256], per slab of rows:
+// partial + k * kColsumSlabs * 256 gets kColsumSlabs x 256 floats.
 constexpr int kColsumSlabs = 64;
-cudaError_t colsum(const __nv_bfloat16 *Y, int ld, int M, int N, float *partial, float *out, cudaStream_t st);
-cudaError_t transpose(const __nv_bfloat16 *in, int R, int C, int ldi, __nv_bfloat16 *out, int ldo, cudaStream_t st);
-cudaError_t adam(float *w, float *m, float *v, const float *g, int rows, int cols, float lr, float b1, float b2,
-                 float eps, int step, __nv_bfloat16 *wb, __nv_bfloat16 *wt, cudaStream_t st);
-cudaError_t to_bf16(const float *in, __nv_bfloat16 *out, int n, cudaStream_t st);
+cudaError_t colsum(const __nv_bfloat16 *const *Y, int count, int M, float *partial, cudaStream_t st);
+// out (cols x rows, row stride rows) = in (rows x cols, contiguous), bf16, for
+// every job; cols a multiple of 2, rows a multiple of 64.
+struct TransposeJob {
+  const __nv_bfloat16 *in;
+  __nv_bfloat16 *out;
+  int cols;
+};
+constexpr int kMaxTransposes = 8;
+cudaError_t transpose(const TransposeJob *jobs, int count, int rows, cudaStream_t st);
+
+// The parameters in one flat array: W1[256][16], b1[256], then W[256][256],
+// b[256] of the other three layers.  wb, wt: the bf16 weights and their
+// transposes at the weights' offsets.
+constexpr int kParams = 256 * 16 + 256 + 3 * (256 * 256 + 256);
+constexpr int weight_offset(int l) { return l == 0 ? 0 : 256 * 16 + 256 + (l - 1) * (256 * 256 + 256); }
+constexpr int bias_offset(int l) { return weight_offset(l) + 256 * (l == 0 ? 16 : 256); }
+// One Adam step on all of them (Kingma & Ba); nothing happens when *err != 0.
+cudaError_t adam(float *w, float *m, float *v, const float *g, float lr, float b1, float b2, float eps, int step,
+                 __nv_bfloat16 *wb, __nv_bfloat16 *wt, const int *err, cudaStream_t st);
+// wb and wt from the fp32 parameters.
+cudaError_t refresh(const float *w, __nv_bfloat16 *wb, __nv_bfloat16 *wt, cudaStream_t st);
+// The inputs of a pass: x0 (bf16 [Mp x 16]) from M rows of fp32 features, zero
+// rows after them; with labels, their padding rows (label -1, steps 1).
+cudaError_t inputs(const float *feats, int M, int Mp, __nv_bfloat16 *x0, int32_t *labels, int32_t *steps,
+                   cudaStream_t st);
 
 }  // namespace mlp
 }  // namespace qp

@@ -10,6 +10,8 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <memory>
+#include <utility>
 #include <vector>
 
 #include "qp_internal.h"
@@ -57,14 +59,6 @@ struct Buf {
     if (!(buf).ensure(bytes)) return set_error(QP_ENOMEM, "warm start: cudaMalloc failed"); \
   } while (0)
 
-uint16_t f32_to_bf16_bits(float f) {
-  uint32_t u;
-  std::memcpy(&u, &f, 4);
-  if ((u & 0x7F800000u) == 0x7F800000u) return (uint16_t)(u >> 16);  // inf / nan
-  u += 0x7FFFu + ((u >> 16) & 1u);                                     // round half to even
-  return (uint16_t)(u >> 16);
-}
-
 uint64_t splitmix64(uint64_t &s) {
   uint64_t z = (s += 0x9E3779B97F4A7C15ull);
   z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
@@ -74,30 +68,38 @@ uint64_t splitmix64(uint64_t &s) {
 
 }  // namespace
 
+// What a call reads back when it ends: the tensor-core waits' flag and the sum
+// of the rows' losses.
+struct PassResult {
+  int err;
+  float loss;
+};
+
 struct qp_ws {
   int dev = 0;
   int step = 0;
-  Buf w[kLayers], b[kLayers];          // fp32 masters
-  Buf mw[kLayers], vw[kLayers], mb[kLayers], vb[kLayers];
-  Buf gw[kLayers], gb[kLayers];        // fp32 gradients
-  Buf wb[kLayers], wt[kLayers];        // bf16 weight and its transpose
+  Buf par, am, av, grad;               // fp32 masters, Adam's moments, gradients: flat (mlp::kParams)
+  Buf wb, wt;                          // bf16 weights and their transposes, at the weights' flat offsets
   int cap = 0;                         // rows the activation buffers hold
   int fwd_mode = QP_WS_FORWARD_FUSED;
-  Buf x0, h[3], z, dz, dh[3], t1, t2, lab, stp, loss, err;
+  Buf xf, x0, h[3], z, dz, dh[3], lab, stp, res;
+  Buf tr;              // transposes for the weight gradients: dY of the four layers, then X of them
   Buf gws, cws, lrow;  // split-K partials, column-sum partials, per-row losses (fixed-order sums)
+
+  float *weight(const Buf &b, int l) const { return b.as<float>() + mlp::weight_offset(l); }
+  float *bias(const Buf &b, int l) const { return b.as<float>() + mlp::bias_offset(l); }
+  __nv_bfloat16 *weight16(const Buf &b, int l) const { return b.as<__nv_bfloat16>() + mlp::weight_offset(l); }
+  PassResult *result() const { return res.as<PassResult>(); }
 };
 
 namespace {
 
-size_t n_params() {
-  size_t n = 0;
-  for (int l = 0; l < kLayers; ++l) n += (size_t)kDimOut[l] * kDimIn[l] + kDimOut[l];
-  return n;
-}
+static_assert(kIn == 16 && kHid == 256 && kOut == 256 && kLayers == 4, "the flat layout of mlp::kParams");
 
 qp_status ensure_rows(qp_ws *m, int Mp) {
   if (Mp <= m->cap) return QP_OK;
   m->cap = 0;  // a failed growth below leaves some buffers empty: check them all next time
+  WS_ALLOC(m->xf, (size_t)Mp * kIn * 4);
   WS_ALLOC(m->x0, (size_t)Mp * kIn * 2);
   for (int i = 0; i < 3; ++i) {
     WS_ALLOC(m->h[i], (size_t)Mp * kHid * 2);
@@ -105,53 +107,29 @@ qp_status ensure_rows(qp_ws *m, int Mp) {
   }
   WS_ALLOC(m->z, (size_t)Mp * kOut * 4);
   WS_ALLOC(m->dz, (size_t)Mp * kOut * 2);
-  WS_ALLOC(m->t1, (size_t)Mp * kHid * 2);
-  WS_ALLOC(m->t2, (size_t)Mp * kHid * 2);
+  WS_ALLOC(m->tr, (size_t)Mp * (kLayers * kHid + kIn + 3 * kHid) * 2);
   WS_ALLOC(m->lab, (size_t)Mp * 4);
   WS_ALLOC(m->stp, (size_t)Mp * 4);
   WS_ALLOC(m->lrow, (size_t)Mp * 4);
-  WS_ALLOC(m->cws, (size_t)mlp::kColsumSlabs * kOut * 4);
+  WS_ALLOC(m->cws, (size_t)kLayers * mlp::kColsumSlabs * kOut * 4);
   m->cap = Mp;
   return QP_OK;
 }
 
-// bf16 copies of every weight (and transposes) from the fp32 masters
-qp_status refresh_bf16(qp_ws *m, cudaStream_t st) {
-  for (int l = 0; l < kLayers; ++l) {
-    const int rows = kDimOut[l], cols = kDimIn[l];
-    std::vector<float> wh((size_t)rows * cols);
-    WS_CU(cudaMemcpyAsync(wh.data(), m->w[l].p, wh.size() * 4, cudaMemcpyDeviceToHost, st));
-    WS_CU(cudaStreamSynchronize(st));
-    std::vector<uint16_t> a(wh.size()), t(wh.size());
-    for (int r = 0; r < rows; ++r)
-      for (int c = 0; c < cols; ++c) {
-        const uint16_t v = f32_to_bf16_bits(wh[(size_t)r * cols + c]);
-        a[(size_t)r * cols + c] = v;
-        t[(size_t)c * rows + r] = v;
-      }
-    WS_CU(cudaMemcpyAsync(m->wb[l].p, a.data(), a.size() * 2, cudaMemcpyHostToDevice, st));
-    WS_CU(cudaMemcpyAsync(m->wt[l].p, t.data(), t.size() * 2, cudaMemcpyHostToDevice, st));
-  }
-  WS_CU(cudaStreamSynchronize(st));
-  return QP_OK;
-}
-
+// The pass's inputs to the device; the features become bf16 there (converting
+// them on the host took 60 us of a 16384-cell pass).  The copies may still be
+// reading the caller's buffers on return: every caller waits for the stream.
 qp_status upload_inputs(qp_ws *m, const float *feats, int M, int Mp, const int32_t *labels, const int32_t *steps,
                         cudaStream_t st) {
   if (qp_status s = ensure_rows(m, Mp); s != QP_OK) return s;
-  std::vector<uint16_t> xb((size_t)Mp * kIn, 0);
-  for (size_t e = 0; e < (size_t)M * kIn; ++e) xb[e] = f32_to_bf16_bits(feats[e]);
-  WS_CU(cudaMemcpyAsync(m->x0.p, xb.data(), xb.size() * 2, cudaMemcpyHostToDevice, st));
-  if (labels && steps) {
-    std::vector<int32_t> lb(Mp, -1), sp(Mp, 1);
-    std::memcpy(lb.data(), labels, (size_t)M * 4);
-    std::memcpy(sp.data(), steps, (size_t)M * 4);
-    WS_CU(cudaMemcpyAsync(m->lab.p, lb.data(), (size_t)Mp * 4, cudaMemcpyHostToDevice, st));
-    WS_CU(cudaMemcpyAsync(m->stp.p, sp.data(), (size_t)Mp * 4, cudaMemcpyHostToDevice, st));
-    WS_CU(cudaStreamSynchronize(st));
-  } else {
-    WS_CU(cudaStreamSynchronize(st));
+  WS_CU(cudaMemcpyAsync(m->xf.p, feats, (size_t)M * kIn * 4, cudaMemcpyHostToDevice, st));
+  const bool train = labels && steps;
+  if (train) {
+    WS_CU(cudaMemcpyAsync(m->lab.p, labels, (size_t)M * 4, cudaMemcpyHostToDevice, st));
+    WS_CU(cudaMemcpyAsync(m->stp.p, steps, (size_t)M * 4, cudaMemcpyHostToDevice, st));
   }
+  WS_CU(mlp::inputs(m->xf.as<float>(), M, Mp, m->x0.as<__nv_bfloat16>(), train ? m->lab.as<int32_t>() : nullptr,
+                    train ? m->stp.as<int32_t>() : nullptr, st));
   return QP_OK;
 }
 
@@ -162,30 +140,35 @@ mlp::GemmArgs gargs(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int
   return g;
 }
 
-// Logits into m->z; the hidden activations into m->h[] when keep_hidden (the
-// backward pass reads them) or when the layers run as separate launches.
-qp_status forward(qp_ws *m, int Mp, bool keep_hidden, cudaStream_t st) {
+// Logits into m->z (and their first rows into out, when given: device memory,
+// 16-byte aligned, fused mode); the hidden activations into m->h[] when
+// keep_hidden (the backward pass reads them) or when the layers run as separate
+// launches.
+qp_status forward(qp_ws *m, int Mp, bool keep_hidden, float *out, int rows, cudaStream_t st) {
+  int *err = &m->result()->err;
   if (m->fwd_mode == QP_WS_FORWARD_FUSED) {
     mlp::FwdArgs g{};
     g.x0 = m->x0.as<__nv_bfloat16>();
     const __nv_bfloat16 *w[kLayers];
     for (int l = 0; l < kLayers; ++l) {
-      g.bias[l] = m->b[l].as<float>();
-      w[l] = m->wb[l].as<__nv_bfloat16>();
+      g.bias[l] = m->bias(m->par, l);
+      w[l] = m->weight16(m->wb, l);
     }
     for (int l = 0; l < 3; ++l) g.h[l] = keep_hidden ? m->h[l].as<__nv_bfloat16>() : nullptr;
     g.z = m->z.as<float>();
+    g.z2 = out;
+    g.rows2 = rows;
     g.Mp = Mp;
-    g.err = m->err.as<int>();
+    g.err = err;
     WS_CU(mlp::forward(g, w, st));
     return QP_OK;
   }
   const __nv_bfloat16 *in = m->x0.as<__nv_bfloat16>();
   int ldin = kIn;
   for (int l = 0; l < kLayers; ++l) {
-    mlp::GemmArgs g = gargs(in, ldin, m->wb[l].as<__nv_bfloat16>(), kDimIn[l], Mp, kDimOut[l], kDimIn[l],
-                            l < 3 ? mlp::kEpiBiasRelu : mlp::kEpiBiasF32, m->err.as<int>());
-    g.bias = m->b[l].as<float>();
+    mlp::GemmArgs g = gargs(in, ldin, m->weight16(m->wb, l), kDimIn[l], Mp, kDimOut[l], kDimIn[l],
+                            l < 3 ? mlp::kEpiBiasRelu : mlp::kEpiBiasF32, err);
+    g.bias = m->bias(m->par, l);
     if (l < 3) {
       g.out_bf16 = m->h[l].as<__nv_bfloat16>();
       g.ldo = kHid;
@@ -193,58 +176,86 @@ qp_status forward(qp_ws *m, int Mp, bool keep_hidden, cudaStream_t st) {
       g.out_f32 = m->z.as<float>();
       g.ldo = kOut;
     }
-    WS_CU(mlp::gemm(g, 1, st));
+    WS_CU(mlp::gemm(&g, 1, 1, st));
     in = m->h[l < 3 ? l : 2].as<__nv_bfloat16>();
     ldin = kHid;
   }
   return QP_OK;
 }
 
-// Gradients of the mean cross-entropy into gw/gb (fp32); loss sum into m->loss.
+// Gradients of the mean cross-entropy into m->grad; the loss sum into m->res.
 // Every sum over rows is taken in a fixed order (split-K partials and slabs
 // added in index order, no atomics), so a training run repeats bit for bit.
+// The chain of the dX products runs in one launch, and everything else of the
+// four layers side by side in one launch of its kind.
 qp_status backward(qp_ws *m, int M, int Mp, cudaStream_t st) {
-  WS_CU(mlp::softmax_ce(m->z.as<float>(), kOut, m->lab.as<int32_t>(), m->stp.as<int32_t>(), Mp, 1.0f / (float)M,
-                        m->dz.as<__nv_bfloat16>(), kOut, m->lrow.as<float>(), m->loss.as<float>(), st));
-  const __nv_bfloat16 *dy = m->dz.as<__nv_bfloat16>();
-  const int splits = std::max(1, Mp / 512);
-  WS_ALLOC(m->gws, (size_t)mlp::gemm_splits(Mp, splits) * kHid * kHid * 4);
-  for (int l = kLayers - 1; l >= 0; --l) {
-    const int nout = kDimOut[l], nin = kDimIn[l];
-    const __nv_bfloat16 *x = l == 0 ? m->x0.as<__nv_bfloat16>() : m->h[l - 1].as<__nv_bfloat16>();
-    // dW[out][in] = sum_m dY[m][out] X[m][in]  (operands transposed so m is contiguous)
-    __nv_bfloat16 *dyt = m->t1.as<__nv_bfloat16>(), *xt = m->t2.as<__nv_bfloat16>();
-    WS_CU(mlp::transpose(dy, Mp, nout, nout, dyt, Mp, st));
-    WS_CU(mlp::transpose(x, Mp, nin, nin, xt, Mp, st));
-    mlp::GemmArgs g = gargs(dyt, Mp, xt, Mp, nout, nin, Mp, mlp::kEpiPartialF32, m->err.as<int>());
-    g.out_f32 = m->gws.as<float>();
-    g.ldo = nin;
-    WS_CU(mlp::gemm(g, splits, st));
-    WS_CU(mlp::sum_splits(m->gws.as<float>(), mlp::gemm_splits(Mp, splits), nout * nin, m->gw[l].as<float>(), st));
-    WS_CU(mlp::colsum(dy, nout, Mp, nout, m->cws.as<float>(), m->gb[l].as<float>(), st));
-    if (l == 0) break;
-    // dX[m][in] = relu'(X) * sum_out dY[m][out] W[out][in]  (B = W^T, out contiguous)
-    mlp::GemmArgs gx = gargs(dy, nout, m->wt[l].as<__nv_bfloat16>(), nout, Mp, nin, nout, mlp::kEpiReluMask,
-                             m->err.as<int>());
-    gx.out_bf16 = m->dh[l - 1].as<__nv_bfloat16>();
-    gx.ldo = nin;
-    gx.relu_ref = x;
-    gx.ldr = nin;
-    WS_CU(mlp::gemm(gx, 1, st));
-    dy = m->dh[l - 1].as<__nv_bfloat16>();
+  int *err = &m->result()->err;
+  mlp::BwdArgs bw{};
+  bw.z = m->z.as<float>();
+  bw.label = m->lab.as<int32_t>();
+  bw.steps = m->stp.as<int32_t>();
+  bw.inv_rows = 1.0f / (float)M;
+  bw.dz = m->dz.as<__nv_bfloat16>();
+  bw.loss_rows = m->lrow.as<float>();
+  bw.Mp = Mp;
+  bw.err = err;
+  const __nv_bfloat16 *wt[kLayers];
+  for (int l = 0; l < kLayers; ++l) wt[l] = m->weight16(m->wt, l);
+  for (int l = 0; l < 3; ++l) {
+    bw.h[l] = m->h[l].as<__nv_bfloat16>();
+    bw.dh[l] = m->dh[l].as<__nv_bfloat16>();
+  }
+  WS_CU(mlp::backward(bw, wt, st));
+  const int splits = std::max(1, Mp / 512), zs = mlp::gemm_splits(Mp, splits);
+  WS_ALLOC(m->gws, (size_t)zs * mlp::kParams * 4);
+  const __nv_bfloat16 *dy[kLayers], *x[kLayers];
+  for (int l = 0; l < kLayers; ++l) {
+    dy[l] = l == kLayers - 1 ? m->dz.as<__nv_bfloat16>() : m->dh[l].as<__nv_bfloat16>();
+    x[l] = l == 0 ? m->x0.as<__nv_bfloat16>() : m->h[l - 1].as<__nv_bfloat16>();
+  }
+  // dW[out][in] = sum_m dY[m][out] X[m][in]  (operands transposed so m is contiguous)
+  __nv_bfloat16 *tr = m->tr.as<__nv_bfloat16>();
+  mlp::TransposeJob tj[2 * kLayers];
+  mlp::GemmArgs g[kLayers];
+  mlp::SumJob sums[2 * kLayers];
+  float *ws = m->gws.as<float>();
+  for (int l = 0; l < kLayers; ++l) {
+    __nv_bfloat16 *dyt = tr, *xt = tr + (size_t)Mp * kDimOut[l];
+    tr = xt + (size_t)Mp * kDimIn[l];
+    tj[2 * l] = {dy[l], dyt, kDimOut[l]};
+    tj[2 * l + 1] = {x[l], xt, kDimIn[l]};
+    g[l] = gargs(dyt, Mp, xt, Mp, kDimOut[l], kDimIn[l], Mp, mlp::kEpiPartialF32, err);
+    g[l].out_f32 = ws;
+    g[l].ldo = kDimIn[l];
+    const int n = kDimOut[l] * kDimIn[l];
+    sums[2 * l] = {ws, zs, n, m->weight(m->grad, l)};
+    sums[2 * l + 1] = {m->cws.as<float>() + (size_t)l * mlp::kColsumSlabs * kOut, mlp::kColsumSlabs, kOut,
+                       m->bias(m->grad, l)};
+    ws += (size_t)zs * n;
+  }
+  WS_CU(mlp::transpose(tj, 2 * kLayers, Mp, st));
+  WS_CU(mlp::gemm(g, kLayers, splits, st));
+  WS_CU(mlp::colsum(dy, kLayers, Mp, m->cws.as<float>(), st));
+  WS_CU(mlp::sum_jobs(sums, 2 * kLayers, m->lrow.as<float>(), Mp, &m->result()->loss, st));
+  return QP_OK;
+}
+
+// Wait for the pass and read its result (and, into grads_out when given, the gradients).
+qp_status finish(qp_ws *m, float *grads_out, PassResult *out, cudaStream_t st) {
+  if (grads_out) WS_CU(cudaMemcpyAsync(grads_out, m->grad.p, (size_t)mlp::kParams * 4, cudaMemcpyDeviceToHost, st));
+  WS_CU(cudaMemcpyAsync(out, m->res.p, sizeof *out, cudaMemcpyDeviceToHost, st));
+  WS_CU(cudaStreamSynchronize(st));
+  if (out->err) {
+    WS_CU(cudaMemsetAsync(&m->result()->err, 0, 4, st));
+    return set_error(QP_ETIMEOUT, "warm start: a tensor-core wait gave up");
   }
   return QP_OK;
 }
 
-qp_status check_err(qp_ws *m, cudaStream_t st) {
-  int e = 0;
-  WS_CU(cudaMemcpyAsync(&e, m->err.p, 4, cudaMemcpyDeviceToHost, st));
-  WS_CU(cudaStreamSynchronize(st));
-  if (e) {
-    WS_CU(cudaMemsetAsync(m->err.p, 0, 4, st));
-    return set_error(QP_ETIMEOUT, "warm start: a tensor-core wait gave up");
-  }
-  return QP_OK;
+// A failed call leaves no copy reading the caller's buffers.
+qp_status settle(qp_status s, cudaStream_t st) {
+  if (s != QP_OK && cudaStreamSynchronize(st) != cudaSuccess) cudaGetLastError();
+  return s;
 }
 
 struct DevGuard {
@@ -266,48 +277,30 @@ struct DevGuard {
 extern "C" qp_status qp_ws_create(uint64_t seed, qp_ws **out) {
   if (!out) return set_error(QP_EINVAL, "out is NULL");
   *out = nullptr;
-  qp_ws *m = new qp_ws();
-  if (cudaGetDevice(&m->dev) != cudaSuccess) {
-    delete m;
-    return set_error(QP_ECUDA, "cudaGetDevice failed");
-  }
+  auto m = std::make_unique<qp_ws>();
+  if (cudaGetDevice(&m->dev) != cudaSuccess) return set_error(QP_ECUDA, "cudaGetDevice failed");
+  const size_t n = mlp::kParams;
+  if (!m->par.ensure(n * 4) || !m->am.ensure(n * 4) || !m->av.ensure(n * 4) || !m->grad.ensure(n * 4) ||
+      !m->wb.ensure(n * 2) || !m->wt.ensure(n * 2) || !m->res.ensure(sizeof(PassResult)))
+    return set_error(QP_ENOMEM, "warm start: cudaMalloc failed");
+  // He-uniform initialisation from a splitmix64 stream, zero biases
+  std::vector<float> p(n, 0.0f);
   uint64_t s = seed;
   for (int l = 0; l < kLayers; ++l) {
-    const int rows = kDimOut[l], cols = kDimIn[l];
-    const size_t nw = (size_t)rows * cols;
-    bool ok = m->w[l].ensure(nw * 4) && m->b[l].ensure(rows * 4) && m->mw[l].ensure(nw * 4) &&
-              m->vw[l].ensure(nw * 4) && m->mb[l].ensure(rows * 4) && m->vb[l].ensure(rows * 4) &&
-              m->gw[l].ensure(nw * 4) && m->gb[l].ensure(rows * 4) && m->wb[l].ensure(nw * 2) &&
-              m->wt[l].ensure(nw * 2);
-    if (!ok) {
-      delete m;
-      return set_error(QP_ENOMEM, "warm start: cudaMalloc failed");
-    }
-    // He-uniform initialisation from a splitmix64 stream
-    const double lim = std::sqrt(6.0 / cols);
-    std::vector<float> wh(nw);
-    for (size_t e = 0; e < nw; ++e) {
+    const double lim = std::sqrt(6.0 / kDimIn[l]);
+    float *w = p.data() + mlp::weight_offset(l);
+    for (int e = 0; e < kDimOut[l] * kDimIn[l]; ++e) {
       const double u = (double)(splitmix64(s) >> 11) * (1.0 / 9007199254740992.0);
-      wh[e] = (float)((2.0 * u - 1.0) * lim);
+      w[e] = (float)((2.0 * u - 1.0) * lim);
     }
-    cudaMemcpy(m->w[l].p, wh.data(), nw * 4, cudaMemcpyHostToDevice);
-    cudaMemset(m->b[l].p, 0, rows * 4);
-    cudaMemset(m->mw[l].p, 0, nw * 4);
-    cudaMemset(m->vw[l].p, 0, nw * 4);
-    cudaMemset(m->mb[l].p, 0, rows * 4);
-    cudaMemset(m->vb[l].p, 0, rows * 4);
   }
-  if (!m->loss.ensure(4) || !m->err.ensure(4)) {
-    delete m;
-    return set_error(QP_ENOMEM, "warm start: cudaMalloc failed");
-  }
-  cudaMemset(m->err.p, 0, 4);
-  const qp_status st = refresh_bf16(m, nullptr);
-  if (st != QP_OK) {
-    delete m;
-    return st;
-  }
-  *out = m;
+  WS_CU(cudaMemset(m->am.p, 0, n * 4));
+  WS_CU(cudaMemset(m->av.p, 0, n * 4));
+  WS_CU(cudaMemset(m->res.p, 0, sizeof(PassResult)));
+  WS_CU(cudaMemcpy(m->par.p, p.data(), n * 4, cudaMemcpyHostToDevice));
+  WS_CU(mlp::refresh(m->par.as<float>(), m->wb.as<__nv_bfloat16>(), m->wt.as<__nv_bfloat16>(), nullptr));
+  WS_CU(cudaStreamSynchronize(nullptr));
+  *out = m.release();
   return QP_OK;
 }
 
@@ -317,47 +310,42 @@ extern "C" void qp_ws_destroy(qp_ws *m) {
   delete m;
 }
 
-extern "C" int64_t qp_ws_param_count(void) { return (int64_t)n_params(); }
+extern "C" int64_t qp_ws_param_count(void) { return mlp::kParams; }
 
 extern "C" qp_status qp_ws_get_params(qp_ws *m, float *out) {
   if (!m || !out) return set_error(QP_EINVAL, "NULL argument");
   DevGuard g(m->dev);
-  size_t o = 0;
-  for (int l = 0; l < kLayers; ++l) {
-    const size_t nw = (size_t)kDimOut[l] * kDimIn[l];
-    WS_CU(cudaMemcpy(out + o, m->w[l].p, nw * 4, cudaMemcpyDeviceToHost));
-    o += nw;
-    WS_CU(cudaMemcpy(out + o, m->b[l].p, (size_t)kDimOut[l] * 4, cudaMemcpyDeviceToHost));
-    o += kDimOut[l];
-  }
+  WS_CU(cudaMemcpy(out, m->par.p, (size_t)mlp::kParams * 4, cudaMemcpyDeviceToHost));
   return QP_OK;
 }
 
 extern "C" qp_status qp_ws_set_params(qp_ws *m, const float *in) {
   if (!m || !in) return set_error(QP_EINVAL, "NULL argument");
   DevGuard g(m->dev);
-  size_t o = 0;
-  for (int l = 0; l < kLayers; ++l) {
-    const size_t nw = (size_t)kDimOut[l] * kDimIn[l];
-    WS_CU(cudaMemcpy(m->w[l].p, in + o, nw * 4, cudaMemcpyHostToDevice));
-    o += nw;
-    WS_CU(cudaMemcpy(m->b[l].p, in + o, (size_t)kDimOut[l] * 4, cudaMemcpyHostToDevice));
-    o += kDimOut[l];
-  }
-  return refresh_bf16(m, nullptr);
+  WS_CU(cudaMemcpy(m->par.p, in, (size_t)mlp::kParams * 4, cudaMemcpyHostToDevice));
+  WS_CU(mlp::refresh(m->par.as<float>(), m->wb.as<__nv_bfloat16>(), m->wt.as<__nv_bfloat16>(), nullptr));
+  WS_CU(cudaStreamSynchronize(nullptr));
+  return QP_OK;
 }
 
 extern "C" qp_status qp_ws_forward(qp_ws *m, const float *feats, int32_t M, float *logits_out, void *stream) {
   if (!m || !feats || !logits_out || M < 1) return set_error(QP_EINVAL, "bad argument");
-  if (device_pointer(logits_out) && !device_range_fits(logits_out, (size_t)M * kOut * 4))
+  const bool dev_out = device_pointer(logits_out);
+  if (dev_out && !device_range_fits(logits_out, (size_t)M * kOut * 4))
     return set_error(QP_EINVAL, "qp_ws_forward: the device buffer for the logits is too small");
   DevGuard g(m->dev);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int Mp = (M + 127) / 128 * 128;
-  if (qp_status s = upload_inputs(m, feats, M, Mp, nullptr, nullptr, st); s != QP_OK) return s;
-  if (qp_status s = forward(m, Mp, false, st); s != QP_OK) return s;
-  WS_CU(cudaMemcpyAsync(logits_out, m->z.p, (size_t)M * kOut * 4, cudaMemcpyDefault, st));
-  return check_err(m, st);
+  // the fused kernel writes the caller's logits beside its own when it can
+  const bool direct = dev_out && m->fwd_mode == QP_WS_FORWARD_FUSED && (reinterpret_cast<uintptr_t>(logits_out) & 15) == 0;
+  PassResult r{};
+  const auto pass = [&]() -> qp_status {
+    if (qp_status s = upload_inputs(m, feats, M, Mp, nullptr, nullptr, st); s != QP_OK) return s;
+    if (qp_status s = forward(m, Mp, false, direct ? logits_out : nullptr, M, st); s != QP_OK) return s;
+    if (!direct) WS_CU(cudaMemcpyAsync(logits_out, m->z.p, (size_t)M * kOut * 4, cudaMemcpyDefault, st));
+    return finish(m, nullptr, &r, st);
+  };
+  return settle(pass(), st);
 }
 
 extern "C" qp_status qp_ws_set_forward_mode(qp_ws *m, int32_t mode) {
@@ -373,43 +361,37 @@ extern "C" qp_status qp_ws_grads(qp_ws *m, const float *feats, const int32_t *la
   DevGuard g(m->dev);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int Mp = (M + 127) / 128 * 128;
-  if (qp_status s = upload_inputs(m, feats, M, Mp, labels, steps, st); s != QP_OK) return s;
-  if (qp_status s = forward(m, Mp, true, st); s != QP_OK) return s;
-  if (qp_status s = backward(m, M, Mp, st); s != QP_OK) return s;
-  if (qp_status s = check_err(m, st); s != QP_OK) return s;
-  if (grads_out) {
-    size_t o = 0;
-    for (int l = 0; l < kLayers; ++l) {
-      const size_t nw = (size_t)kDimOut[l] * kDimIn[l];
-      WS_CU(cudaMemcpy(grads_out + o, m->gw[l].p, nw * 4, cudaMemcpyDeviceToHost));
-      o += nw;
-      WS_CU(cudaMemcpy(grads_out + o, m->gb[l].p, (size_t)kDimOut[l] * 4, cudaMemcpyDeviceToHost));
-      o += kDimOut[l];
-    }
-  }
-  if (loss_out) {
-    float ls = 0.0f;
-    WS_CU(cudaMemcpy(&ls, m->loss.p, 4, cudaMemcpyDeviceToHost));
-    *loss_out = ls / (float)M;
-  }
+  PassResult r{};
+  const auto pass = [&]() -> qp_status {
+    if (qp_status s = upload_inputs(m, feats, M, Mp, labels, steps, st); s != QP_OK) return s;
+    if (qp_status s = forward(m, Mp, true, nullptr, 0, st); s != QP_OK) return s;
+    if (qp_status s = backward(m, M, Mp, st); s != QP_OK) return s;
+    return finish(m, grads_out, &r, st);
+  };
+  if (qp_status s = settle(pass(), st); s != QP_OK) return s;
+  if (loss_out) *loss_out = r.loss / (float)M;
   return QP_OK;
 }
 
 extern "C" qp_status qp_ws_train_step(qp_ws *m, const float *feats, const int32_t *labels, const int32_t *steps,
                                       int32_t M, float lr, float *loss_out, void *stream) {
-  const qp_status s0 = qp_ws_grads(m, feats, labels, steps, M, nullptr, loss_out, stream);
-  if (s0 != QP_OK) return s0;
+  if (!m || !feats || !labels || !steps || M < 1) return set_error(QP_EINVAL, "bad argument");
   DevGuard g(m->dev);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  const int Mp = (M + 127) / 128 * 128;
+  PassResult r{};
+  const auto pass = [&]() -> qp_status {
+    if (qp_status s = upload_inputs(m, feats, M, Mp, labels, steps, st); s != QP_OK) return s;
+    if (qp_status s = forward(m, Mp, true, nullptr, 0, st); s != QP_OK) return s;
+    if (qp_status s = backward(m, M, Mp, st); s != QP_OK) return s;
+    // the update reads the pass's error flag on the device and leaves a failed pass's parameters alone
+    WS_CU(mlp::adam(m->par.as<float>(), m->am.as<float>(), m->av.as<float>(), m->grad.as<float>(), lr, 0.9f, 0.999f,
+                    1e-8f, m->step + 1, m->wb.as<__nv_bfloat16>(), m->wt.as<__nv_bfloat16>(), &m->result()->err, st));
+    return finish(m, nullptr, &r, st);
+  };
+  if (qp_status s = settle(pass(), st); s != QP_OK) return s;
   m->step += 1;
-  for (int l = 0; l < kLayers; ++l) {
-    const int rows = kDimOut[l], cols = kDimIn[l];
-    WS_CU(mlp::adam(m->w[l].as<float>(), m->mw[l].as<float>(), m->vw[l].as<float>(), m->gw[l].as<float>(), rows,
-                    cols, lr, 0.9f, 0.999f, 1e-8f, m->step, m->wb[l].as<__nv_bfloat16>(),
-                    m->wt[l].as<__nv_bfloat16>(), st));
-    WS_CU(mlp::adam(m->b[l].as<float>(), m->mb[l].as<float>(), m->vb[l].as<float>(), m->gb[l].as<float>(), 1,
-                    rows, lr, 0.9f, 0.999f, 1e-8f, m->step, nullptr, nullptr, st));
-  }
+  if (loss_out) *loss_out = r.loss / (float)M;
   return QP_OK;
 }
 
@@ -419,38 +401,23 @@ extern "C" qp_status qp_ws_get_state(qp_ws *m, int32_t which, float *out) {
     return set_error(QP_EINVAL, "bad argument");
   DevGuard g(m->dev);
   WS_CU(cudaDeviceSynchronize());
-  size_t o = 0;
-  for (int l = 0; l < kLayers; ++l) {
-    const Buf &W = which == QP_WS_STATE_PARAMS ? m->w[l]
-                   : which == QP_WS_STATE_ADAM_M ? m->mw[l]
-                   : which == QP_WS_STATE_ADAM_V ? m->vw[l] : m->gw[l];
-    const Buf &B = which == QP_WS_STATE_PARAMS ? m->b[l]
-                   : which == QP_WS_STATE_ADAM_M ? m->mb[l]
-                   : which == QP_WS_STATE_ADAM_V ? m->vb[l] : m->gb[l];
-    const size_t nw = (size_t)kDimOut[l] * kDimIn[l];
-    WS_CU(cudaMemcpy(out + o, W.p, nw * 4, cudaMemcpyDeviceToHost));
-    o += nw;
-    WS_CU(cudaMemcpy(out + o, B.p, (size_t)kDimOut[l] * 4, cudaMemcpyDeviceToHost));
-    o += kDimOut[l];
-  }
+  const Buf &b = which == QP_WS_STATE_PARAMS ? m->par
+                 : which == QP_WS_STATE_ADAM_M ? m->am
+                 : which == QP_WS_STATE_ADAM_V ? m->av : m->grad;
+  WS_CU(cudaMemcpy(out, b.p, (size_t)mlp::kParams * 4, cudaMemcpyDeviceToHost));
   return QP_OK;
 }
 
 extern "C" qp_status qp_ws_get_buffer(qp_ws *m, int32_t which, int32_t rows, void *out) {
   if (!m || !out) return set_error(QP_EINVAL, "bad argument");
   DevGuard g(m->dev);
-  if (which >= QP_WS_BUF_W_BF16 && which < QP_WS_BUF_W_BF16 + kLayers) {
-    const int l = which - QP_WS_BUF_W_BF16;
-    WS_CU(cudaDeviceSynchronize());
-    WS_CU(cudaMemcpy(out, m->wb[l].p, (size_t)kDimOut[l] * kDimIn[l] * 2, cudaMemcpyDeviceToHost));
-    return QP_OK;
-  }
-  if (which >= QP_WS_BUF_WT_BF16 && which < QP_WS_BUF_WT_BF16 + kLayers) {
-    const int l = which - QP_WS_BUF_WT_BF16;
-    WS_CU(cudaDeviceSynchronize());
-    WS_CU(cudaMemcpy(out, m->wt[l].p, (size_t)kDimOut[l] * kDimIn[l] * 2, cudaMemcpyDeviceToHost));
-    return QP_OK;
-  }
+  for (const auto &w : {std::make_pair((int)QP_WS_BUF_W_BF16, &m->wb), std::make_pair((int)QP_WS_BUF_WT_BF16, &m->wt)})
+    if (which >= w.first && which < w.first + kLayers) {
+      const int l = which - w.first;
+      WS_CU(cudaDeviceSynchronize());
+      WS_CU(cudaMemcpy(out, m->weight16(*w.second, l), (size_t)kDimOut[l] * kDimIn[l] * 2, cudaMemcpyDeviceToHost));
+      return QP_OK;
+    }
   if (rows < 1 || rows > m->cap) return set_error(QP_EINVAL, "rows beyond the last pass's buffers");
   const Buf *b = nullptr;
   size_t row_bytes = (size_t)kHid * 2;
