@@ -338,154 +338,25 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
       }
     };
 
-    // Row t, exactly.  pre (PRE, rows of one block): the next row's draws are
-    // computed beside this row's evaluation, of which they are independent (u
-    // and top hold this row's on entry, the next one's on return).
-    uint32_t u[4];
-    int top[4];
-    auto event_row = [&](int t, auto pre) {
-      constexpr bool PRE = decltype(pre)::value;
-      const Row p0 = unpack_row(rec[t - 1]), p1 = unpack_row(rec[t]), p2 = unpack_row(rec[t + 1]);
-      const int tC = t * C;
-      int r = p1.n, l0 = p1.c0, l1 = p1.c1, l2 = p1.c2;
-      bool lost = p1.n > kRowCells, flipped = false;
-      const uint32_t m1 = (uint32_t)(tC + C - 1) >> 2;
-            for (uint32_t mb = (uint32_t)tC >> 2; mb <= m1; mb += 32) {
-        uint32_t un[4];
-        int topn[4];
-        if (PRE) draws(tC + C, ((uint32_t)(tC + C) >> 2) + lane, un, topn, pre);
-        else draws(tC, mb + lane, u, top, pre);
-        const int i0 = (int)(4 * (mb + lane)) - tC;  // the lane's columns i0 .. i0 + 3, -4 < i0
-        const int ic = min(i0, C);
-        int f[4] = {0, 0, 0, 0}, c[4];
-        uint32_t xi[4] = {0, 0, 0, 0};
-        if (DM == 2) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) xi[j] = D.xy[ic + j];
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) c[j] = cc[ic + j];
-        D.add4(p0.c0, ic, xi, f);
-        D.add4(p2.c0, ic, xi, f);
-        int xm = 0;  // x of the lane's columns
-#pragma unroll
-        for (int j = 0; j < 4; ++j) xm |= (int)(i0 + j == p1.c0) << j;
-        if (p0.n > 1 || p1.n > 1 || p2.n > 1) {  // rows of several cells
-          if (p1.n > kRowCells) {
-            xm = 0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              const int i = i0 + j;
-              if (i >= 0 && i < C)
-                xm |= (int)((bits_word<SB>(bits + QP_IX(t * Cw + (i >> 5), C * Cw, 3)) >> (i & 31)) & 1u) << j;
-            }
-          } else if (p1.n > 1) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j)
-              xm |= (int)(i0 + j == p1.c1 || (p1.n > 2 && i0 + j == p1.c2)) << j;
-          }
-#pragma unroll 1
-          for (int side = -1; side <= 1; side += 2) {
-            const Row &p = side < 0 ? p0 : p2;
-            if (p.n > kRowCells) {  // the cells from the row's bits, but the one already added
-              for (int w0 = 0; w0 < Cw; w0 += 32) {
-                uint32_t word = w0 + lane < Cw ? bits_word<SB>(bits + QP_IX((t + side) * Cw + w0 + lane, C * Cw, 3)) : 0u;
-                if ((p.c0 >> 5) == w0 + lane) word &= ~(1u << (p.c0 & 31));
-                for (uint32_t b = __ballot_sync(kFull, word != 0); b; b &= b - 1) {
-                  const int w = __ffs(b) - 1;
-                  for (uint32_t wd = __shfl_sync(kFull, word, w); wd; wd &= wd - 1)
-                    D.add4(((w0 + w) << 5) + __ffs(wd) - 1, ic, xi, f);
-                }
-              }
-            } else if (p.n > 1) {
-              D.add4(p.c1, ic, xi, f);
-              if (p.n > 2) D.add4(p.c2, ic, xi, f);
-            }
-          }
-        }
-        // dE of x = 0, and 4A less it for x = 1
-        int dE[4], step[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-          const int v = twoA * (c[j] + r - 1) + B * f[j];
-          const bool x = (xm >> j) & 1;
-          dE[j] = x ? 2 * twoA - v : v;
-          step[j] = x ? -twoA : twoA;
-        }
-        while (true) {
-          if (!__any_sync(kFull, dE[0] <= top[0] || dE[1] <= top[1] || dE[2] <= top[2] || dE[3] <= top[3])) break;
-          // the first proposal that may be accepted
-          const int jl = dE[0] <= top[0] ? 0 : (dE[1] <= top[1] ? 1 : (dE[2] <= top[2] ? 2 : 3));
-          const int dl = sel4(dE, jl), tl = sel4(top, jl);
-          const int L = __ffs(__ballot_sync(kFull, dl <= tl)) - 1;
-          int pk0 = jl | (sel4(step, jl) < 0) << 2 | sel4(c, jl) << 3;
-          if (lane == L && dl >= tl - band) {
-            const uint32_t uj = jl == 0 ? u[0] : (jl == 1 ? u[1] : (jl == 2 ? u[2] : u[3]));
-            if (!(dl <= 0 || (dl < len && uj < __ldg(thr + QP_IX(dl, len, 1))))) pk0 = -1;
-          }
-          const int de = __shfl_sync(kFull, dl, L);
-          const int pk = __shfl_sync(kFull, pk0, L);
-          if (pk < 0) {  // rejected by the table
-            if (lane == L) {
-#pragma unroll
-              for (int j = 0; j < 4; ++j)
-                if (j == jl) top[j] = INT_MIN;
-            }
-            continue;
-          }
-          const int cm = pk >> 3, dlt = 1 - 2 * ((pk >> 2) & 1);
-          const int im = (int)(4 * (mb + L)) - tC + (pk & 3);
-          E += de;
-          ++acc;
-          viol += (cm + dlt != 1) - (cm != 1);
-          nz += (cm + dlt == 0) - (cm == 0);
-          if (lane == 0) cc[im] = (uint16_t)(cm + dlt);
-          // every proposal up to it is decided; the row's sum moved for the rest
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            dE[j] += dlt * step[j];
-            if (i0 + j <= im) top[j] = INT_MIN;
-          }
-          if (lost || (dlt > 0 && r >= kRowCells)) {  // a row of more than three cells: its bits
-            if (!lost) {
-              for (int w = lane; w < Cw; w += 32)
-                bits[QP_IX(t * Cw + w, C * Cw, 3)] = ((l0 >> 5) == w ? 1u << (l0 & 31) : 0u) |
-                                                     ((l1 >> 5) == w ? 1u << (l1 & 31) : 0u) |
-                                                     ((l2 >> 5) == w ? 1u << (l2 & 31) : 0u);
-              lost = true;
-              __syncwarp();
-            }
-            if (lane == 0) {
-              uint32_t *wp = bits + QP_IX(t * Cw + (im >> 5), C * Cw, 3);
-              if (SB) *wp ^= 1u << (im & 31);
-              else atomicXor(wp, 1u << (im & 31));
-            }
-          } else if (dlt > 0) {
-            l2 = l1;
-            l1 = l0;
-            l0 = im;
-          } else {
-            const bool first = l0 == im, second = l1 == im;
-            l0 = first ? l1 : l0;
-            l1 = first || second ? l2 : l1;
-          }
-          r += dlt;
-          flipped = true;
-        }
-        if (PRE) {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            u[j] = un[j];
-            top[j] = topn[j];
-          }
-        }
-      }
-      if (flipped) {
+    // The row in hand: its number of cells r, the cells (l0, l1, l2) unless lost (see Row).
+    int r = 0, l0 = 0, l1 = 0, l2 = 0, flips = 0, flips0 = 0;
+    bool lost = false;
+    auto start_row = [&](const Row &p) {
+      r = p.n;
+      l0 = p.c0;
+      l1 = p.c1;
+      l2 = p.c2;
+      lost = p.n > kRowCells;
+      flips0 = flips;
+    };
+    // Row t is done (n cells before): its record, stored when it changed.
+    auto finish_row = [&](int t, int n) -> uint2 {
+      uint2 q = pack_row(r, r > 0 ? l0 : C, l1, l2);
+      if (flips != flips0) {
         ++rows_flipped;
         zok = false;
-        viol += (r != 1) - (p1.n != 1);
+        viol += (r != 1) - (n != 1);
         __syncwarp();
-        uint2 q = pack_row(r, r > 0 ? l0 : C, l1, l2);
         if (lost) q = record_from_bits<SB>(bits, Cw, C, t, r, lane);
         if (lane == 0) {
           rec[t] = q;
@@ -493,6 +364,148 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
         }
         __syncwarp();
       }
+      return q;
+    };
+
+    // dE of the lane's four columns i0 .. i0 + 3 (-4 < i0) of row t, whose
+    // records are p1 and, around it, p0 and p2, at the row's sum r; how it moves
+    // when the row gains a cell (step), and the columns' place, x and sums
+    // (code: j | x << 2 | c << 3).
+    auto evaluate = [&](int t, const Row &p0, const Row &p1, const Row &p2, int i0, int (&dE)[4], int (&step)[4],
+                        int (&code)[4]) {
+      const int ic = min(i0, C);
+      int f[4] = {0, 0, 0, 0}, c[4];
+      uint32_t xi[4] = {0, 0, 0, 0};
+      if (DM == 2) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) xi[j] = D.xy[ic + j];
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) c[j] = cc[ic + j];
+      D.add4(p0.c0, ic, xi, f);
+      D.add4(p2.c0, ic, xi, f);
+      bool x[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] = i0 + j == p1.c0;
+      if (p0.n > 1 || p1.n > 1 || p2.n > 1) {  // rows of several cells
+        if (p1.n > kRowCells) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int i = i0 + j;
+            x[j] = i >= 0 && i < C && ((bits_word<SB>(bits + QP_IX(t * Cw + (i >> 5), C * Cw, 3)) >> (i & 31)) & 1u);
+          }
+        } else if (p1.n > 1) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) x[j] = x[j] || i0 + j == p1.c1 || (p1.n > 2 && i0 + j == p1.c2);
+        }
+#pragma unroll 1
+        for (int side = -1; side <= 1; side += 2) {
+          const Row &p = side < 0 ? p0 : p2;
+          if (p.n > kRowCells) {  // the cells from the row's bits, but the one already added
+            for (int w0 = 0; w0 < Cw; w0 += 32) {
+              uint32_t word = w0 + lane < Cw ? bits_word<SB>(bits + QP_IX((t + side) * Cw + w0 + lane, C * Cw, 3)) : 0u;
+              if ((p.c0 >> 5) == w0 + lane) word &= ~(1u << (p.c0 & 31));
+              for (uint32_t b = __ballot_sync(kFull, word != 0); b; b &= b - 1) {
+                const int w = __ffs(b) - 1;
+                for (uint32_t wd = __shfl_sync(kFull, word, w); wd; wd &= wd - 1)
+                  D.add4(((w0 + w) << 5) + __ffs(wd) - 1, ic, xi, f);
+              }
+            }
+          } else if (p.n > 1) {
+            D.add4(p.c1, ic, xi, f);
+            if (p.n > 2) D.add4(p.c2, ic, xi, f);
+          }
+        }
+      }
+      // dE of x = 0, and 4A less it for x = 1
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const int v = twoA * (c[j] + r - 1) + B * f[j];
+        dE[j] = x[j] ? 2 * twoA - v : v;
+        step[j] = x[j] ? -twoA : twoA;
+        code[j] = c[j] << 3 | (x[j] ? 4 + j : j);
+      }
+    };
+
+    // The row's proposals of one block, in order: the first that may be accepted
+    // is settled, applied to the row and to the state, and the rest looked at again.
+    auto resolve = [&](int t, int i0, int (&dE)[4], const int (&step)[4], int (&top)[4], const int (&code)[4],
+                       const uint32_t (&u)[4]) {
+      while (true) {
+        const bool ok0 = dE[0] <= top[0], ok1 = dE[1] <= top[1], ok2 = dE[2] <= top[2], ok3 = dE[3] <= top[3];
+        const uint32_t bal = __ballot_sync(kFull, ok0 || ok1 || ok2 || ok3);
+        if (bal == 0) break;
+        const int L = __ffs(bal) - 1;
+        const int dl = ok0 ? dE[0] : (ok1 ? dE[1] : (ok2 ? dE[2] : dE[3]));
+        const int tl = ok0 ? top[0] : (ok1 ? top[1] : (ok2 ? top[2] : top[3]));
+        const int cl = ok0 ? code[0] : (ok1 ? code[1] : (ok2 ? code[2] : code[3]));
+        const int de = __shfl_sync(kFull, dl, L);
+        const int pk = __shfl_sync(kFull, cl | (tl - dl <= band ? 1 << 20 : 0), L);
+        const int jm = pk & 3;
+        const int im = __shfl_sync(kFull, i0, L) + jm;
+        if (pk >> 20) {  // within the estimate's band: the table decides
+          const uint32_t ul = jm == 0 ? u[0] : (jm == 1 ? u[1] : (jm == 2 ? u[2] : u[3]));
+          const uint32_t um = __shfl_sync(kFull, ul, L);
+          if (!(de <= 0 || (de < len && um < __ldg(thr + QP_IX(de, len, 1))))) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (lane == L && j == jm) top[j] = INT_MIN;
+            continue;
+          }
+        }
+        const int cm = (pk >> 3) & 0x1FFFF, dlt = pk & 4 ? -1 : 1;
+        E += de;
+        ++flips;
+        viol += (cm + dlt != 1) - (cm != 1);
+        nz += (cm + dlt == 0) - (cm == 0);
+        if (lane == 0) cc[im] = (uint16_t)(cm + dlt);
+        // every proposal up to it is decided; the row's sum moved for the rest
+        const int rel = im - i0;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          dE[j] += dlt * step[j];
+          if (rel >= j) top[j] = INT_MIN;
+        }
+        if (lost || (dlt > 0 && r >= kRowCells)) {  // a row of more than three cells: its bits
+          if (!lost) {
+            for (int w = lane; w < Cw; w += 32)
+              bits[QP_IX(t * Cw + w, C * Cw, 3)] = ((l0 >> 5) == w ? 1u << (l0 & 31) : 0u) |
+                                                   ((l1 >> 5) == w ? 1u << (l1 & 31) : 0u) |
+                                                   ((l2 >> 5) == w ? 1u << (l2 & 31) : 0u);
+            lost = true;
+            __syncwarp();
+          }
+          if (lane == 0) {
+            uint32_t *wp = bits + QP_IX(t * Cw + (im >> 5), C * Cw, 3);
+            if (SB) *wp ^= 1u << (im & 31);
+            else atomicXor(wp, 1u << (im & 31));
+          }
+        } else {
+          const bool add = dlt > 0, first = l0 == im, second = l1 == im;
+          const int n0 = add ? im : (first ? l1 : l0), n1 = add ? l0 : (first || second ? l2 : l1);
+          l2 = add ? l1 : l2;
+          l1 = n1;
+          l0 = n0;
+        }
+        r += dlt;
+      }
+    };
+
+    // Row t, exactly.
+    auto event_row = [&](int t) {
+      const Row p0 = unpack_row(rec[t - 1]), p1 = unpack_row(rec[t]), p2 = unpack_row(rec[t + 1]);
+      const int tC = t * C;
+      start_row(p1);
+      const uint32_t m1 = (uint32_t)(tC + C - 1) >> 2;
+      for (uint32_t mb = (uint32_t)tC >> 2; mb <= m1; mb += 32) {
+        uint32_t u[4];
+        int top[4], dE[4], step[4], code[4];
+        draws(tC, mb + lane, u, top, std::false_type());
+        const int i0 = (int)(4 * (mb + lane)) - tC;
+        evaluate(t, p0, p1, p2, i0, dE, step, code);
+        resolve(t, i0, dE, step, top, code, u);
+      }
+      finish_row(t, p1.n);
     };
 
     // A cold sweep over a permutation (every row and column holds one cell):
@@ -516,8 +529,30 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
     if (quiet) {
     } else if (rowwise && C <= 125) {  // a row is one block of 128 columns, whatever t C mod 4
       hit = true;
+      // the next row's draws and record are fetched beside a row's evaluation, of which they are independent
+      uint32_t u[4];
+      int top[4];
       draws(C, ((uint32_t)C >> 2) + lane, u, top, std::true_type());
-      for (int t = 1; t < C; ++t) event_row(t, std::true_type());
+      Row p0 = unpack_row(rec[0]), p1 = unpack_row(rec[1]), p2 = unpack_row(rec[2]);
+      for (int t = 1; t < C; ++t) {
+        const int tC = t * C;
+        uint32_t un[4];
+        int topn[4], dE[4], step[4], code[4];
+        draws(tC + C, ((uint32_t)(tC + C) >> 2) + lane, un, topn, std::true_type());
+        const uint2 q3 = rec[min(t + 2, C)];
+        start_row(p1);
+        const int i0 = 4 * lane - (tC & 3);
+        evaluate(t, p0, p1, p2, i0, dE, step, code);
+        resolve(t, i0, dE, step, top, code, u);
+        p0 = unpack_row(finish_row(t, p1.n));
+        p1 = p2;
+        p2 = unpack_row(q3);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          u[j] = un[j];
+          top[j] = topn[j];
+        }
+      }
     } else {
       for (int t0 = 1; t0 < C; t0 += 32) {
         const int t1 = min(C, t0 + 32);
@@ -600,10 +635,11 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
             t = t0 + __ffs(bal) - 1;
           }
           hit = true;
-          event_row(t, std::false_type());
+          event_row(t);
         }
       }
     }
+    acc += flips;
     if (viol == 0 && E < best) best = E;
     settled = a.skip_settled && !hit;
     settled_len = len;
