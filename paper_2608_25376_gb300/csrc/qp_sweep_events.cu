@@ -25,20 +25,23 @@
 //           is found by one ballot; every row before it is final.
 //   event   the row evaluated exactly, 128 columns at a time (a lane takes the
 //           four columns of one Philox block), the first accepted proposal
-//           applied and the rest re-evaluated, in proposal order.
+//           applied and the rest re-evaluated, in proposal order.  Of a row of
+//           several blocks those that hold none of its cells, no empty column
+//           and no survivor are passed over (491 cells: 100.9 -> 91.4 ms).
 // After an event the check resumes at the next row.  A sweep most of whose
 // rows are events goes from row to row without draws and checks of its own.
 // Every decision is the sequential chain's: the same words of the generator
 // against the same tables.
 //
-// What bounds it: the latency of one chain (a check is ~150 dependent cycles,
-// an event ~1500), and in hot sweeps of large fields the Philox multiplies
-// (88 cycles of a scheduler per warp-wide block, whatever the occupancy).
-// Against the row kernels, which evaluate every column of every row (one GB300;
-// microseconds per sweep of all chains): 92 cells, 1024 chains: 161 -> 84 at
-// T = 1000 (1.2 flips a row), 72 -> 20 at T = 436, 20.9 -> 0.5 below T = 115;
-// 491 cells, 4096 chains x 1000 sweeps: 899 -> 101 ms; 893 cells, 512 chains x
-// 40 sweeps (the general kernel): 272 -> 25.9 ms.  It is also the faster one far
+// What bounds it: the latency of one chain, that is its count of dependent
+// instructions (92 cells, T = 1000: 367 warp instructions a row at 3.2 cycles
+// each with one warp on the SM, memory idle), and in hot sweeps of large fields
+// the Philox multiplies (88 cycles of a scheduler per warp-wide block, whatever
+// the occupancy; 42 of the 90.6 ms below).  Against the row kernels, which
+// evaluate every column of every row (one GB300): 92 cells, 1024 chains x 5000
+// sweeps: 166 -> 32.8 ms (161 -> 64 us a sweep at T = 1000, 1.2 flips a row);
+// 491 cells, 4096 chains x 1000 sweeps: 899 -> 90.6 ms; 893 cells, 512 chains x
+// 40 sweeps (the general kernel): 272 -> 22.0 ms.  It is also the faster one far
 // above the temperatures of a useful schedule (T = 1e6, a third of the cells
 // set: 1.5 to 2.2 times), so every structured launch uses it.
 #include <algorithm>
@@ -59,6 +62,13 @@ __device__ __forceinline__ int sel4(const int (&v)[4], int j) {
 
 constexpr int kZCheck = 4;    // most empty columns the check looks at; above, rows are processed one by one
 constexpr int kRowCells = 3;  // cells of a row kept in its record
+// What rows a kernel is compiled for: of one block of columns (C <= kNarrow), of
+// several, or both.  A single field's launch knows, and each kernel holds only its
+// own row loops (92 cells, 5000 sweeps: 33.3 -> 32.8 ms; instruction fetch is a
+// fifteenth of a chain's time).  The batch, whose SMs run fields of both kinds at
+// once, takes one body for both: with two bodies 13.5 -> 21.8 ms (256 fields).
+enum { kOneBlock, kWide, kAny };
+constexpr int kNarrow = 125;  // most cells of a row that is one block of 128 columns, whatever t C mod 4
 constexpr int kPad = 8;       // entries before and after the arrays read by four columns at a time
 
 __host__ __device__ constexpr size_t align16e(size_t x) { return (x + 15) & ~size_t(15); }
@@ -175,7 +185,7 @@ __device__ __forceinline__ uint2 record_from_bits(const uint32_t *bits, int Cw, 
 // The sweeps of one replica.  rec: C + 1 row records (the last stays empty),
 // hx: what D.near needs of the cell of a row that holds one, cc:
 // column sums with kPad entries on both sides, bits: C x Cw words.
-template <typename DT, int DM, bool SB, typename KEY>
+template <typename DT, int DM, bool SB, int ROWS, typename KEY>
 __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uint2 *rec, uint16_t *hx, uint16_t *cc,
                                                uint32_t *bits, const Dist<DT, DM> &D, int lane, const KEY &key) {
   const int C = a.C, s0 = a.start, B = a.B, twoA = 2 * a.A;
@@ -354,7 +364,7 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
       uint2 q = pack_row(r, r > 0 ? l0 : C, l1, l2);
       if (flips != flips0) {
         ++rows_flipped;
-        zok = false;
+        if (ROWS != kWide) zok = false;
         viol += (r != 1) - (n != 1);
         __syncwarp();
         if (lost) q = record_from_bits<SB>(bits, Cw, C, t, r, lane);
@@ -459,6 +469,15 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
         viol += (cm + dlt != 1) - (cm != 1);
         nz += (cm + dlt == 0) - (cm == 0);
         if (lane == 0) cc[im] = (uint16_t)(cm + dlt);
+        if (ROWS == kWide && zok) {  // the list of empty columns follows (491 cells: 91.7 -> 90.6 ms)
+          if (cm + dlt == 0) {
+            if (lane == nz - 1) zreg = im;
+            zok = nz <= kZCheck;
+          } else if (cm == 0) {  // the last entry takes the filled column's place
+            const int last = __shfl_sync(kFull, zreg, nz);
+            if (lane < nz && zreg == im) zreg = last;
+          }
+        }
         // every proposal up to it is decided; the row's sum moved for the rest
         const int rel = im - i0;
 #pragma unroll
@@ -491,8 +510,11 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
       }
     };
 
-    // Row t, exactly.
-    auto event_row = [&](int t) {
+    // Row t, exactly.  Blocks of 128 columns in which nothing can be accepted are
+    // passed over: with r >= 1 a block needs one of the row's own cells, or (r = 1)
+    // an empty column, or a survivor; everything else costs dE >= 2A.  sv: whether
+    // the row may hold survivors; a block whose draws all bound dE below 2A has none.
+    auto event_row = [&](int t, bool sv) {
       const Row p0 = unpack_row(rec[t - 1]), p1 = unpack_row(rec[t]), p2 = unpack_row(rec[t + 1]);
       const int tC = t * C;
       start_row(p1);
@@ -500,10 +522,27 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
       for (uint32_t mb = (uint32_t)tC >> 2; mb <= m1; mb += 32) {
         uint32_t u[4];
         int top[4], dE[4], step[4], code[4];
-        draws(tC, mb + lane, u, top, std::false_type());
         const int i0 = (int)(4 * (mb + lane)) - tC;
+        bool live = true;
+        if (ROWS == kWide && r >= 1 && !lost) {
+          const int ib = (int)(4 * mb) - tC;
+          live = (unsigned)(l0 - ib) < 128u || (r > 1 && (unsigned)(l1 - ib) < 128u) || (r > 2 && (unsigned)(l2 - ib) < 128u);
+          if (!live && r == 1 && nz > 0) {
+            bool z = false;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const int i = min(max(i0 + j, 0), C - 1);
+              z = z || cc[i] == 0;
+            }
+            live = __any_sync(kFull, z);
+          }
+          if (!live && !sv) continue;
+        }
+        draws(tC, mb + lane, u, top, std::bool_constant<ROWS == kOneBlock>());
+        if (ROWS == kWide && !live && !__any_sync(kFull, max(max(top[0], top[1]), max(top[2], top[3])) >= twoA)) continue;
         evaluate(t, p0, p1, p2, i0, dE, step, code);
         resolve(t, i0, dE, step, top, code, u);
+        if (ROWS == kOneBlock) break;
       }
       finish_row(t, p1.n);
     };
@@ -527,7 +566,7 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
     const bool rowwise = (float)rows_flipped + 0.5f * lambda * (float)C > 0.5f * (float)C;
     rows_flipped = 0;
     if (quiet) {
-    } else if (rowwise && C <= 125) {  // a row is one block of 128 columns, whatever t C mod 4
+    } else if (ROWS != kWide && rowwise && C <= kNarrow) {  // a row is one block of 128 columns, whatever t C mod 4
       hit = true;
       // the next row's draws and record are fetched beside a row's evaluation, of which they are independent
       uint32_t u[4];
@@ -635,7 +674,7 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
             t = t0 + __ffs(bal) - 1;
           }
           hit = true;
-          event_row(t);
+          event_row(t, hot && (rowwise || ((smask >> (t - t0)) & 1u)));
         }
       }
     }
@@ -730,7 +769,7 @@ __device__ __forceinline__ WarpArea warp_area(unsigned char *p, int C) {
   return w;
 }
 
-template <typename DT, int DM, bool SB>
+template <typename DT, int DM, bool SB, int ROWS>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * 32) k_sweep_events(const StructArgs a, const RoundKeys rk) {
   extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = blockDim.x >> 5;
@@ -740,7 +779,8 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * 32) k_sweep_events(const Str
   if (rep >= a.R) return;  // no CTA-wide barrier after this point
   const WarpArea w = warp_area(smem + events_dist_bytes(a.C, a.Cp, sizeof(DT), DM, a.tab_n) +
                                    warp * events_warp_bytes(a.C, SB), a.C);
-  events_replica<DT, DM, SB>(a, rep, w.rec, w.hx, w.cc, SB ? w.bits : a.gstate + (size_t)rep * a.nw_pad, D, lane, rk);
+  events_replica<DT, DM, SB, ROWS>(a, rep, w.rec, w.hx, w.cc, SB ? w.bits : a.gstate + (size_t)rep * a.nw_pad, D, lane,
+                                   rk);
 }
 
 // Many fields in one persistent launch: a warp takes (field, replica) units
@@ -748,9 +788,9 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * 32) k_sweep_events(const Str
 // L1 (consecutive units are replicas of the same field).  No warp waits on
 // another.  per: shared memory of a warp, sized for the largest field;
 // gbits: one replica's bitsets per warp of the grid (without SB).  256 fields
-// of 10-169 cells x 128 replicas x 2000 sweeps: 198 ms (the row kernel's batch:
-// 1190), 182 with the matrix staged in shared memory by 8 warps (1054).  At 128
-// registers and 16 warps per SM: 96 registers (20 warps) 273, 168 (12 warps) 216.
+// of 10-169 cells x 128 replicas x 2000 sweeps: 189 ms (the row kernel's batch:
+// 1190), 173 with the matrix staged in shared memory by 8 warps (1054).  At 128
+// registers and 16 warps per SM (198 at the time: 96 registers, 20 warps 273; 168, 12 warps 216).
 template <bool SB>
 __global__ void __launch_bounds__(kMaxWarpsPerCta * 32)
     k_events_batch(const StructArgs *fields, const int2 *units, int n_units, int *counter, size_t per, uint32_t *gbits,
@@ -766,9 +806,8 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * 32)
     const StructArgs &a = fields[unit.x];
     const Dist<int16_t, 0> D{static_cast<const int16_t *>(a.d), a.Cp, a.C, nullptr, 0, 0};
     const WarpArea w = warp_area(smem + warp * per, a.C);
-    events_replica<int16_t, 0, SB>(a, unit.y, w.rec, w.hx, w.cc,
-                                   SB ? w.bits : gbits + (size_t)(blockIdx.x * W + warp) * gwords, D, lane,
-                                   PhiloxKey{a.key0, a.key1});
+    uint32_t *bits = SB ? w.bits : gbits + (size_t)(blockIdx.x * W + warp) * gwords;
+    events_replica<int16_t, 0, SB, kAny>(a, unit.y, w.rec, w.hx, w.cc, bits, D, lane, PhiloxKey{a.key0, a.key1});
     __syncwarp();
   }
 }
@@ -794,9 +833,8 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * 32)
     const int rep = unit.y + warp;
     if (rep < a.R) {
       const WarpArea w = warp_area(smem + dist + warp * per, a.C);
-      events_replica<int16_t, 1, SB>(a, rep, w.rec, w.hx, w.cc,
-                                     SB ? w.bits : gbits + (size_t)(blockIdx.x * W + warp) * gwords, D, lane,
-                                     PhiloxKey{a.key0, a.key1});
+      uint32_t *bits = SB ? w.bits : gbits + (size_t)(blockIdx.x * W + warp) * gwords;
+      events_replica<int16_t, 1, SB, kAny>(a, rep, w.rec, w.hx, w.cc, bits, D, lane, PhiloxKey{a.key0, a.key1});
     }
     __syncthreads();  // every warp is done with the matrix and s_unit before the next unit
   }
@@ -805,6 +843,8 @@ __global__ void __launch_bounds__(kMaxWarpsPerCta * 32)
 constexpr size_t kSmemLimitEvents = 227 * 1024;
 constexpr size_t kBitsSmem = 8 * 1024;       // most bytes of a replica's bitsets kept in shared memory
 constexpr size_t kMatrixSmem = 40 * 1024;    // largest distance matrix staged in shared memory
+static_assert(4 * kNarrow * ((kNarrow + 31) / 32) <= kBitsSmem, "narrow rows keep their bitsets in shared memory");
+static_assert(2 * 181 * 181 > kMatrixSmem && 4 * 181 * ((181 + 31) / 32) <= kBitsSmem, "a staged matrix implies the same");
 
 struct EventsShape {
   int dm;
@@ -823,9 +863,9 @@ EventsShape events_shape(const StructArgs &a, bool d_i16) {
   return s;
 }
 
-template <typename DT, int DM, bool SB>
+template <typename DT, int DM, bool SB, int ROWS>
 cudaError_t launch_e(const StructArgs &a, const RoundKeys &rk, int W, size_t smem, cudaStream_t st) {
-  auto k = k_sweep_events<DT, DM, SB>;
+  auto k = k_sweep_events<DT, DM, SB, ROWS>;
   std::lock_guard<std::mutex> lk(launch_mutex());
   cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -836,9 +876,14 @@ cudaError_t launch_e(const StructArgs &a, const RoundKeys &rk, int W, size_t sme
 template <typename DT>
 cudaError_t launch_e2(const StructArgs &a, const RoundKeys &rk, const EventsShape &s, int W, size_t smem,
                       cudaStream_t st) {
-  if (s.dm == 1) return s.sb ? launch_e<DT, 1, true>(a, rk, W, smem, st) : launch_e<DT, 1, false>(a, rk, W, smem, st);
-  if (s.dm == 2) return s.sb ? launch_e<DT, 2, true>(a, rk, W, smem, st) : launch_e<DT, 2, false>(a, rk, W, smem, st);
-  return s.sb ? launch_e<DT, 0, true>(a, rk, W, smem, st) : launch_e<DT, 0, false>(a, rk, W, smem, st);
+  if (a.C <= kNarrow)  // the bitsets are in shared memory
+    return s.dm == 1   ? launch_e<DT, 1, true, kOneBlock>(a, rk, W, smem, st)
+           : s.dm == 2 ? launch_e<DT, 2, true, kOneBlock>(a, rk, W, smem, st)
+                       : launch_e<DT, 0, true, kOneBlock>(a, rk, W, smem, st);
+  if (s.dm == 1) return launch_e<DT, 1, true, kWide>(a, rk, W, smem, st);  // so here, too
+  if (s.dm == 2)
+    return s.sb ? launch_e<DT, 2, true, kWide>(a, rk, W, smem, st) : launch_e<DT, 2, false, kWide>(a, rk, W, smem, st);
+  return s.sb ? launch_e<DT, 0, true, kWide>(a, rk, W, smem, st) : launch_e<DT, 0, false, kWide>(a, rk, W, smem, st);
 }
 
 }  // namespace

@@ -98,3 +98,19 @@ def test_replica_offset(dev, orc):
     whole = run(h, 12, sc, 3)
     part = run(h, 5, sc, 3, offset=7)
     assert all(np.array_equal(w[7:], p) for w, p in zip(whole, part))
+
+
+# Rows of one block of columns end at 125 cells; above, blocks without a cell of
+# the row, an empty column or a survivor are passed over: rows of several cells
+# and many survivors, rows and columns that empty and fill, cells in every block.
+@pytest.mark.parametrize("cells,T0,density", [(125, 1500.0, 0.02), (126, 1500.0, 0.02), (127, 600.0, None),
+                                              (253, 2000.0, 0.008), (254, 900.0, None), (381, 2500.0, 0.005)])
+def test_blocks_of_columns(dev, orc, cells, T0, density):
+    f = strip(21, 21, cells)
+    R, S = 4, 14
+    P = orc.Problem(f.rows, f.cols, f.free_mask, f.start)
+    init = None if density is None else (np.random.default_rng(7).random((R, P.n)) < density).astype(np.uint8)
+    ref = orc.anneal_structured(P, R, S, T0=T0, T1=50.0, seed=13, init_states=init)
+    got = run(qpath.qp_build_qubo(f), R, qpath.schedule(S, T0, 50.0), 13, init)
+    for g, r in zip(got, (ref.states, ref.energies, ref.best, ref.accepts)):
+        assert np.array_equal(g, r)
