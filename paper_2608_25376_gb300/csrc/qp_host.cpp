@@ -319,14 +319,14 @@ static qp_status build_field_qubo(const qp_field *f, int32_t A, int32_t B, int32
   h->n = (int64_t)C * C;
   h->d.resize((size_t)C * C);
   int64_t maxd = 0, mind = INT32_MAX;
-  for (int i = 0; i < C; ++i)
-    for (int j = 0; j < C; ++j) {
+  for (int i = 0; i < C; ++i)  // d is symmetric, and zero on the diagonal
+    for (int j = 0; j < i; ++j) {
       const int64_t dr = cr[i] - cr[j], dc = cc[i] - cc[j];
       const int64_t v = round_scaled_sqrt(dr * dr + dc * dc, scale);
       if (v > INT32_MAX) return fail(QP_ERANGE, "distance beyond int32");
-      h->d[(size_t)i * C + j] = (int32_t)v;
+      h->d[(size_t)i * C + j] = h->d[(size_t)j * C + i] = (int32_t)v;
       maxd = std::max(maxd, v);
-      if (i != j) mind = std::min(mind, v);
+      mind = std::min(mind, v);
     }
   h->max_d = (int32_t)maxd;
   h->min_d = (int32_t)mind;
