@@ -1,5 +1,5 @@
-// Device helpers of the row-parallel structured sweep (qp_sweep_rows.cu:
-// the single-field and the batched persistent kernels): distance-row loads,
+// Device helpers of the row-parallel structured sweep (qp_sweep_rows.cu):
+// distance-row loads,
 // row fields, the single-cell cache and the evaluation of one row chunk.
 // Included inside namespace qp::{anon}.
 #pragma once

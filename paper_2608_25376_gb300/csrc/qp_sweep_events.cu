@@ -37,10 +37,10 @@
 // instructions (92 cells, T = 1000: 367 warp instructions a row at 3.2 cycles
 // each with one warp on the SM, memory idle), and in hot sweeps of large fields
 // the Philox multiplies (88 cycles of a scheduler per warp-wide block, whatever
-// the occupancy; 42 of the 90.6 ms below).  Against the row kernels, which
+// the occupancy; 42 of the 83.2 ms below).  Against the row kernels, which
 // evaluate every column of every row (one GB300): 92 cells, 1024 chains x 5000
 // sweeps: 166 -> 32.8 ms (161 -> 64 us a sweep at T = 1000, 1.2 flips a row);
-// 491 cells, 4096 chains x 1000 sweeps: 899 -> 90.6 ms; 893 cells, 512 chains x
+// 491 cells, 4096 chains x 1000 sweeps: 899 -> 83.2 ms; 893 cells, 512 chains x
 // 40 sweeps (the general kernel): 272 -> 22.0 ms.  It is also the faster one far
 // above the temperatures of a useful schedule (T = 1e6, a third of the cells
 // set: 1.5 to 2.2 times), so every structured launch uses it.
@@ -55,10 +55,6 @@ namespace qp {
 namespace {
 
 using namespace dev;
-
-__device__ __forceinline__ int sel4(const int (&v)[4], int j) {
-  return j == 0 ? v[0] : (j == 1 ? v[1] : (j == 2 ? v[2] : v[3]));
-}
 
 constexpr int kZCheck = 4;    // most empty columns the check looks at; above, rows are processed one by one
 constexpr int kRowCells = 3;  // cells of a row kept in its record
@@ -903,9 +899,16 @@ cudaError_t launch_events(const StructArgs &a_in, bool d_i16, int W, cudaStream_
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
-  // one chain per scheduler first: a chain's latency is its time, so few
-  // chains spread over the SMs, many share the staged distances
-  if (W <= 0) W = std::max(1, std::min(8, (a.R + sms - 1) / sms));
+  // One chain per scheduler first: a chain's latency is its time, so few chains
+  // spread over the SMs.  Above 8 per SM 8 share the staged distances, or 4
+  // where that leaves fewer chains on the fullest SM, whose time the launch takes
+  // (8 -> 4: 491 cells, 4096 chains, 32 -> 28 on it: 90.5 -> 82.7 ms; 1824 chains,
+  // 16 -> 12: 46.0 -> 39.0; 92 cells, 4096 chains: 79.2 -> 73.5; where both leave as
+  // many 8 stays: 236 cells, 2000 chains, 16 each: 38.5 against 39.8).
+  if (W <= 0) {
+    auto fullest = [&](int w) { return ((a.R + w - 1) / w + sms - 1) / sms * w; };
+    W = a.R <= 8 * sms ? std::max(1, (a.R + sms - 1) / sms) : (fullest(4) < fullest(8) ? 4 : 8);
+  }
   while (W > 1 && s.dist + W * s.per > kSmemLimitEvents) --W;
   const size_t smem = s.dist + W * s.per;
   if (smem > kSmemLimitEvents) return cudaErrorInvalidValue;

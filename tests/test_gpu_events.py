@@ -114,3 +114,14 @@ def test_blocks_of_columns(dev, orc, cells, T0, density):
     got = run(qpath.qp_build_qubo(f), R, qpath.schedule(S, T0, 50.0), 13, init)
     for g, r in zip(got, (ref.states, ref.energies, ref.best, ref.accepts)):
         assert np.array_equal(g, r)
+
+
+# More chains than 8 per SM: CTAs of 4 or of 8 chains, the last one in part.
+@pytest.mark.parametrize("R", [1217, 1300, 2000, 2433])
+def test_many_chains(dev, R):
+    h = qpath.qp_build_qubo(strip(5, 5, 22))
+    sc = qpath.schedule(6, 900.0, 200.0)
+    whole = run(h, R, sc, 3)
+    for a, b in ((0, 600), (600, R - 1), (R - 1, R)):
+        part = run(h, b - a, sc, 3, offset=a, rpc=1)
+        assert all(np.array_equal(w[a:b], p) for w, p in zip(whole, part))
