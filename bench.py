@@ -27,6 +27,7 @@ from __future__ import annotations
 import argparse
 import hashlib
 import json
+import math
 import os
 import re
 import statistics
@@ -45,6 +46,9 @@ UNIT = "flip attempts/s"
 # the A, A, B products (3), two sums (2), the sign (2), the two comparisons (2)
 OPS_PER_ATTEMPT = 17
 INT_LANES_PER_SM = 128
+# integer operations of one Philox4x32-10 block (four draws): ten rounds of two
+# wide products and two three-way XORs
+OPS_PER_DRAW_BLOCK = 40
 L2_FLUSH_BYTES = 512 << 20
 DEFAULT_WORKLOAD = "24x24-p0.15"
 
@@ -67,8 +71,8 @@ def parse():
     ap.add_argument("--no-skip-settled", action="store_true")
     ap.add_argument("--no-other-configs", action="store_true")
     ap.add_argument("--replicas-per-cta", type=int, default=0)
-    ap.add_argument("--structured-kernel", default="rows", choices=["rows", "flat"])
-    ap.add_argument("--profile-case", default=None, choices=["rows", "flat", "dense", "mlp", "batch", "repair"],
+    ap.add_argument("--structured-kernel", default="events", choices=["events", "rows", "flat"])
+    ap.add_argument("--profile-case", default=None, choices=["events", "rows", "flat", "dense", "mlp", "batch", "repair"],
                     help="run one warm-up and one measured launch of that kernel on a sub-range of "
                          "the workload (--sweep-window, --replicas), for ncu captures")
     ap.add_argument("--sweep-window", nargs=2, type=int, default=[0, 100])
@@ -93,38 +97,44 @@ def peaks():
 
 
 def kernel_source_hash():
-    """Hash of the row kernel's sources; a recorded ncu figure is used only
-    while it matches."""
+    """Hash of the event-driven kernel's sources; a recorded ncu figure is used
+    only while it matches."""
     h = hashlib.sha256()
-    for f in ["qp_sweep_rows.cu", "qp_rows.cuh", "qp_device.cuh"]:
+    for f in ["qp_sweep_events.cu", "qp_device.cuh"]:
         h.update(open(os.path.join(ROOT, "paper_2608_25376_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
 
-PROFILE_OF = {"24x24-p0.15": "sweep_rows_24x24.md", "10x10-p0.10": "sweep_rows_10x10.md"}
-
-
-def recorded_traffic(workload, kernel_tag="rows"):
-    """DRAM bytes per full launch of the row kernel on `workload`, from the
-    committed ncu summary, if it was taken on the current kernel source (else
-    None)."""
-    name = PROFILE_OF.get(workload)
-    p = os.path.join(ROOT, "profiles", name) if name else None
-    if not p or not os.path.exists(p):
+def recorded_traffic(workload):
+    """DRAM bytes per full launch of the event-driven kernel on `workload`, from
+    the committed ncu summary, if it was taken on the current kernel source
+    (else None)."""
+    p = os.path.join(ROOT, "profiles", "sweep_events.md")
+    if not os.path.exists(p):
         return None
     txt = open(p).read()
     m = re.search(r"kernel_source_hash:\s*([0-9a-f]+)", txt)
-    t = re.search(rf"{kernel_tag}_dram_bytes_per_launch_full:\s*([0-9.eE+]+)", txt)
+    t = re.search(rf"{re.escape(workload)}_dram_bytes_per_launch_full:\s*([0-9.eE+]+)", txt)
     if not m or not t or m.group(1) != kernel_source_hash():
         return None
     return float(t.group(1))
 
 
 def bytes_per_attempt(C):
-    """Algorithmic bytes per flip attempt of the structured sweep (the
-    bytes-per-flip model): each row t of C-1 proposals reads the distance rows
-    of the hot cells of rows t-1 and t+1, 2 rows x C entries x 2 B (int16)."""
+    """Bytes per flip attempt of a structured sweep that evaluates every proposal
+    (the bytes-per-flip model): each row t of C-1 proposals reads the distance
+    rows of the hot cells of rows t-1 and t+1, 2 rows x C entries x 2 B (int16).
+    The event-driven sweep passes over proposals that bounds on the state
+    reject, without reading their distances, so it is no bound on that kernel."""
     return 2 * C * 2 / (C - 1)
+
+
+def hot_sweeps(S, A, T0=1e3, T1=1.0):
+    """Sweeps of the geometric schedule in which a proposal of dE = 2A can be
+    accepted (2A <= T ln 2^32).  Only these need a draw for every proposal: one
+    that adds a second cell to a row or column costs at least 2A, and a cold
+    sweep needs draws at a handful of cells."""
+    return sum(2 * A <= T0 * (T1 / T0) ** (s / max(1, S - 1)) * 32 * math.log(2) for s in range(S))
 
 
 def workload_config(name, f, C, n, w):
@@ -503,9 +513,9 @@ def timed_anneal(h, R, sc, seed, flush, stream, runs=2, warm=True, **kw):
 
 def bench_10x10(flush, stream, pk, pk_kind, skip_settled=True, repair=True):
     """The 10x10 workload (10% obstacles, 92 cells, 1024 replicas x 5000
-    sweeps): the row kernel (d staged in shared memory), the dense-Q kernel
-    (int16 S, 143 MB, streamed from HBM), the row kernel with settled sweeps
-    skipped (same results) and the repair of the final states.  Returns the
+    sweeps): the event-driven kernel (d staged in shared memory), the dense-Q
+    kernel (int16 S, 143 MB, streamed from HBM), the event-driven kernel with
+    settled sweeps skipped (same results) and the repair of the final states.  Returns the
     variant's record and 8 final states for the CPU repair reference."""
     import torch
     from paper_2608_25376_gb300 import inputs, qpath
@@ -518,11 +528,9 @@ def bench_10x10(flush, stream, pk, pk_kind, skip_settled=True, repair=True):
     attempts = R * S * (C - 1) ** 2
     out = {"workload": f"{name}: {C} cells, {R} replicas x {S} sweeps", "attempts": attempts}
     ms, st, E, B, _ = timed_anneal(h, R, sc, seed, flush, stream, runs=3, kernel=qpath.QP_KERNEL_STRUCTURED)
-    rows_ms = statistics.mean(ms)
-    bpa = bytes_per_attempt(C)
-    out["rows"] = {"value": attempts / (rows_ms / 1e3), "unit": UNIT, "kernel_ms": rows_ms,
-                   "bytes_per_flip_GBps": bpa * attempts / (rows_ms / 1e3) / 1e9,
-                   "traffic": recorded_traffic(name)}
+    structured_ms = statistics.mean(ms)
+    out["structured"] = {"value": attempts / (structured_ms / 1e3), "unit": UNIT, "kernel_ms": structured_ms,
+                         "traffic": recorded_traffic(name)}
     ref_E, ref_B = E.clone(), B.clone()
     dms, _, dE, dB, dacc = timed_anneal(h, R, sc, seed, flush, stream, runs=2, kernel=qpath.QP_KERNEL_DENSE)
     dm = statistics.mean(dms)
@@ -531,11 +539,11 @@ def bench_10x10(flush, stream, pk, pk_kind, skip_settled=True, repair=True):
                     "column_bytes_per_launch": col_bytes, "column_GBps": col_bytes / (dm / 1e3) / 1e9,
                     "frac_of_hbm": col_bytes / (dm / 1e3) / 1e9 / pk["hbm_gbs"] if pk.get("hbm_gbs") else None,
                     "hbm_peak_GBps": pk.get("hbm_gbs"), "peak_kind": pk_kind,
-                    "same_results_as_rows": bool(torch.equal(dE, ref_E) and torch.equal(dB, ref_B))}
+                    "same_results_as_structured": bool(torch.equal(dE, ref_E) and torch.equal(dB, ref_B))}
     if skip_settled:
         sms, _, sE, sB, _ = timed_anneal(h, R, sc, seed, flush, stream, runs=3, warm=False,
                                          flags=qpath.QP_ANNEAL_SKIP_SETTLED)
-        out["skip_settled"] = {"ms": statistics.mean(sms), "speedup": rows_ms / statistics.mean(sms),
+        out["skip_settled"] = {"ms": statistics.mean(sms), "speedup": structured_ms / statistics.mean(sms),
                                "same_results": bool(torch.equal(sE, ref_E) and torch.equal(sB, ref_B)),
                                "note": "sweeps after a replica met no proposal with dE < len are not evaluated; "
                                        "not a headline number"}
@@ -602,7 +610,8 @@ def run_ours(args):
     flush = torch.empty(L2_FLUSH_BYTES // 4, dtype=torch.int32, device=dev)
     offset, _ = shard.replica_range(rank, world, R, "weak")
     rpc = args.replicas_per_cta
-    skernel = qpath.QP_KERNEL_STRUCTURED if args.structured_kernel == "rows" else qpath.QP_KERNEL_STRUCTURED_FLAT
+    skernel = {"events": qpath.QP_KERNEL_STRUCTURED, "rows": qpath.QP_KERNEL_STRUCTURED_ROWS,
+               "flat": qpath.QP_KERNEL_STRUCTURED_FLAT}[args.structured_kernel]
 
     def step():
         qpath.qp_anneal_ex(h, R, sc, seed, None, states, E, best, kernel=skernel, replicas_per_cta=rpc,
@@ -650,30 +659,31 @@ def run_ours(args):
     pk, pk_kind = peaks()
     sm_mhz = pk.get("sm_max_mhz", 2070.0)
     ann_ms = statistics.mean(anneal_ms)
-    # the bytes-per-flip roofline: algorithmic bytes per launch / kernel time
-    # against the measured HBM copy rate
-    bpa = bytes_per_attempt(C)
-    achieved_gbs = bpa * attempts / (ann_ms / 1e3) / 1e9
-    # the integer-issue view beside it
+    # the work no kernel of this chain can leave out: one draw per proposal of the
+    # hot sweeps, against the integer issue rate
     peak_tops = sms * INT_LANES_PER_SM * sm_mhz * 1e6 / 1e12
-    achieved_tops = OPS_PER_ATTEMPT * attempts / (ann_ms / 1e3) / 1e12
+    n_hot = hot_sweeps(S, info["A"])
+    draw_blocks = R * n_hot * (C - 1) * C / 4
+    draw_tops = OPS_PER_DRAW_BLOCK * draw_blocks / (ann_ms / 1e3) / 1e12
+    bpa = bytes_per_attempt(C)
+    every_tops = OPS_PER_ATTEMPT * attempts / (ann_ms / 1e3) / 1e12
     d_i16 = info["max_d"] <= 32767
     Cp = (C + 7) // 8 * 8
-    d_where = "shared memory" if C * Cp * 4 <= 160 * 1024 else "L2 (global memory)"
-    roofline = {"bound": "hbm", "achieved": achieved_gbs, "peak": pk.get("hbm_gbs"), "unit": "GB/s",
-                "frac": achieved_gbs / pk["hbm_gbs"] if pk.get("hbm_gbs") else None,
-                "traffic": recorded_traffic(args.workload),
-                "kernel": ("k_sweep_structured" if args.structured_kernel != "rows"
-                           else ("k_sweep_rows_g" if 256 < C <= 512 else "k_sweep_rows")),
-                "kernel_ms": ann_ms, "bytes_per_attempt": bpa,
-                "algorithmic_bytes_per_launch": bpa * attempts,
-                "note": (f"bytes-per-flip model: 2 distance rows x {C} int16 entries per row of {C - 1} "
-                         f"proposals ({bpa:.3f} B per attempt); peak = {pk_kind} HBM copy rate; the d rows "
-                         f"come from {d_where}, so DRAM moves only the tables and the states ('traffic')"),
-                "alu_view": {"achieved": achieved_tops, "peak": peak_tops, "unit": "Tops/s",
-                             "frac": achieved_tops / peak_tops,
-                             "note": f"{OPS_PER_ATTEMPT} algorithmic int ops per attempt; peak = {sms} SMs x "
-                                     f"{INT_LANES_PER_SM} lanes x {sm_mhz:.0f} MHz ({pk_kind} clock)"}}
+    roofline = {"bound": "alu", "achieved": draw_tops, "peak": peak_tops, "unit": "Tops/s",
+                "frac": draw_tops / peak_tops,
+                "traffic": recorded_traffic(args.workload) if args.structured_kernel == "events" else None,
+                "kernel": {"events": "k_sweep_events", "flat": "k_sweep_structured",
+                           "rows": "k_sweep_rows_g" if 256 < C <= 512 else "k_sweep_rows"}[args.structured_kernel],
+                "kernel_ms": ann_ms, "hot_sweeps": n_hot, "draw_blocks_per_launch": draw_blocks,
+                "note": (f"the draws of the {n_hot} of {S} sweeps whose acceptance table reaches 2A, "
+                         f"{OPS_PER_DRAW_BLOCK} integer ops per four draws; peak = {sms} SMs x {INT_LANES_PER_SM} lanes "
+                         f"x {sm_mhz:.0f} MHz ({pk_kind} clock); wide products issue at a quarter of it.  The other "
+                         f"proposals are decided by bounds on the state, row by row of one chain: latency"),
+                "every_attempt_view": {
+                    "note": "what a kernel that evaluates every proposal would have had to do in this time; above the "
+                            "peaks because most proposals are decided without being evaluated",
+                    "bytes_per_attempt": bpa, "GBps": bpa * attempts / (ann_ms / 1e3) / 1e9,
+                    "hbm_peak_GBps": pk.get("hbm_gbs"), "ops_per_attempt": OPS_PER_ATTEMPT, "Tops": every_tops}}
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_max, "higher_is_better": True, "scaling": "weak",
@@ -845,7 +855,7 @@ def run_profile_case(args):
         return 0
     w = inputs.WORKLOADS[args.workload]
     f = w["field"]()
-    kernel = {"rows": qpath.QP_KERNEL_STRUCTURED, "flat": qpath.QP_KERNEL_STRUCTURED_FLAT,
+    kernel = {"events": qpath.QP_KERNEL_STRUCTURED, "rows": qpath.QP_KERNEL_STRUCTURED_ROWS, "flat": qpath.QP_KERNEL_STRUCTURED_FLAT,
               "dense": qpath.QP_KERNEL_DENSE}[args.profile_case]
     flags = qpath.QP_STRUCTURED | (qpath.QP_DENSE if args.profile_case == "dense" else 0)
     h = qpath.qp_build_qubo(f, flags=flags)
