@@ -1,6 +1,6 @@
 // Device helpers of the row-parallel structured sweep (qp_sweep_rows.cu):
-// distance-row loads,
-// row fields, the single-cell cache and the evaluation of one row chunk.
+// distance-row loads, row fields, the single-cell cache and the evaluation of
+// one row chunk.
 // Included inside namespace qp::{anon}.
 #pragma once
 

@@ -34,12 +34,12 @@
 // against the same tables.
 //
 // What bounds it: the latency of one chain, that is its count of dependent
-// instructions (92 cells, T = 1000: 367 warp instructions a row at 3.2 cycles
+// instructions (92 cells, T = 1000: 369 warp instructions a row at 3.2 cycles
 // each with one warp on the SM, memory idle), and in hot sweeps of large fields
 // the Philox multiplies (88 cycles of a scheduler per warp-wide block, whatever
-// the occupancy; 42 of the 83.2 ms below).  Against the row kernels, which
+// the occupancy; 43 of the 83.2 ms below).  Against the row kernels, which
 // evaluate every column of every row (one GB300): 92 cells, 1024 chains x 5000
-// sweeps: 166 -> 32.8 ms (161 -> 64 us a sweep at T = 1000, 1.2 flips a row);
+// sweeps: 166 -> 32.8 ms (161 -> 63 us a sweep at T = 1000, 1.2 flips a row);
 // 491 cells, 4096 chains x 1000 sweeps: 899 -> 83.2 ms; 893 cells, 512 chains x
 // 40 sweeps (the general kernel): 272 -> 22.0 ms.  It is also the faster one far
 // above the temperatures of a useful schedule (T = 1e6, a third of the cells
