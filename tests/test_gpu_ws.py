@@ -148,3 +148,27 @@ def test_training_repeats_bit_for_bit(dev):
         runs.append((losses, qpath.qp_ws_get_params(m)))
     assert runs[0][0] == runs[1][0]
     assert np.array_equal(runs[0][1].view(np.uint32), runs[1][1].view(np.uint32))
+
+
+@pytest.mark.parametrize("rows", [1, 128, 129, 8300])
+def test_launches_that_overlap_keep_their_order(dev, rows):
+    """The launches of a pass start before the one ahead of them has ended: passes
+    over changing inputs and sizes, on two streams, give what each gives alone."""
+    import torch
+    rng = np.random.default_rng(rows)
+    A = rng.random((rows, 16), dtype=np.float32)
+    Bx, Y, T = field_batch(3, seed=9)
+    alone = qpath.WarmStartModel(seed=8)
+    zA, zB = qpath.qp_ws_forward(alone, A), qpath.qp_ws_forward(alone, Bx)
+    loss, g = qpath.qp_ws_grads(alone, Bx, Y, T)
+    m = qpath.WarmStartModel(seed=8)
+    qpath.qp_ws_set_forward_mode(m, qpath.QP_WS_FORWARD_LAYERED)
+    assert np.array_equal(qpath.qp_ws_forward(m, A), zA)
+    qpath.qp_ws_set_forward_mode(m, qpath.QP_WS_FORWARD_FUSED)
+    streams = [None, torch.cuda.Stream()]
+    for k in range(12):
+        st = streams[k & 1]
+        assert np.array_equal(qpath.qp_ws_forward(m, A, stream=st), zA)
+        l2, g2 = qpath.qp_ws_grads(m, Bx, Y, T, stream=st)
+        assert l2 == loss and np.array_equal(g2, g)
+        assert np.array_equal(qpath.qp_ws_forward(m, Bx, stream=st), zB)
