@@ -42,3 +42,28 @@ def test_walk(rows, cols, cells, scale):
         x = st.cpu().numpy().reshape(cells, cells)
         assert x.sum() == cells and (x[np.arange(cells), ref] == 1).all()
     assert (buf[:5] == 9).all()
+
+
+# Without a slack a step is one reduction over (distance, place in the order of
+# scores): distances around the largest that fit beside the place, and scores
+# that tie, are signed zeros or infinite.
+@pytest.mark.parametrize("cells,scale", [(32, 100), (130, 2000), (256, 16384), (257, 25000), (512, 12000), (511, 100)])
+def test_walk_ranked(cells, scale):
+    if not has_gpu():
+        pytest.skip("no CUDA device")
+    import torch
+    qbuild.build()
+    rng = np.random.default_rng(cells + scale)
+    mask = np.zeros(24 * 24, np.uint8)
+    mask[rng.permutation(24 * 24)[:cells]] = 1
+    start = int(np.flatnonzero(mask)[-1])
+    h = qpath.qp_build_qubo(inputs.Field(24, 24, mask, start), scale=scale)
+    d = qpath.qp_export_dist(h)
+    score = np.round(rng.normal(0, 2, cells)).astype(np.float32)
+    score[::7], score[3::11], score[5::13] = -0.0, np.inf, -np.inf
+    for sc in (score, np.zeros(cells, np.float32), None):
+        _, path, ln = qpath.qp_ws_walk(h, None if sc is None else torch.from_numpy(sc).cuda(), 0)
+        torch.cuda.synchronize()
+        ref = mlp_ref.walk(d, cells, cells - 1, sc, 0)
+        assert path.cpu().numpy().tolist() == ref
+        assert int(ln.item()) == sum(int(d[a, b]) for a, b in zip(ref, ref[1:]))
