@@ -21,6 +21,10 @@ constexpr unsigned kFull = 0xffffffffu;
 // index cannot reach memory outside its array.  Sites: 1 threshold table,
 // 2 distance row, 3 spin word, 4 row of S, 5 repair distance, 6 hot-cell list.
 // In the release build QP_IX(i, n, site) is i.
+// QP_POISON(p, bytes, tid, nthreads), called by a whole CTA, fills a 16-byte
+// aligned piece of shared memory with negative numbers before it is staged, and
+// QP_VALUE(v, site) is v, or 0 with the failure recorded when v is negative: a
+// distance read from an entry that nothing wrote.  Site 7: distance value.
 #if QP_DEVICE_CHECKS
 static __device__ unsigned int g_check_word;
 __device__ __forceinline__ long long check_ix(long long i, long long n, unsigned site) {
@@ -29,6 +33,13 @@ __device__ __forceinline__ long long check_ix(long long i, long long n, unsigned
   return 0;
 }
 #define QP_IX(i, n, site) ((decltype(i))::qp::dev::check_ix((long long)(i), (long long)(n), (site)))
+__device__ __forceinline__ void poison(void *p, size_t bytes, int tid, int nthreads) {
+  for (size_t v = tid; v < bytes / 16; v += nthreads)
+    static_cast<uint4 *>(p)[v] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
+  __syncthreads();
+}
+#define QP_POISON(p, bytes, tid, nthreads) ::qp::dev::poison(p, bytes, tid, nthreads)
+#define QP_VALUE(v, site) ((v) >= 0 ? (v) : (int)::qp::dev::check_ix(-1, 0, (site)))
 // Host accessor of the translation unit's word: returns it and clears it.
 #define QP_CHECK_ACCESSOR(fn)                                                        \
   uint32_t fn() {                                                                    \
@@ -41,6 +52,8 @@ __device__ __forceinline__ long long check_ix(long long i, long long n, unsigned
   }
 #else
 #define QP_IX(i, n, site) (i)
+#define QP_POISON(p, bytes, tid, nthreads)
+#define QP_VALUE(v, site) (v)
 #define QP_CHECK_ACCESSOR(fn) \
   uint32_t fn() { return 0; }
 #endif

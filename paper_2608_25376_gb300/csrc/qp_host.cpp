@@ -347,15 +347,20 @@ static qp_status build_field_qubo(const qp_field *f, int32_t A, int32_t B, int32
   QP_CU(cudaMemcpy(h->d32_dev.p, h->d.data(), (size_t)C * C * 4, cudaMemcpyHostToDevice));
   {
     const size_t es = h->d_i16 ? 2 : 4;
-    // The matrix with 16 bytes before it and a row of zeros after it (the
-    // event-driven sweep reads four columns at a time around a row's ends, and
-    // an empty row's distances), the cells' grid coordinates, and d by grid
-    // difference.
+    // The matrix with 16 bytes of zeros before it, and after it a row of zeros
+    // and 16 bytes more (the event-driven sweep reads four columns at a time
+    // around a row's ends, and an empty row's distances), the cells' grid
+    // coordinates, and d by grid difference.
     const int r0 = *std::min_element(cr.begin(), cr.end()), c0 = *std::min_element(cc.begin(), cc.end());
     const int rows = *std::max_element(cr.begin(), cr.end()) - r0 + 1, cols = *std::max_element(cc.begin(), cc.end()) - c0 + 1;
     while ((1 << h->tab_sh) < cols) ++h->tab_sh;
-    if (rows <= 256 && cols <= 256 && (size_t)(rows << h->tab_sh) * es <= 32 * 1024) h->tab_n = rows << h->tab_sh;
-    h->xy_at = 16 + ((size_t)C + 1) * h->Cp * es;
+    // The sweep's columns outside the field lie at the bounding box's first corner, which need be no cell: with the
+    // distances to it, too, |dE| has to fit int32.
+    const int64_t far = round_scaled_sqrt((int64_t)(rows - 1) * (rows - 1) + (int64_t)(cols - 1) * (cols - 1), scale);
+    const bool corner_fits = (double)maxw * far * 2.0 * C + 2.0 * h->A * (2.0 * C + 1.0) < 2147483647.0;
+    if (rows <= 256 && cols <= 256 && corner_fits && (size_t)(rows << h->tab_sh) * es <= 32 * 1024)
+      h->tab_n = rows << h->tab_sh;
+    h->xy_at = 16 + ((size_t)C + 1) * h->Cp * es + 16;
     h->tab_at = h->xy_at + (size_t)h->Cp * 2;
     std::vector<uint8_t> pad(h->tab_at + (size_t)h->tab_n * es, 0);
     if (h->tab_n) {

@@ -120,8 +120,8 @@ struct qp_handle {
   int64_t n = 0, c0 = 0;
   std::vector<int32_t> d;  // C x C (host)
   // device data
-  qp::host::DevBuf d_dev;            // 16 bytes, C x Cp (int16 or int32), a row of zeros, the cells'
-                                     // coordinates, the distance table
+  qp::host::DevBuf d_dev;            // 16 bytes, C x Cp (int16 or int32), a row of zeros, 16 bytes, the
+                                     // cells' coordinates, the distance table
   bool d_i16 = false;
   int32_t Cp = 0;
   const void *d_matrix() const { return d_dev.as<uint8_t>() + 16; }

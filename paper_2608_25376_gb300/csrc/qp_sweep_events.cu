@@ -95,7 +95,7 @@ struct Dist {
   int sh, tab_n;
   __device__ __forceinline__ int lookup(uint32_t a, uint32_t b) const {
     const uint32_t ad = __vabsdiffu4(a, b);
-    return (int)m[QP_IX((int)(((ad >> 8) << sh) + (ad & 0xFFu)), tab_n, 2)];
+    return QP_VALUE((int)m[QP_IX((int)(((ad >> 8) << sh) + (ad & 0xFFu)), tab_n, 2)], 7);
   }
   // A cell as hx keeps it (its coordinates when they are all a distance needs,
   // which spares the gather of them), and the distance of two of those.
@@ -122,7 +122,7 @@ struct Dist {
     } else {
       const DT *p = m + QP_IX(h, C + 1, 2) * Cp + i;
 #pragma unroll
-      for (int j = 0; j < 4; ++j) f[j] += DM == 1 ? (int)p[j] : (int)__ldg(p + j);
+      for (int j = 0; j < 4; ++j) f[j] += QP_VALUE(DM == 1 ? (int)p[j] : (int)__ldg(p + j), 7);
     }
   }
 };
@@ -726,6 +726,10 @@ __host__ __device__ inline size_t events_dist_bytes(int C, int Cp, size_t es, in
   return 0;
 }
 
+// A column outside the field is rejected by its bound INT_MIN, so its dE must not
+// be INT_MIN too: it stays within the bound that keeps a cell's inside int32.  The
+// entries around the matrix are zeros; with the table such a column lies at grid
+// difference (0, 0), which the table's owner takes into that bound.
 template <typename DT, int DM>
 __device__ __forceinline__ Dist<DT, DM> stage_dist(const StructArgs &a, unsigned char *p, int tid, int nthreads) {
   Dist<DT, DM> D{static_cast<const DT *>(a.d), a.Cp, a.C, nullptr, a.tab_sh, a.tab_n};
@@ -733,12 +737,15 @@ __device__ __forceinline__ Dist<DT, DM> stage_dist(const StructArgs &a, unsigned
     const int nv = (int)((size_t)a.C * a.Cp * sizeof(DT) / 16);
     const int4 *src = static_cast<const int4 *>(a.d);
     DT *m = reinterpret_cast<DT *>(p) + kPad;
+    QP_POISON(p, events_dist_bytes(a.C, a.Cp, sizeof(DT), DM, 0), tid, nthreads);
     for (int v = tid; v < nv; v += nthreads) reinterpret_cast<int4 *>(m)[v] = __ldg(src + v);
-    for (int i = tid; i < a.Cp; i += nthreads) m[a.C * a.Cp + i] = 0;
+    if (tid < kPad) m[tid - kPad] = 0;
+    for (int i = tid; i < a.Cp + kPad; i += nthreads) m[a.C * a.Cp + i] = 0;
     D.m = m;
   } else if (DM == 2) {
     uint16_t *xy = reinterpret_cast<uint16_t *>(p) + kPad;
     DT *tab = reinterpret_cast<DT *>(p + align16e(2 * ((size_t)a.C + 2 * kPad)));
+    QP_POISON(p, events_dist_bytes(a.C, a.Cp, sizeof(DT), DM, a.tab_n), tid, nthreads);
     for (int i = tid - kPad; i < a.C + kPad; i += nthreads) xy[i] = i >= 0 && i < a.C ? __ldg(a.xy + i) : 0;
     for (int i = tid; i < a.tab_n; i += nthreads) tab[i] = __ldg(static_cast<const DT *>(a.tab) + i);
     D.xy = xy;
