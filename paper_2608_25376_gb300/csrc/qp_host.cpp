@@ -859,6 +859,16 @@ void clear_error() { g_err.clear(); }
 
 bool device_pointer(const void *p) { return is_device_ptr(p); }
 
+int memory_place(const void *p) {
+  if (!p) return kHostMemory;
+  cudaPointerAttributes at;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return kHostMemory;
+  }
+  return at.type == cudaMemoryTypeDevice ? at.device : at.type == cudaMemoryTypeManaged ? kManagedMemory : kHostMemory;
+}
+
 namespace {
 using GetAddressRange = int (*)(unsigned long long *, size_t *, unsigned long long);
 GetAddressRange address_range_fn() {

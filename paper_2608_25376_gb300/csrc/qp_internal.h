@@ -187,6 +187,9 @@ bool schedule_lookup(const qp_schedule &sc, DeviceSchedule *out, std::shared_ptr
 qp_status set_error(qp_status s, const char *msg);
 void clear_error();  // empties this thread's qp_last_error message
 bool device_pointer(const void *p);
+// The device that holds p, or one of the two below.
+constexpr int kHostMemory = -1, kManagedMemory = -2;
+int memory_place(const void *p);
 // True when the caller's device buffer [p, p + bytes) lies inside the one
 // allocation that holds p (cuMemGetAddressRange), or when the driver cannot
 // tell (p not in its allocation tables).  A pooling allocator's buffer lies

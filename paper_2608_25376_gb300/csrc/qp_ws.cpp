@@ -330,14 +330,16 @@ extern "C" qp_status qp_ws_set_params(qp_ws *m, const float *in) {
 
 extern "C" qp_status qp_ws_forward(qp_ws *m, const float *feats, int32_t M, float *logits_out, void *stream) {
   if (!m || !feats || !logits_out || M < 1) return set_error(QP_EINVAL, "bad argument");
-  const bool dev_out = device_pointer(logits_out);
-  if (dev_out && !device_range_fits(logits_out, (size_t)M * kOut * 4))
+  const int place = memory_place(logits_out);
+  if (place != kHostMemory && !device_range_fits(logits_out, (size_t)M * kOut * 4))
     return set_error(QP_EINVAL, "qp_ws_forward: the device buffer for the logits is too small");
   DevGuard g(m->dev);
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int Mp = (M + 127) / 128 * 128;
-  // the fused kernel writes the caller's logits beside its own when it can
-  const bool direct = dev_out && m->fwd_mode == QP_WS_FORWARD_FUSED && (reinterpret_cast<uintptr_t>(logits_out) & 15) == 0;
+  // the fused kernel writes the caller's logits beside its own when they lie on its GPU (another GPU's memory need not
+  // be mapped here: those are copied)
+  const bool direct =
+      place == m->dev && m->fwd_mode == QP_WS_FORWARD_FUSED && (reinterpret_cast<uintptr_t>(logits_out) & 15) == 0;
   PassResult r{};
   const auto pass = [&]() -> qp_status {
     if (qp_status s = upload_inputs(m, feats, M, Mp, nullptr, nullptr, st); s != QP_OK) return s;
