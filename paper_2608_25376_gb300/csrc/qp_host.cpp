@@ -60,6 +60,11 @@ cudaError_t dev_malloc(void **p, size_t bytes) {
     }
     if (left > 0) --left;
   }
+  if (const char *over = std::getenv("QPATH_FAIL_ALLOC_OVER"))
+    if (*over && bytes > std::strtoull(over, nullptr, 10)) {
+      *p = nullptr;
+      return cudaErrorMemoryAllocation;
+    }
   return cudaMalloc(p, bytes);
 }
 

@@ -206,7 +206,8 @@ void noalloc_preload();
 // Every device allocation of the library.  Fault injection for tests: when
 // the environment variable QPATH_FAIL_ALLOC holds N, the next N allocations
 // (counted from the moment the value was first seen) succeed and every later
-// one fails with cudaErrorMemoryAllocation, until the value changes.
+// one fails with cudaErrorMemoryAllocation, until the value changes; when
+// QPATH_FAIL_ALLOC_OVER holds N, every allocation of more than N bytes fails.
 cudaError_t dev_malloc(void **p, size_t bytes);
 
 // Device bounds checks of the checked build (QP_DEVICE_CHECKS=1): each

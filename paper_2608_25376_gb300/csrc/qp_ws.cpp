@@ -45,6 +45,11 @@ struct Buf {
     bytes = want;
     return true;
   }
+  void release() {
+    if (p) cudaFree(p);
+    p = nullptr;
+    bytes = 0;
+  }
   template <typename T>
   T *as() const { return static_cast<T *>(p); }
 };
@@ -80,11 +85,14 @@ struct qp_ws {
   int step = 0;
   Buf par, am, av, grad;               // fp32 masters, Adam's moments, gradients: flat (mlp::kParams)
   Buf wb, wt;                          // bf16 weights and their transposes, at the weights' flat offsets
-  int cap = 0;                         // rows the activation buffers hold
+  int cap = 0;                         // rows of the largest pass so far
   int fwd_mode = QP_WS_FORWARD_FUSED;
-  Buf xf, x0, h[3], z, dz, dh[3], lab, stp, res;
-  Buf tr;              // transposes for the weight gradients: dY of the four layers, then X of them
-  Buf gws, cws, lrow;  // split-K partials, column-sum partials, per-row losses (fixed-order sums)
+  Buf x0, z, res;                      // z holds the fp32 features until they are converted
+  Buf h[3];                            // passes that keep the hidden activations
+  Buf dz, dh[3], lab, stp;             // training passes, as the rest
+  Buf tr;              // transposes for the weight gradients: dY and X of `group` layers
+  Buf gws, cws, lrow;  // split-K partials of `group` layers, column-sum partials, per-row losses (fixed-order sums)
+  int group = 0;       // layers whose weight gradients are computed side by side: all, or 1 when memory is short
 
   float *weight(const Buf &b, int l) const { return b.as<float>() + mlp::weight_offset(l); }
   float *bias(const Buf &b, int l) const { return b.as<float>() + mlp::bias_offset(l); }
@@ -96,23 +104,37 @@ namespace {
 
 static_assert(kIn == 16 && kHid == 256 && kOut == 256 && kLayers == 4, "the flat layout of mlp::kParams");
 
-qp_status ensure_rows(qp_ws *m, int Mp) {
-  if (Mp <= m->cap) return QP_OK;
-  m->cap = 0;  // a failed growth below leaves some buffers empty: check them all next time
-  WS_ALLOC(m->xf, (size_t)Mp * kIn * 4);
-  WS_ALLOC(m->x0, (size_t)Mp * kIn * 2);
-  for (int i = 0; i < 3; ++i) {
-    WS_ALLOC(m->h[i], (size_t)Mp * kHid * 2);
-    WS_ALLOC(m->dh[i], (size_t)Mp * kHid * 2);
+int weight_splits(int Mp) { return std::max(1, Mp / 512); }
+
+// The buffers of a pass over Mp rows.  A row takes 1056 bytes, 2592 with the
+// hidden activations and 8268 in training; where those cannot be had, the weight
+// gradients of the layers share one layer's buffers and it is 5676.
+qp_status ensure_rows(qp_ws *m, int Mp, bool hidden, bool train) {
+  const int cap = m->cap;
+  if (Mp > cap) m->cap = 0;  // until the growth below has succeeded
+  const size_t rows = Mp;
+  WS_ALLOC(m->x0, rows * kIn * 2);
+  WS_ALLOC(m->z, rows * kOut * 4);
+  if (hidden)
+    for (int i = 0; i < 3; ++i) WS_ALLOC(m->h[i], rows * kHid * 2);
+  if (train) {
+    for (int i = 0; i < 3; ++i) WS_ALLOC(m->dh[i], rows * kHid * 2);
+    WS_ALLOC(m->dz, rows * kOut * 2);
+    WS_ALLOC(m->lab, rows * 4);
+    WS_ALLOC(m->stp, rows * 4);
+    WS_ALLOC(m->lrow, rows * 4);
+    WS_ALLOC(m->cws, (size_t)kLayers * mlp::kColsumSlabs * kOut * 4);
+    const size_t zs = mlp::gemm_splits(Mp, weight_splits(Mp));
+    m->group = kLayers;
+    if (!m->tr.ensure(rows * (kLayers * kHid + kIn + 3 * kHid) * 2) || !m->gws.ensure(zs * mlp::kParams * 4)) {
+      m->group = 1;
+      m->tr.release();
+      m->gws.release();
+      WS_ALLOC(m->tr, rows * 2 * kHid * 2);
+      WS_ALLOC(m->gws, zs * kHid * kHid * 4);
+    }
   }
-  WS_ALLOC(m->z, (size_t)Mp * kOut * 4);
-  WS_ALLOC(m->dz, (size_t)Mp * kOut * 2);
-  WS_ALLOC(m->tr, (size_t)Mp * (kLayers * kHid + kIn + 3 * kHid) * 2);
-  WS_ALLOC(m->lab, (size_t)Mp * 4);
-  WS_ALLOC(m->stp, (size_t)Mp * 4);
-  WS_ALLOC(m->lrow, (size_t)Mp * 4);
-  WS_ALLOC(m->cws, (size_t)kLayers * mlp::kColsumSlabs * kOut * 4);
-  m->cap = Mp;
+  m->cap = std::max(cap, Mp);
   return QP_OK;
 }
 
@@ -121,14 +143,14 @@ qp_status ensure_rows(qp_ws *m, int Mp) {
 // reading the caller's buffers on return: every caller waits for the stream.
 qp_status upload_inputs(qp_ws *m, const float *feats, int M, int Mp, const int32_t *labels, const int32_t *steps,
                         cudaStream_t st) {
-  if (qp_status s = ensure_rows(m, Mp); s != QP_OK) return s;
-  WS_CU(cudaMemcpyAsync(m->xf.p, feats, (size_t)M * kIn * 4, cudaMemcpyHostToDevice, st));
   const bool train = labels && steps;
+  if (qp_status s = ensure_rows(m, Mp, train || m->fwd_mode != QP_WS_FORWARD_FUSED, train); s != QP_OK) return s;
+  WS_CU(cudaMemcpyAsync(m->z.p, feats, (size_t)M * kIn * 4, cudaMemcpyHostToDevice, st));
   if (train) {
     WS_CU(cudaMemcpyAsync(m->lab.p, labels, (size_t)M * 4, cudaMemcpyHostToDevice, st));
     WS_CU(cudaMemcpyAsync(m->stp.p, steps, (size_t)M * 4, cudaMemcpyHostToDevice, st));
   }
-  WS_CU(mlp::inputs(m->xf.as<float>(), M, Mp, m->x0.as<__nv_bfloat16>(), train ? m->lab.as<int32_t>() : nullptr,
+  WS_CU(mlp::inputs(m->z.as<float>(), M, Mp, m->x0.as<__nv_bfloat16>(), train ? m->lab.as<int32_t>() : nullptr,
                     train ? m->stp.as<int32_t>() : nullptr, st));
   return QP_OK;
 }
@@ -187,7 +209,8 @@ qp_status forward(qp_ws *m, int Mp, bool keep_hidden, float *out, int rows, cuda
 // Every sum over rows is taken in a fixed order (split-K partials and slabs
 // added in index order, no atomics), so a training run repeats bit for bit.
 // The chain of the dX products runs in one launch, and everything else of the
-// four layers side by side in one launch of its kind.
+// four layers side by side in one launch of its kind (of one layer after the
+// other when the buffers are shared: the same products and sums).
 qp_status backward(qp_ws *m, int M, int Mp, cudaStream_t st) {
   int *err = &m->result()->err;
   mlp::BwdArgs bw{};
@@ -206,37 +229,39 @@ qp_status backward(qp_ws *m, int M, int Mp, cudaStream_t st) {
     bw.dh[l] = m->dh[l].as<__nv_bfloat16>();
   }
   WS_CU(mlp::backward(bw, wt, st));
-  const int splits = std::max(1, Mp / 512), zs = mlp::gemm_splits(Mp, splits);
-  WS_ALLOC(m->gws, (size_t)zs * mlp::kParams * 4);
+  const int splits = weight_splits(Mp), zs = mlp::gemm_splits(Mp, splits);
   const __nv_bfloat16 *dy[kLayers], *x[kLayers];
   for (int l = 0; l < kLayers; ++l) {
     dy[l] = l == kLayers - 1 ? m->dz.as<__nv_bfloat16>() : m->dh[l].as<__nv_bfloat16>();
     x[l] = l == 0 ? m->x0.as<__nv_bfloat16>() : m->h[l - 1].as<__nv_bfloat16>();
   }
   // dW[out][in] = sum_m dY[m][out] X[m][in]  (operands transposed so m is contiguous)
-  __nv_bfloat16 *tr = m->tr.as<__nv_bfloat16>();
-  mlp::TransposeJob tj[2 * kLayers];
-  mlp::GemmArgs g[kLayers];
-  mlp::SumJob sums[2 * kLayers];
-  float *ws = m->gws.as<float>();
-  for (int l = 0; l < kLayers; ++l) {
-    __nv_bfloat16 *dyt = tr, *xt = tr + (size_t)Mp * kDimOut[l];
-    tr = xt + (size_t)Mp * kDimIn[l];
-    tj[2 * l] = {dy[l], dyt, kDimOut[l]};
-    tj[2 * l + 1] = {x[l], xt, kDimIn[l]};
-    g[l] = gargs(dyt, Mp, xt, Mp, kDimOut[l], kDimIn[l], Mp, mlp::kEpiPartialF32, err);
-    g[l].out_f32 = ws;
-    g[l].ldo = kDimIn[l];
-    const int n = kDimOut[l] * kDimIn[l];
-    sums[2 * l] = {ws, zs, n, m->weight(m->grad, l)};
-    sums[2 * l + 1] = {m->cws.as<float>() + (size_t)l * mlp::kColsumSlabs * kOut, mlp::kColsumSlabs, kOut,
-                       m->bias(m->grad, l)};
-    ws += (size_t)zs * n;
+  for (int l0 = 0; l0 < kLayers; l0 += m->group) {
+    __nv_bfloat16 *tr = m->tr.as<__nv_bfloat16>();
+    mlp::TransposeJob tj[2 * kLayers];
+    mlp::GemmArgs g[kLayers];
+    mlp::SumJob sums[2 * kLayers];
+    float *ws = m->gws.as<float>();
+    for (int k = 0; k < m->group; ++k) {
+      const int l = l0 + k;
+      __nv_bfloat16 *dyt = tr, *xt = tr + (size_t)Mp * kDimOut[l];
+      tr = xt + (size_t)Mp * kDimIn[l];
+      tj[2 * k] = {dy[l], dyt, kDimOut[l]};
+      tj[2 * k + 1] = {x[l], xt, kDimIn[l]};
+      g[k] = gargs(dyt, Mp, xt, Mp, kDimOut[l], kDimIn[l], Mp, mlp::kEpiPartialF32, err);
+      g[k].out_f32 = ws;
+      g[k].ldo = kDimIn[l];
+      const int n = kDimOut[l] * kDimIn[l];
+      sums[2 * k] = {ws, zs, n, m->weight(m->grad, l)};
+      sums[2 * k + 1] = {m->cws.as<float>() + (size_t)l * mlp::kColsumSlabs * kOut, mlp::kColsumSlabs, kOut,
+                         m->bias(m->grad, l)};
+      ws += (size_t)zs * n;
+    }
+    WS_CU(mlp::transpose(tj, 2 * m->group, Mp, st));
+    WS_CU(mlp::gemm(g, m->group, splits, st));
+    if (l0 == 0) WS_CU(mlp::colsum(dy, kLayers, Mp, m->cws.as<float>(), st));
+    WS_CU(mlp::sum_jobs(sums, 2 * m->group, l0 == 0 ? m->lrow.as<float>() : nullptr, Mp, &m->result()->loss, st));
   }
-  WS_CU(mlp::transpose(tj, 2 * kLayers, Mp, st));
-  WS_CU(mlp::gemm(g, kLayers, splits, st));
-  WS_CU(mlp::colsum(dy, kLayers, Mp, m->cws.as<float>(), st));
-  WS_CU(mlp::sum_jobs(sums, 2 * kLayers, m->lrow.as<float>(), Mp, &m->result()->loss, st));
   return QP_OK;
 }
 
@@ -421,7 +446,7 @@ extern "C" qp_status qp_ws_get_buffer(qp_ws *m, int32_t which, int32_t rows, voi
       return QP_OK;
     }
   if (rows < 1 || rows > m->cap) return set_error(QP_EINVAL, "rows beyond the last pass's buffers");
-  const Buf *b = nullptr;
+  Buf *b = nullptr;
   size_t row_bytes = (size_t)kHid * 2;
   switch (which) {
     case QP_WS_BUF_X0: b = &m->x0; row_bytes = (size_t)kIn * 2; break;
@@ -432,6 +457,7 @@ extern "C" qp_status qp_ws_get_buffer(qp_ws *m, int32_t which, int32_t rows, voi
     default: return set_error(QP_EINVAL, "unknown buffer");
   }
   WS_CU(cudaDeviceSynchronize());
+  WS_ALLOC(*b, (size_t)rows * row_bytes);  // no pass has written it: no defined values
   WS_CU(cudaMemcpy(out, b->p, (size_t)rows * row_bytes, cudaMemcpyDeviceToHost));
   return QP_OK;
 }

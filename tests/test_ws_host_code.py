@@ -11,6 +11,7 @@ from paper_2608_25376_gb300 import build as qbuild
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 HOST, MANAGED = -1, -2
+ENOMEM = 2
 
 
 @pytest.fixture(scope="module")
@@ -61,3 +62,58 @@ def test_forward_writes_only_its_own_gpu(lib, model, place, direct):
     assert lib.qp_ws_forward(model, ptr(feats), M, ptr(out), None) == 0
     assert (lib.fake_z2() == out.ctypes.data) == direct
     assert (lib.fake_copied() - before == 0) == direct
+
+
+# What a pass over Mp rows took when every product had its buffers to itself: one layer's transposes and split-K
+# partials at a time.  A card whose memory is nearly full has to go on taking the row counts that fitted then.
+ROW_BYTES = 5676
+
+
+def old_training_bytes(Mp):
+    splits = max(1, Mp // 512)
+    per = -(-(-(-Mp // splits)) // 64) * 64
+    return ROW_BYTES * Mp + -(-Mp // per) * 256 * 256 * 4 + 64 * 256 * 4  # and the column sums' slabs
+
+
+@pytest.mark.parametrize("mode", [0, 1])
+def test_forward_memory(lib, model, mode):
+    M = 5000
+    Mp = 5120
+    base = lib.fake_bytes()
+    assert lib.qp_ws_set_forward_mode(model, mode) == 0
+    lib.fake_limit(base + ROW_BYTES * Mp)
+    out, feats = logits(M), np.zeros((M, 16), np.float32)
+    assert lib.qp_ws_forward(model, ptr(feats), M, ptr(out), None) == 0, lib.fake_error()
+    assert lib.fake_bytes() - base <= ROW_BYTES * Mp
+    # every buffer can still be read back, whether or not the pass wrote it
+    lib.fake_limit(1 << 60)
+    buf = np.zeros(Mp * 1024, np.uint8)
+    for which in range(9):
+        assert lib.qp_ws_get_buffer(model, which, Mp, ptr(buf)) == 0
+    assert lib.qp_ws_get_buffer(model, 0, Mp + 1, ptr(buf)) != 0
+
+
+def test_training_memory(lib, model):
+    M = 5000
+    Mp = 5120
+    base = lib.fake_bytes()
+    feats = np.zeros((M, 16), np.float32)
+    labels, steps = np.zeros(M, np.int32), np.full(M, 7, np.int32)
+    loss = ctypes.c_float()
+
+    def step():
+        return lib.qp_ws_train_step(model, ptr(feats), ptr(labels), ptr(steps), M, ctypes.c_float(1e-3),
+                                    ctypes.byref(loss), None)
+
+    lib.fake_limit(base + old_training_bytes(Mp) + 3 * 64 * 256 * 4)  # the slabs of three more layers: no row's worth
+    assert step() == 0, lib.fake_error()
+    assert lib.fake_launches() == b"ifb" + b"tgcs" + 3 * b"tgs" + b"a"
+    assert lib.qp_ws_forward(model, ptr(feats), M, ptr(logits(M)), None) == 0
+    lib.fake_launches()
+    lib.fake_limit(lib.fake_bytes())  # more rows: refused before any launch, and the model goes on
+    more = np.zeros((4 * M, 16), np.float32)
+    assert lib.qp_ws_forward(model, ptr(more), 4 * M, ptr(logits(4 * M)), None) == ENOMEM
+    assert lib.fake_launches() == b""
+    lib.fake_limit(1 << 60)
+    assert step() == 0
+    assert lib.fake_launches() == b"ifbtgcsa"  # all layers side by side
