@@ -5,15 +5,19 @@ Picks replicas-per-CTA for the single-field structured sweep, and
 staging choice being each field's distance matrix read from L2 by every warp,
 or staged in shared memory by a CTA that runs a block of that field's
 replicas (QP_BATCH_D_SHARED) -- by timing each candidate on short windows of
-the actual schedule (its hottest and its coldest sweeps) with CUDA events.  Results are cached in a JSON file keyed by GPU
-model, kernel and field-size class (cells rounded up to a multiple of 32, plus
-the replica count), so a configuration is measured once per machine.  The
-choice never changes results: every configuration runs the same chains.
+the actual schedule (its hottest and its coldest sweeps) with CUDA events.
+Results are cached in a JSON file keyed by GPU model, kernel (with a hash of its
+source: a configuration measured on another version of it is measured again) and
+field-size class (cells rounded up to a multiple of 32, plus the replica count),
+so a configuration is measured once per machine.  The choice never changes
+results: every configuration runs the same chains.
 
 Cache file: $QPATH_AUTOTUNE_CACHE, else _build/autotune.json next to this file.
 """
 from __future__ import annotations
 
+import functools
+import hashlib
 import json
 import math
 import os
@@ -52,6 +56,20 @@ def _gpu_key() -> str:
     return f"{p.name}/{p.multi_processor_count}sm"
 
 
+@functools.lru_cache(maxsize=None)
+def _kernel_key() -> str:
+    """The kernel the configurations are for, and a hash of its source and launch rules."""
+    csrc = os.path.join(os.path.dirname(os.path.abspath(__file__)), "csrc")
+    h = hashlib.sha256()
+    try:
+        for name in ("qp_sweep_events.cu", "qp_device.cuh"):
+            with open(os.path.join(csrc, name), "rb") as f:
+                h.update(f.read())
+    except OSError:  # a library without its sources
+        return "events"
+    return f"events-{h.hexdigest()[:12]}"
+
+
 def size_class(C: int) -> int:
     return int(math.ceil(C / 32.0)) * 32
 
@@ -77,11 +95,11 @@ def _time(fn, reps: int = 2) -> float:
 
 
 def tune_single(h: "qpath.Handle", replicas: int, n_sweeps: int, T0: float = 1e3, T1: float = 1.0,
-                candidates=(1, 2, 4, 8, 16), window: int = 40, refresh: bool = False) -> int:
-    """Best replicas-per-CTA for qp_anneal_ex's structured kernel on this field size."""
+                candidates=(0, 1, 2, 4, 8, 16), window: int = 40, refresh: bool = False) -> int:
+    """Best replicas-per-CTA for qp_anneal_ex's structured kernel on this field size (0: the launch's own choice)."""
     import torch
     C = h.info["C"]
-    key = f"{_gpu_key()}|rows|C{size_class(C)}|R{replicas}"
+    key = f"{_gpu_key()}|{_kernel_key()}|C{size_class(C)}|R{replicas}"
     with _lock:
         cache = _load()
         if not refresh and key in cache:
@@ -114,7 +132,7 @@ def tune_batch(handles, replicas: int, n_sweeps: int, T0: float = 1e3, T1: float
     staged in shared memory per CTA)."""
     import torch
     Cs = sorted(h.info["C"] for h in handles)
-    key = (f"{_gpu_key()}|batch|F{len(handles)}|Cmax{size_class(Cs[-1])}|Cmed{size_class(Cs[len(Cs) // 2])}"
+    key = (f"{_gpu_key()}|{_kernel_key()}|batch|F{len(handles)}|Cmax{size_class(Cs[-1])}|Cmed{size_class(Cs[len(Cs) // 2])}"
            f"|R{replicas}|stagings{','.join(str(x) for x in stagings)}")
     with _lock:
         cache = _load()
