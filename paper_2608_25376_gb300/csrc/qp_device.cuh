@@ -19,8 +19,11 @@ constexpr unsigned kFull = 0xffffffffu;
 // the first failure of the translation unit's kernels is recorded as
 // (site << 24) | (i mod 2^24) and the access goes to element 0, so a wrong
 // index cannot reach memory outside its array.  Sites: 1 threshold table,
-// 2 distance row, 3 spin word, 4 row of S, 5 repair distance, 6 hot-cell list.
+// 2 distance row, 3 spin word, 4 row of S, 5 repair distance, 6 hot-cell list,
+// 8 column sum, 9 row record, 10 cell coordinates, 11 state, path or order of
+// the output, 12 repair path and edges.
 // In the release build QP_IX(i, n, site) is i.
+// QP_RANGE(i, lo, hi, site): the same for lo <= i < hi (element lo instead).
 // QP_POISON(p, bytes, tid, nthreads), called by a whole CTA, fills a 16-byte
 // aligned piece of shared memory with negative numbers before it is staged, and
 // QP_VALUE(v, site) is v, or 0 with the failure recorded when v is negative: a
@@ -32,12 +35,14 @@ __device__ __forceinline__ long long check_ix(long long i, long long n, unsigned
   atomicCAS(&g_check_word, 0u, (site << 24) | ((unsigned)i & 0xFFFFFFu));
   return 0;
 }
-#define QP_IX(i, n, site) ((decltype(i))::qp::dev::check_ix((long long)(i), (long long)(n), (site)))
+#define QP_IX(i, n, site) ((decltype((i) + 0))::qp::dev::check_ix((long long)(i), (long long)(n), (site)))
 __device__ __forceinline__ void poison(void *p, size_t bytes, int tid, int nthreads) {
   for (size_t v = tid; v < bytes / 16; v += nthreads)
     static_cast<uint4 *>(p)[v] = make_uint4(0x80808080u, 0x80808080u, 0x80808080u, 0x80808080u);
   __syncthreads();
 }
+#define QP_RANGE(i, lo, hi, site) \
+  ((decltype((i) + 0))(::qp::dev::check_ix((long long)(i) - (lo), (long long)(hi) - (lo), (site)) + (lo)))
 #define QP_POISON(p, bytes, tid, nthreads) ::qp::dev::poison(p, bytes, tid, nthreads)
 #define QP_VALUE(v, site) ((v) >= 0 ? (v) : (int)::qp::dev::check_ix(-1, 0, (site)))
 // Host accessor of the translation unit's word: returns it and clears it.
@@ -52,6 +57,7 @@ __device__ __forceinline__ void poison(void *p, size_t bytes, int tid, int nthre
   }
 #else
 #define QP_IX(i, n, site) (i)
+#define QP_RANGE(i, lo, hi, site) (i)
 #define QP_POISON(p, bytes, tid, nthreads)
 #define QP_VALUE(v, site) (v)
 #define QP_CHECK_ACCESSOR(fn) \

@@ -517,7 +517,8 @@ extern "C" qp_status qp_device_checks(int32_t *enabled, uint32_t *first_failure)
   *enabled = qp::chk::enabled();
   uint32_t w = 0;
   bool read_failed = false;
-  for (uint32_t (*take)() : {qp::chk::rows, qp::chk::kernels, qp::chk::group, qp::chk::events, qp::chk::repair}) {
+  for (uint32_t (*take)() : {qp::chk::rows, qp::chk::kernels, qp::chk::group, qp::chk::events, qp::chk::repair,
+                             qp::chk::walk}) {
     const uint32_t v = take();
     if (v == 0xFFFFFFFFu) {  // the record could not be read from the device
       read_failed = true;

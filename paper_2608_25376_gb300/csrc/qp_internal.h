@@ -219,6 +219,7 @@ uint32_t rows();
 uint32_t group();
 uint32_t events();
 uint32_t repair();
+uint32_t walk();
 int32_t enabled();
 }  // namespace chk
 

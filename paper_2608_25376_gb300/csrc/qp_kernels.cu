@@ -669,7 +669,7 @@ __global__ void k_decode(const uint8_t *states, int C, const int32_t *d, int32_t
   if (tid == 0) s_len = 0;
   __syncthreads();
   auto set = [&](int k) {
-    const int t = k / C, i = k - t * C;
+    const int t = QP_IX(k / C, C, 11), i = k - t * C;
     atomicMax(at + t, i);
     atomicAdd(cnt + t, 1u);
     atomicAdd(cnt + i, 0x10000u);
@@ -698,7 +698,7 @@ __global__ void k_decode(const uint8_t *states, int C, const int32_t *d, int32_t
   long long L = 0;
   for (int t = tid; t < C; t += nt) {
     path[t] = at[t];
-    if (ok && t + 1 < C) L += d[(size_t)at[t] * C + at[t + 1]];
+    if (ok && t + 1 < C) L += d[(size_t)QP_IX(at[t], C, 2) * C + QP_IX(at[t + 1], C, 2)];
   }
   L = warp_sum64(L);
   if (nt == 32) {

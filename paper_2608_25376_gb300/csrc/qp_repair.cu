@@ -243,7 +243,7 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
   }
   __syncwarp();
   auto set = [&](int k) {
-    const int t = k / C, i = k - t * C;
+    const int t = QP_IX(k / C, C, 12), i = k - t * C;
     at[t] = i;  // any of them when there are several
     atomicAdd(cnt + t, 1u);
     atomicAdd(cnt + i, 0x10000u);
@@ -270,7 +270,7 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
   if (feasible) {
     for (int t = lane; t < C; t += 32) {
       id[t] = (uint16_t)at[t];
-      path[t] = xy[at[t]];
+      path[t] = xy[QP_IX(at[t], C, 12)];
     }
   } else {
     // greedy fix
@@ -293,7 +293,7 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
           for (int i = lane; i < C; i += 32) {
             if ((used[i >> 5] >> (i & 31)) & 1u) continue;
             if (!any && x[(size_t)t * C + i] == 0) continue;
-            const uint32_t v = D(prev, xy[i]);
+            const uint32_t v = D(prev, xy[QP_IX(i, C, 12)]);
             if (v < bd) {  // i ascends: ties keep the smaller
               bd = v;
               bi = (uint32_t)i;
@@ -304,7 +304,7 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
           if (b != 0xFFFFFFFFu) pick = (int)b;
         }
       }
-      prev = xy[pick];
+      prev = xy[QP_IX(pick, C, 12)];
       __syncwarp();
       if (lane == 0) {
         id[t] = (uint16_t)pick;
@@ -335,7 +335,7 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
           const uint32_t e1 = edge[i - 1];
           {
             const int j = j0 + lane, jc = min(j, C - 2);
-            const uint32_t n1 = D(a, path[min(j, C - 1)]), n2 = j + 1 < C ? D(b, path[jc + 1]) : 0u;
+            const uint32_t n1 = D(a, path[QP_IX(min(j, C - 1), C, 12)]), n2 = j + 1 < C ? D(b, path[QP_IX(jc + 1, C, 12)]) : 0u;
             const unsigned m = __ballot_sync(kFull, j < C && n1 + n2 < e1 + (j + 1 < C ? edge[jc] : 0u));
             if (m) {
               const int f = __ffs(m) - 1;
@@ -350,9 +350,9 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
               const int j = jb + 32 * q + lane, jc = min(j, C - 2);
-              n1[q] = D(a, path[min(j, C - 1)]);
-              n2[q] = j + 1 < C ? D(b, path[jc + 1]) : 0u;
-              imp[q] = j < C && n1[q] + n2[q] < e1 + (j + 1 < C ? edge[jc] : 0u);
+              n1[q] = D(a, path[QP_IX(min(j, C - 1), C, 12)]);
+              n2[q] = j + 1 < C ? D(b, path[QP_IX(jc + 1, C, 12)]) : 0u;
+              imp[q] = j < C && n1[q] + n2[q] < e1 + (j + 1 < C ? edge[QP_IX(jc, C, 12)] : 0u);
             }
             if (__any_sync(kFull, imp[0] | imp[1] | imp[2] | imp[3])) {
 #pragma unroll
@@ -373,7 +373,7 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
             for (int t = 0; t + 1 < C; t += 32) {
               const bool l = t + lane + 1 < C && edge[t + lane] > dmin;
               const unsigned m = __ballot_sync(kFull, l);
-              if (l) lng[nl + __popc(m & ((1u << lane) - 1u))] = (uint16_t)(t + lane);
+              if (l) lng[QP_IX(nl + __popc(m & ((1u << lane) - 1u)), C, 12)] = (uint16_t)(t + lane);
               nl += __popc(m);
             }
             __syncwarp();
@@ -381,7 +381,7 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
             lp = 0;
           }
           while (lp < nl) {  // past the edges up to i
-            const unsigned m = __ballot_sync(kFull, lp + lane < nl && lng[lp + lane] <= i);
+            const unsigned m = __ballot_sync(kFull, lp + lane < nl && lng[QP_IX(lp + lane, C, 12)] <= i);
             lp += __popc(m);
             if (m != kFull) break;
           }
@@ -395,9 +395,9 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
 #pragma unroll
               for (int q = 0; q < 4; ++q) {
                 const int l = l0 + 32 * q + lane;
-                j[q] = l < nl ? lng[l] : 0;
-                n1[q] = D(a, path[j[q]]);
-                n2[q] = D(b, path[j[q] + 1]);
+                j[q] = l < nl ? lng[QP_IX(l, C, 12)] : 0;
+                n1[q] = D(a, path[QP_IX(j[q], C, 12)]);
+                n2[q] = D(b, path[QP_IX(j[q] + 1, C, 12)]);
                 imp[q] = j[q] >= j0 && n1[q] + n2[q] < dmin + edge[j[q]];
               }
               if (__any_sync(kFull, imp[0] | imp[1] | imp[2] | imp[3])) {
@@ -425,12 +425,12 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
             uint2 pv[kRun + 1];
             int first[kRun];  // this lane's first improving j for each i
 #pragma unroll
-            for (int q = 0; q <= kRun; ++q) pv[q] = path[min(i - 1 + q, C - 1)];
+            for (int q = 0; q <= kRun; ++q) pv[q] = path[QP_IX(min(i - 1 + q, C - 1), C, 12)];
 #pragma unroll
             for (int q = 0; q < kRun; ++q) first[q] = INT_MAX;
             for (int l0 = lp; l0 < nl; l0 += 32) {
-              const int j = l0 + lane < nl ? lng[l0 + lane] : 0;
-              const uint2 pj = path[j], pj1 = path[j + 1];
+              const int j = l0 + lane < nl ? lng[QP_IX(l0 + lane, C, 12)] : 0;
+              const uint2 pj = path[QP_IX(j, C, 12)], pj1 = path[QP_IX(j + 1, C, 12)];
               const uint32_t lim = dmin + edge[j];
 #pragma unroll
               for (int q = 0; q < kRun; ++q)
@@ -462,10 +462,10 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
         __syncwarp();
         const int len = js - i + 1;
         for (int k = lane; k < len / 2; k += 32) {
-          const uint2 p0 = path[i + k], p1 = path[js - k];
+          const uint2 p0 = path[QP_IX(i + k, C, 12)], p1 = path[QP_IX(js - k, C, 12)];
           const uint16_t i0 = id[i + k], i1 = id[js - k];
           const bool inner = k < (len - 1) / 2;
-          const uint32_t ea = edge[i + k], eb = edge[js - 1 - k];
+          const uint32_t ea = edge[QP_IX(i + k, C, 12)], eb = edge[QP_IX(js - 1 - k, C, 12)];
           path[i + k] = p1;
           path[js - k] = p0;
           id[i + k] = i1;
@@ -477,8 +477,8 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
         }
         __syncwarp();
         if (lane == 0) {
-          edge[i - 1] = n1s;
-          if (js + 1 < C) edge[js] = n2s;
+          edge[QP_IX(i - 1, C, 12)] = n1s;
+          if (js + 1 < C) edge[QP_IX(js, C, 12)] = n2s;
         }
         __syncwarp();
         moved = changed = stale = true;
@@ -490,7 +490,7 @@ __global__ void k_repair_table(const uint8_t *__restrict__ states, int R, int C,
   int32_t *out = paths + (size_t)r * C;
   long long L = 0;
   for (int t = lane; t < C; t += 32) {
-    out[t] = id[t];
+    out[t] = QP_IX((int)id[t], C, 12);
     if (t + 1 < C) L += edge[t];
   }
   L = dev::warp_sum64(L);

@@ -120,7 +120,7 @@ struct Dist {
 #pragma unroll
       for (int j = 0; j < 4; ++j) f[j] += lookup(a, xi[j]);
     } else {
-      const DT *p = m + QP_IX(h, C + 1, 2) * Cp + i;
+      const DT *p = m + QP_IX(h, C + 1, 2) * Cp + QP_RANGE(i, -3, C + 1, 2);
 #pragma unroll
       for (int j = 0; j < 4; ++j) f[j] += QP_VALUE(DM == 1 ? (int)p[j] : (int)__ldg(p + j), 7);
     }
@@ -205,7 +205,7 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
     // the bytes that are set, found 16 at a time
     const uint8_t *x = a.init + (size_t)rep * n;
     auto set = [&](int k) {
-      const int t = k / C, i = k - t * C;
+      const int t = QP_IX(k / C, C, 9), i = k - t * C;
       if (t == 0 || i == s0) return;
       atomicOr(bits + QP_IX(t * Cw + (i >> 5), C * Cw, 3), 1u << (i & 31));
       const int at = (int)(atomicAdd(&rec[t].x, 1u) & 0xFFFFu);
@@ -365,8 +365,8 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
         __syncwarp();
         if (lost) q = record_from_bits<SB>(bits, Cw, C, t, r, lane);
         if (lane == 0) {
-          rec[t] = q;
-          if (r == 1) hx[t] = (uint16_t)D.code((int)(q.x >> 16));
+          rec[QP_RANGE(t, 1, C, 9)] = q;
+          if (r == 1) hx[QP_RANGE(t, 1, C, 9)] = (uint16_t)D.code((int)(q.x >> 16));
         }
         __syncwarp();
       }
@@ -384,10 +384,10 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
       uint32_t xi[4] = {0, 0, 0, 0};
       if (DM == 2) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) xi[j] = D.xy[ic + j];
+        for (int j = 0; j < 4; ++j) xi[j] = D.xy[QP_RANGE(ic + j, -kPad, C + kPad, 10)];
       }
 #pragma unroll
-      for (int j = 0; j < 4; ++j) c[j] = cc[ic + j];
+      for (int j = 0; j < 4; ++j) c[j] = cc[QP_RANGE(ic + j, -kPad, C + kPad, 8)];
       D.add4(p0.c0, ic, xi, f);
       D.add4(p2.c0, ic, xi, f);
       bool x[4];
@@ -464,7 +464,7 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
         ++flips;
         viol += (cm + dlt != 1) - (cm != 1);
         nz += (cm + dlt == 0) - (cm == 0);
-        if (lane == 0) cc[im] = (uint16_t)(cm + dlt);
+        if (lane == 0) cc[QP_IX(im, C, 8)] = (uint16_t)(cm + dlt);
         if (ROWS == kWide && zok) {  // the list of empty columns follows (491 cells: 91.7 -> 90.6 ms)
           if (cm + dlt == 0) {
             if (lane == nz - 1) zreg = im;
@@ -511,7 +511,8 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
     // an empty column, or a survivor; everything else costs dE >= 2A.  sv: whether
     // the row may hold survivors; a block whose draws all bound dE below 2A has none.
     auto event_row = [&](int t, bool sv) {
-      const Row p0 = unpack_row(rec[t - 1]), p1 = unpack_row(rec[t]), p2 = unpack_row(rec[t + 1]);
+      const Row p0 = unpack_row(rec[QP_IX(t - 1, C + 1, 9)]), p1 = unpack_row(rec[QP_IX(t, C + 1, 9)]),
+                p2 = unpack_row(rec[QP_IX(t + 1, C + 1, 9)]);
       const int tC = t * C;
       start_row(p1);
       const uint32_t m1 = (uint32_t)(tC + C - 1) >> 2;
@@ -528,7 +529,7 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
               const int i = min(max(i0 + j, 0), C - 1);
-              z = z || cc[i] == 0;
+              z = z || cc[QP_IX(i, C, 8)] == 0;
             }
             live = __any_sync(kFull, z);
           }
@@ -551,8 +552,8 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
       bool any = false;
 #pragma unroll 4
       for (int t = 1 + lane; t < C; t += 32) {
-        const uint32_t h = hx[t];
-        const int f = D.near(hx[t - 1], h) + (t + 1 < C ? D.near(hx[t + 1], h) : 0);
+        const uint32_t h = hx[QP_IX(t, C, 9)];
+        const int f = D.near(hx[QP_IX(t - 1, C, 9)], h) + (t + 1 < C ? D.near(hx[t + 1], h) : 0);
         any |= twoA - B * f < len;
       }
       quiet = !__any_sync(kFull, any);
@@ -574,7 +575,7 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
         uint32_t un[4];
         int topn[4], dE[4], step[4], code[4];
         draws(tC + C, ((uint32_t)(tC + C) >> 2) + lane, un, topn, std::true_type());
-        const uint2 q3 = rec[min(t + 2, C)];
+        const uint2 q3 = rec[QP_IX(min(t + 2, C), C + 1, 9)];
         start_row(p1);
         const int i0 = 4 * lane - (tC & 3);
         evaluate(t, p0, p1, p2, i0, dE, step, code);
@@ -624,7 +625,7 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
             if (!zok) {  // list the empty columns
               int k = 0;
               for (int i0 = 0; i0 < C && k < nz; i0 += 32) {
-                uint32_t b = __ballot_sync(kFull, i0 + lane < C && cc[i0 + lane] == 0);
+                uint32_t b = __ballot_sync(kFull, i0 + lane < C && cc[QP_IX(i0 + lane, C, 8)] == 0);
                 while (b) {
                   if (lane == k) zreg = i0 + __ffs(b) - 1;
                   b &= b - 1;
@@ -637,11 +638,12 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
             const int tl = t0 + lane;
             const bool in = tl >= t && tl < t1;
             const int tr = min(tl, C - 1);
-            const Row p0 = unpack_row(rec[tr - 1]), p1 = unpack_row(rec[tr]), p2 = unpack_row(rec[tr + 1]);
+            const Row p0 = unpack_row(rec[QP_IX(tr - 1, C + 1, 9)]), p1 = unpack_row(rec[QP_IX(tr, C + 1, 9)]),
+                      p2 = unpack_row(rec[QP_IX(tr + 1, C + 1, 9)]);
             bool ev = p1.n != 1 || p0.n > 1 || p2.n > 1 || ((smask >> lane) & 1u);
             const int h = p1.c0;
             int dE = len;
-            if (in && !ev) dE = twoA * (2 - (int)cc[h]) - B * (D(p0.c0, h) + D(p2.c0, h));
+            if (in && !ev) dE = twoA * (2 - (int)cc[QP_IX(h, C, 8)]) - B * (D(p0.c0, h) + D(p2.c0, h));
             bool need = dE < len;
             if (__any_sync(kFull, need)) {
               hit = true;
@@ -692,14 +694,14 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
     const Row q = unpack_row(rec[t]);
     uint8_t *o = out + (size_t)t * C;
     if (q.n <= kRowCells) {
-      if (q.n > 0) o[q.c0] = 1;
-      if (q.n > 1) o[q.c1] = 1;
-      if (q.n > 2) o[q.c2] = 1;
+      if (q.n > 0) o[QP_IX(q.c0, C, 11)] = 1;
+      if (q.n > 1) o[QP_IX(q.c1, C, 11)] = 1;
+      if (q.n > 2) o[QP_IX(q.c2, C, 11)] = 1;
     } else {
       for (int w = 0; w < Cw; ++w) {
         uint32_t wd = bits_word<SB>(bits + t * Cw + w);
         while (wd) {
-          o[(w << 5) + __ffs(wd) - 1] = 1;
+          o[QP_IX((w << 5) + __ffs(wd) - 1, C, 11)] = 1;
           wd &= wd - 1;
         }
       }

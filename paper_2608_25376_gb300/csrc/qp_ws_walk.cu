@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(32) k_ws_walk(const int32_t *d, int C, int sta
       best = key < best ? key : best;
     }
     best = warp_min_u64(best);
-    const int nxt = (int)(best & 0xFFFu);
+    const int nxt = QP_IX((int)(best & 0xFFFu), C, 11);
     L += __ldg(row + nxt);
     if (lane == 0) {
       vis[nxt >> 5] |= 1u << (nxt & 31);
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(32) k_ws_walk(const int32_t *d, int C, int sta
     cur = nxt;
   }
   for (int t = lane; t < C; t += 32) {
-    const int i = pth[t];
+    const int i = QP_IX(pth[t], C, 11);
     if (path) path[t] = i;
     if (state) state[(size_t)t * C + i] = 1;
   }
@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kWalkThreads)
 #pragma unroll 4
       for (int j = 0; j < C; ++j) r += skey[j] < k || (skey[j] == k && j < i);
       place[i] = (uint16_t)r;
-      at[r] = make_uint2((uint32_t)(cxy[i] >> 8) << sh, (uint32_t)i << 16 | (cxy[i] & 0xFFu));
+      at[QP_IX(r, C, 11)] = make_uint2((uint32_t)(cxy[i] >> 8) << sh, (uint32_t)i << 16 | (cxy[i] & 0xFFu));
     }
     __syncthreads();
   }
@@ -198,11 +198,11 @@ __global__ void __launch_bounds__(kWalkThreads)
       uint32_t best = 0xFFFFFFFFu;
 #pragma unroll
       for (int q = 0; q < K; ++q) {
-        const uint32_t key = (uint32_t)(int)tb[__usad(ccol, col[q], __usad(crow, row[q], 0u))] << kWalkRankBits | pl[q];
+        const uint32_t key = (uint32_t)(int)tb[QP_IX((int)__usad(ccol, col[q], __usad(crow, row[q], 0u)), tab_n, 2)] << kWalkRankBits | pl[q];
         best = (open >> q) & 1u ? min(best, key) : best;
       }
       best = __reduce_min_sync(kFull, best);
-      const uint2 w = at[best & ((1u << kWalkRankBits) - 1u)];
+      const uint2 w = at[QP_IX((int)(best & ((1u << kWalkRankBits) - 1u)), C, 11)];
       const uint32_t id = w.y >> 16;
       crow = w.x;
       ccol = w.y & 0xFFFFu;
@@ -229,7 +229,7 @@ __global__ void __launch_bounds__(kWalkThreads)
 #pragma unroll
       for (int q = 0; q < K; ++q) {
         const uint32_t ad = __vabsdiffu4(cur, c[q]);
-        const uint32_t v = (uint32_t)(int)tb[((ad >> 8) << sh) + (ad & 0xFFu)];
+        const uint32_t v = (uint32_t)(int)tb[QP_IX((int)(((ad >> 8) << sh) + (ad & 0xFFu)), tab_n, 2)];
         d[q] = (open >> q) & 1u ? v : 0xFFFFFFFFu;
         dmin = min(dmin, d[q]);
       }
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(kWalkThreads)
 #pragma unroll
       for (int q = K - 1; q >= 0; --q) id = d[q] == win ? (uint32_t)(lane + 32 * q) : id;
       id = __reduce_min_sync(kFull, id);
-      cur = cxy[id];
+      cur = cxy[QP_IX((int)id, C, 10)];
       L += win;
       if (lane == (int)(id & 31)) open &= ~(1u << (id >> 5));
       if (lane == 0) pth[t] = (int)id;
@@ -259,7 +259,7 @@ __global__ void __launch_bounds__(kWalkThreads)
   }
   __syncthreads();
   for (int t = tid; t < C; t += kWalkThreads) {
-    const int i = pth[t];
+    const int i = QP_IX(pth[t], C, 11);
     if (path) path[t] = i;
     if (state) state[(size_t)t * C + i] = 1;
   }
@@ -434,3 +434,9 @@ extern "C" qp_status qp_ws_greedy(const float *logits, int32_t ld, int32_t C, in
   if (e != cudaSuccess) return set_error(QP_ECUDA, cudaGetErrorString(e));
   return QP_OK;
 }
+
+namespace qp {
+namespace chk {
+QP_CHECK_ACCESSOR(walk)
+}  // namespace chk
+}  // namespace qp

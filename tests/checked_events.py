@@ -1,9 +1,10 @@
-"""Cases of the event-driven sweep for the checked build of the library: every
-place its distances can be read from (matrix in shared memory, table of grid
+"""Cases of the event-driven sweep, the repair, the walk and the decode for the
+checked build of the library.  The sweep: every place its distances can be read from (matrix in shared memory, table of grid
 differences, matrix in global memory), both distance types, row lengths that
 fill the padded row and that do not, rows of one and of several blocks, states
-from nothing and from many cells, single fields and batches.  Each is compared
-with the CPU oracle, then the library's record of failed checks must be empty:
+from nothing and from many cells, single fields and batches.  The others: with
+and without a distance table, states that are no paths.  Each is compared with
+the CPU reference, then the library's record of failed checks must be empty:
 no index outside its array, and no distance from an entry that nothing wrote.
 Run by tests/test_gpu_device_checks_events.py in a fresh interpreter with
 QPATH_LIBRARY pointing at the checked library; prints one JSON line and exits
@@ -20,6 +21,7 @@ sys.path.insert(0, ROOT)
 import torch  # noqa: E402
 
 import oracle  # noqa: E402
+from oracle import mlp_ref, repair_ref  # noqa: E402
 from paper_2608_25376_gb300 import inputs, qpath  # noqa: E402
 
 
@@ -104,6 +106,55 @@ def batches(results):
                 for s, e, r in zip(sts, Es, refs))
 
 
+# Field and scale of the repair, the walk and the decode; "none": too wide for a distance table.
+PATHS = {
+    "2": (inputs.rect(1, 2), 100), "33": (strip(7, 7, 33), 100), "64-i32": (strip(9, 9, 64), 20000),
+    "129": (strip(12, 13, 129), 100), "none-90": (strip(1, 300, 90), 100), "300": (strip(18, 18, 300), 100),
+    "513": (strip(24, 24, 513), 100),
+}
+
+
+def paths(results):
+    stream = torch.cuda.current_stream()
+    for name, (f, scale) in PATHS.items():
+        h = qpath.qp_build_qubo(f, scale=scale)
+        C = h.info["C"]
+        d = qpath.qp_export_dist(h)
+        start = int(np.cumsum(f.free_mask)[f.start] - 1)
+        rng = np.random.default_rng(C)
+        # a path, one with a few cells flipped, random cells, no cell
+        X = np.zeros((4, C, C), np.uint8)
+        X[:2, np.arange(C), np.r_[start, rng.permutation([i for i in range(C) if i != start])].astype(int)] = 1
+        X[1] ^= (rng.random((C, C)) < 1.0 / C).astype(np.uint8)
+        X[2] = rng.random((C, C)) < 3.0 / C
+        st = torch.from_numpy(X.reshape(4, -1)).cuda()
+        p = torch.zeros((4, C), dtype=torch.int32, device="cuda")
+        n = torch.zeros(4, dtype=torch.int64, device="cuda")
+        s = torch.zeros(4, dtype=torch.int32, device="cuda")
+        qpath.qp_decode_batch(h, 4, st, p, n, stream=stream)
+        torch.cuda.synchronize()
+        on = X != 0
+        cells = np.where(on.any(2), C - 1 - on[:, :, ::-1].argmax(2), -1)
+        ok = (on.sum(1) == 1).all(1) & (on.sum(2) == 1).all(1)
+        lengths = np.where(ok, d[cells[:, :-1], cells[:, 1:]].astype(np.int64).sum(1), -1)
+        results[f"decode-{name}"] = bool((p.cpu().numpy() == cells).all() and (n.cpu().numpy() == lengths).all())
+        passes = -1 if C < 100 else 1  # the reference takes C^3 a pass
+        good = True
+        if C <= 300:
+            qpath.qp_repair_batch(h, 4, st, passes, p, n, s, stream=stream)
+            torch.cuda.synchronize()
+            for r in range(4):
+                path, length, status = repair_ref.repair(X[r].reshape(-1).tolist(), d.tolist(), C, start, passes)
+                good &= p[r].cpu().tolist() == path and int(n[r]) == length and int(s[r]) == status
+            results[f"repair-{name}"] = bool(good)
+        for score, slack in ((None, 0), (rng.normal(0, 5, C).astype(np.float32), 0),
+                             (rng.normal(0, 5, C).astype(np.float32), 2 * scale)):
+            _, path, ln = qpath.qp_ws_walk(h, None if score is None else torch.from_numpy(score).cuda(), slack)
+            torch.cuda.synchronize()
+            ref = mlp_ref.walk(d, C, start, score, slack)
+            results[f"walk-{name}-{slack}-{score is None}"] = path.cpu().numpy().tolist() == ref
+
+
 def main():
     assert os.environ.get("QPATH_LIBRARY"), "run with QPATH_LIBRARY set to the checked build"
     assert qpath.qp_device_checks()[0], "the loaded library was built without device checks"
@@ -111,6 +162,7 @@ def main():
     results = {}
     singles(results)
     batches(results)
+    paths(results)
     enabled, first_failure = qpath.qp_device_checks()
     print(json.dumps({"enabled": enabled, "first_failure": first_failure, "results": results}))
     return 0 if enabled and first_failure == 0 and all(v is True for v in results.values()) else 1
