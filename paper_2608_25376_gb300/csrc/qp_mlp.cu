@@ -3,10 +3,11 @@
 // cross-entropy on the annealer's own best paths.
 //
 // The forward pass of all four layers runs as one kernel (k_mlp_forward, the
-// activations of a 128-cell tile kept in shared memory between layers).
-// Every other matrix product (dX = dY W, dW = dY^T X, and the forward as four
-// separate launches when asked) runs on one tcgen05
-// kernel: D[M x N] (+)= A[M x K] B[N x K]^T with bf16 operands (both K-major,
+// activations of a 128-cell tile kept in shared memory between layers), and so
+// do the three products dX = dY W of the backward pass (k_mlp_backward).  Every
+// other matrix product (dW = dY^T X, and the forward as four separate launches
+// when asked) runs on one tcgen05 kernel (k_gemm_tc): D[M x N] = A[M x K]
+// B[N x K]^T with bf16 operands (both K-major,
 // i.e. K contiguous) and fp32 accumulation in tensor memory.  A CTA owns a
 // 128 x N tile (N <= 256, multiple of 16) and walks K in chunks of 64 through
 // two shared-memory stages: one thread has the tensor-memory-access engine
@@ -17,9 +18,9 @@
 // chunk after next; the load of chunk c+1 overlaps the MMAs of chunk c.
 // Every wait is bounded.  The epilogue reads the accumulator back with
 // tcgen05.ld (warp w owns TMEM lanes 32w..32w+31 = rows of the tile), applies
-// bias/ReLU/masking and stages the rows in the freed stages, so that the
-// stores (and the ReLU reference loads) cover whole sectors.  Split-K partial
-// tiles are added into an fp32 output with atomics.
+// bias and ReLU and stages the rows in the freed stages, so that the stores
+// cover whole sectors.  Split-K partial tiles are stored per split; k_sums adds
+// them in index order.
 #include <cuda.h>  // CUtensorMap and the tile-encoder types; the encoder comes from the runtime
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -310,17 +311,6 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ GemmGro
       }
       __syncwarp();
       const int cl = 4 * (lane & 15);  // this lane's 4 columns of the block
-      // the ReLU reference of the lane's 16 (row, 4-column) pieces, all loads in flight at once
-      uint2 rref[16];
-      if (g.mode == kEpiReluMask) {
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-          const int row = row0 + 2 * q + (lane >> 4);
-          rref[q] = (cl < nb && row < g.M)
-                        ? *reinterpret_cast<const uint2 *>(g.relu_ref + (size_t)row * g.ldr + c0 + cl)
-                        : make_uint2(0u, 0u);
-        }
-      }
 #pragma unroll
       for (int rr = 0; rr < 32; rr += 2) {
         const int r = rr + (lane >> 4), row = row0 + r;
@@ -332,17 +322,7 @@ __global__ void __launch_bounds__(128) k_gemm_tc(const __grid_constant__ GemmGro
         } else if (g.mode == kEpiPartialF32) {
           *reinterpret_cast<float4 *>(g.out_f32 + (size_t)blockIdx.z * g.M * g.ldo + (size_t)row * g.ldo + col) = x;
         } else {
-          float a = x.x, b = x.y, c = x.z, e = x.w;
-          if (g.mode == kEpiReluMask) {  // gradient through the ReLU of the stored activation
-            const uint2 rq = rref[rr >> 1];
-            const __nv_bfloat162 r01 = *reinterpret_cast<const __nv_bfloat162 *>(&rq.x);
-            const __nv_bfloat162 r23 = *reinterpret_cast<const __nv_bfloat162 *>(&rq.y);
-            a = __low2float(r01) > 0.0f ? a : 0.0f;
-            b = __high2float(r01) > 0.0f ? b : 0.0f;
-            c = __low2float(r23) > 0.0f ? c : 0.0f;
-            e = __high2float(r23) > 0.0f ? e : 0.0f;
-          }
-          const __nv_bfloat162 o01 = __floats2bfloat162_rn(a, b), o23 = __floats2bfloat162_rn(c, e);
+          const __nv_bfloat162 o01 = __floats2bfloat162_rn(x.x, x.y), o23 = __floats2bfloat162_rn(x.z, x.w);
           uint2 oq;
           oq.x = *reinterpret_cast<const uint32_t *>(&o01);
           oq.y = *reinterpret_cast<const uint32_t *>(&o23);
@@ -1096,8 +1076,7 @@ cudaError_t gemm(const GemmArgs *g, int count, int splits, cudaStream_t st) {
   int zs = 0, tiles = 0;
   for (int k = 0; k < count; ++k) {
     const GemmArgs &a = g[k];
-    if (a.N < 16 || a.N > 256 || (a.N & 15) || (a.K & 15) || (a.lda & 7) || (a.ldb & 7) || (a.ldo & 3) ||
-        (a.mode == kEpiReluMask && (a.ldr & 3)))
+    if (a.N < 16 || a.N > 256 || (a.N & 15) || (a.K & 15) || (a.lda & 7) || (a.ldb & 7) || (a.ldo & 3))
       return cudaErrorInvalidValue;
     if (!tile_map(&grp.a[k], a.A, a.M, a.K, a.lda, kTileM) || !tile_map(&grp.b[k], a.B, a.N, a.K, a.ldb, a.N))
       return cudaErrorInvalidValue;

@@ -11,11 +11,10 @@ namespace mlp {
 enum EpiMode {
   kEpiBiasRelu = 0,   // out_bf16 = bf16(relu(acc + bias))
   kEpiBiasF32 = 1,    // out_f32 = acc + bias
-  kEpiPartialF32 = 4, // out_f32 + z * M * ldo = acc for split z (sum_splits adds them in order)
-  kEpiReluMask = 3,   // out_bf16 = bf16(relu_ref > 0 ? acc : 0)
+  kEpiPartialF32 = 2, // out_f32 + z * M * ldo = acc for split z (sum_jobs adds them in order)
 };
 
-// D[M x N] (+)= A[M x K] B[N x K]^T; A, B bf16 row-major with K contiguous.
+// D[M x N] = A[M x K] B[N x K]^T; A, B bf16 row-major with K contiguous.
 // N in [16, 256] and a multiple of 16; K, lda, ldb multiples of 16 / 8.
 struct GemmArgs {
   const __nv_bfloat16 *A;
@@ -29,8 +28,6 @@ struct GemmArgs {
   float *out_f32;
   __nv_bfloat16 *out_bf16;
   int ldo;
-  const __nv_bfloat16 *relu_ref;
-  int ldr;
   int *err;  // set to 1 if a bounded wait gave up
 };
 
