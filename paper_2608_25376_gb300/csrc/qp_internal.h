@@ -44,8 +44,9 @@ struct StructArgs {
   int64_t *E_out, *best_out, *acc_out;  // best/acc may be null
   uint32_t *gstate;          // R x nw_pad words when the state lives in global memory
   int32_t nw_pad;
-  // Replica exchange: the table row replica r (local index) uses in every
-  // sweep of the launch (its ladder level); null = row s for sweep s.
+  // Replica exchange (event-driven kernel only): the table row replica r (local
+  // index) uses in every sweep of the launch (its ladder level); null = row s
+  // for sweep s.
   const int32_t *level;
   // QP_ANNEAL_SKIP_SETTLED: skip sweeps that provably change nothing
   int32_t skip_settled;

@@ -65,7 +65,6 @@ __device__ __forceinline__ void rows_replica(const StructArgs &a, int r, uint32_
   long long best = LLONG_MAX, acc = 0;
 
   // ---- sweeps
-  const int lev = a.level ? __ldg(a.level + r) : -1;
   // A sweep that met no proposal with dE < len leaves the state as it was, so
   // every later sweep with a table no longer than len does too (each of its
   // proposals sees the same state and the same dE): those sweeps are skipped
@@ -73,18 +72,17 @@ __device__ __forceinline__ void rows_replica(const StructArgs &a, int r, uint32_
   bool settled = false;
   int settled_len = 0;
   for (int s = a.sweep_begin; s < a.sweep_end; ++s) {
-    const int ts = lev >= 0 ? lev : s;  // table row: the sweep, or the replica's ladder level
-    const uint32_t *thr = a.thr + a.thr_off[ts];
-    const int len = a.thr_len[ts];
+    const uint32_t *thr = a.thr + a.thr_off[s];
+    const int len = a.thr_len[s];
     if (settled && len <= settled_len) continue;
     bool any_hit = false;
     const unsigned lenm1 = (unsigned)(len - 1);
-    const float cT = a.thr_c[ts];
+    const float cT = a.thr_c[s];
     // quick rejection: a draw u >= thr[dq] rejects every dE >= dq (thr is
     // non-increasing); dq ~ 8 T ln 2 puts thr[dq] near 2^24, so almost every
     // draw of a proposal with dE >= dq is rejected by two compares
     const int dq = len > 1 ? min(len - 1, max(1, (int)fminf(8.0f / cT, 1.0e9f))) : 1;
-    const uint32_t Q = len > 1 ? __ldg(a.thr + a.thr_off[ts] + dq) : 0u;
+    const uint32_t Q = len > 1 ? __ldg(a.thr + a.thr_off[s] + dq) : 0u;
     // P, Cu, N: the fields of rows t-1, t, t+1; N1 (and N2 when LA = 2): rows
     // t+2 (and t+3).  Row t+1+LA's field is loaded LA rows ahead of its use, so
     // an L2 read of d (LA = 2 when d is in global memory) has that many rows of
@@ -439,19 +437,17 @@ __device__ __forceinline__ void rows_replica_g(const StructArgs &a, int r, uint3
   rows_init<DT, NCH, 0, true>(a, r, st, hot, d, lane, tAc, validc, E, viol, !fresh);
   int tl = 0;  // tAc holds 2A c_i - tl (shifted by the sweep's table length)
 
-  const int lev = a.level ? __ldg(a.level + r) : -1;
   bool settled = false;
   int settled_len = 0;
   for (int s = sb; s < se; ++s) {
-    const int ts = lev >= 0 ? lev : s;
-    const uint32_t *thr = a.thr + a.thr_off[ts];
-    const int len = a.thr_len[ts];
+    const uint32_t *thr = a.thr + a.thr_off[s];
+    const int len = a.thr_len[s];
     if (settled && len <= settled_len) continue;
     bool any_hit = false;
     const unsigned lenm1 = (unsigned)(len - 1);
-    const float cT = a.thr_c[ts];
+    const float cT = a.thr_c[s];
     const int dq = len > 1 ? min(len - 1, max(1, (int)fminf(8.0f / cT, 1.0e9f))) : 1;
-    const uint32_t Q = len > 1 ? __ldg(a.thr + a.thr_off[ts] + dq) : 0u;
+    const uint32_t Q = len > 1 ? __ldg(a.thr + a.thr_off[s] + dq) : 0u;
     if (len != tl) {  // tAc holds 2A c_i - len for this sweep's len
 #pragma unroll
       for (int c = 0; c < NCH; ++c)
