@@ -69,7 +69,8 @@ typedef enum {
  * buffer it could not allocate, and leaves the handle usable.  Failure
  * injection for tests: with the environment variable QPATH_FAIL_ALLOC = N the
  * library's next N device allocations succeed and every later one fails
- * (QP_ENOMEM), until the variable changes or is removed. */
+ * (QP_ENOMEM), until the variable changes or is removed; with
+ * QPATH_FAIL_ALLOC_OVER = N every allocation of more than N bytes fails. */
 
 typedef struct qp_handle qp_handle;
 

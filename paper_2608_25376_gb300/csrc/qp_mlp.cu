@@ -163,7 +163,8 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols) {
 // before it lets the next kernel start, so that completion is transitive.
 // What an earlier kernel of the pass wrote is not read through the read-only
 // path, which wants it unchanged while the kernel lives, its early start included.
-// 16384-cell forward call 71.7 -> 66.7 us, a training step of 8000 rows 173 -> 161.
+// 16384-cell forward call 71.7 -> 66.7 us, a training step of 8000 rows 173 -> 161
+// (in turn on one machine; others give 67-72 us for the call as it is).
 __device__ __forceinline__ void pdl_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -195,7 +195,7 @@ __global__ void k_repair(const uint8_t *__restrict__ states, int R, int C, int s
 //   So at an i whose edge e1 is dmin only the j whose edge is longer than dmin
 //   can improve: those are kept as a list in path order (rebuilt after a move),
 //   the others are passed over.  On a good path most edges are dmin.
-// 1024 states of 491 cells, 2-opt to the end (1500 moves a state): 13.9 -> 3.6 ms
+// 1024 states of 491 cells, 2-opt to the end (1500 moves a state): 13.1-13.9 -> 3.6-3.7 ms
 // (5.3 with one list entry per lane and one i at a time). What is left is the
 // chain of dependent steps: ~400 cycles a move, ~500-1000 a scan.
 constexpr int kRun = 4;  // consecutive i scanned at once

@@ -123,7 +123,7 @@ __global__ void __launch_bounds__(32) k_ws_walk(const int32_t *d, int C, int sta
   if (lane == 0 && length) *length = L;
 }
 
-// The walk of a field of up to 32 K cells whose distances fit a table over the
+// The walk of a field of up to 32 * K cells (K a template argument) whose distances fit a table over the
 // grid differences (kernel arguments as StructArgs).  A step's chain is what
 // takes the time: with d read from L2 twice a step it was 2.8 us.  Here lane L
 // of warp 0 keeps the cells L + 32 q, their coordinates, score codes and whether
