@@ -289,13 +289,11 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
     viol = __reduce_add_sync(kFull, v);
     nz = __reduce_add_sync(kFull, z);
   }
-  // The energy (Eqs. 3-6) of the state without cells but the clamped one: its C - 1
-  // empty rows and columns.  From a given state energies are kept relative to its
-  // until the end, and the last state's is summed there: it rarely has rows of many
-  // cells, and summed over an initial state with half its cells set it took longer
-  // than the sweeps (230 cells, 256 chains, one sweep: 31.0 -> 15.9 ms; 491 cells
-  // 233 -> 110).
-  long long E = a.init ? 0 : 2LL * a.A * (C - 1);
+  // Energies are kept relative to the initial state's until the end: the last
+  // state's is summed there (it rarely has rows of many cells; summed over an
+  // initial state with half its cells set it took longer than the sweeps: 230
+  // cells, 256 chains, one sweep: 31.0 -> 15.9 ms; 491 cells 233 -> 110).
+  long long E = 0;
   long long best = LLONG_MAX, acc = 0;
   int zreg = 0;          // lane q < nz: an empty column (when zok)
   bool zok = false;
@@ -697,9 +695,8 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
     settled_len = len;
   }
 
-  // ---- from a given state, the last state's energy
-  if (!a.init) {
-  } else if (ROWS == kWide && !SB) {
+  // ---- the last state's energy (Eqs. 3-6)
+  if (ROWS == kWide && !SB) {
     const long long last = state_energy<DT, DM, SB>(a, rec, cc, bits, D, lane);
     if (best != LLONG_MAX) best += last - E;
     E = last;
