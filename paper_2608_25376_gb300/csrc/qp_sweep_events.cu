@@ -178,38 +178,6 @@ __device__ __forceinline__ uint2 record_from_bits(const uint32_t *bits, int Cw, 
   return pack_row(r, c[0], c[1], c[2]);
 }
 
-// The energy (Eqs. 3-6) of the state that the records, bits and column sums hold,
-// as a call, for wide rows with their bits in global memory: inlined it costs
-// their sweeps 1% (893 cells 22.1 -> 22.3 ms); called it costs the batch as much.
-template <typename DT, int DM, bool SB>
-__device__ __noinline__ long long state_energy(const StructArgs &a, const uint2 *rec, const uint16_t *cc, const uint32_t *bits,
-                                               const Dist<DT, DM> &D, int lane) {
-  const int C = a.C, Cw = (C + 31) >> 5;
-  long long hd = 0, pen = 0;
-  for (int t = lane; t < C; t += 32) {
-    const Row q = unpack_row(rec[QP_IX(t, C, 9)]);
-    pen += (long long)(1 - q.n) * (1 - q.n);
-    if (t + 1 < C && q.n > 0) {
-      const Row p = unpack_row(rec[t + 1]);
-      if (q.n <= kRowCells) {
-        hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c0);
-        if (q.n > 1) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c1);
-        if (q.n > 2) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c2);
-      } else {
-        for (int w = 0; w < Cw; ++w) {
-          uint32_t wd = bits_word<SB>(bits + QP_IX(t * Cw + w, C * Cw, 3));
-          while (wd) {
-            hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, (w << 5) + __ffs(wd) - 1);
-            wd &= wd - 1;
-          }
-        }
-      }
-    }
-  }
-  for (int i = lane; i < C; i += 32) pen += (long long)(1 - (int)cc[i]) * (1 - (int)cc[i]);
-  return (long long)a.B * warp_sum64(hd) + (long long)a.A * warp_sum64(pen);
-}
-
 // The sweeps of one replica.  rec: C + 1 row records (the last stays empty),
 // hx: what D.near needs of the cell of a row that holds one, cc:
 // column sums with kPad entries on both sides, bits: C x Cw words.
@@ -271,13 +239,36 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
       if ((rec[t].x & 0xFFFFu) == 0) rec[t] = pack_row(0, C, 0, 0);
     __syncwarp();
   }
-  // ---- violation count, empty columns
+  // ---- energy (Eqs. 3-6), violation count, empty columns
+  long long E;
   int viol, nz;
   {
+    long long hd = 0, pen = 0;
     int v = 0, z = 0;
-    for (int t = lane; t < C; t += 32) v += (rec[t].x & 0xFFFFu) != 1;
+    for (int t = lane; t < C; t += 32) {
+      const Row q = unpack_row(rec[t]);
+      pen += (long long)(1 - q.n) * (1 - q.n);
+      v += q.n != 1;
+      if (a.init && t + 1 < C && q.n > 0) {
+        const Row p = unpack_row(rec[t + 1]);
+        if (q.n <= kRowCells) {
+          hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c0);
+          if (q.n > 1) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c1);
+          if (q.n > 2) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c2);
+        } else {
+          for (int w = 0; w < Cw; ++w) {
+            uint32_t wd = bits_word<SB>(bits + t * Cw + w);
+            while (wd) {
+              hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, (w << 5) + __ffs(wd) - 1);
+              wd &= wd - 1;
+            }
+          }
+        }
+      }
+    }
     for (int i = lane; i < C; i += 32) {
       const int c = cc[i];
+      pen += (long long)(1 - c) * (1 - c);
       v += c != 1;
       z += c == 0;
     }
@@ -286,14 +277,10 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
       hx[t] = (uint16_t)D.code(min(h, C - 1));
     }
     __syncwarp();
+    E = (long long)B * warp_sum64(hd) + (long long)a.A * warp_sum64(pen);
     viol = __reduce_add_sync(kFull, v);
     nz = __reduce_add_sync(kFull, z);
   }
-  // Energies are kept relative to the initial state's until the end: the last
-  // state's is summed there (it rarely has rows of many cells; summed over an
-  // initial state with half its cells set it took longer than the sweeps: 230
-  // cells, 256 chains, one sweep: 31.0 -> 15.9 ms; 491 cells 233 -> 110).
-  long long E = 0;
   long long best = LLONG_MAX, acc = 0;
   int zreg = 0;          // lane q < nz: an empty column (when zok)
   bool zok = false;
@@ -695,38 +682,6 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
     settled_len = len;
   }
 
-  // ---- the last state's energy (Eqs. 3-6)
-  if (ROWS == kWide && !SB) {
-    const long long last = state_energy<DT, DM, SB>(a, rec, cc, bits, D, lane);
-    if (best != LLONG_MAX) best += last - E;
-    E = last;
-  } else {
-    long long hd = 0, pen = 0;
-    for (int t = lane; t < C; t += 32) {
-      const Row q = unpack_row(rec[t]);
-      pen += (long long)(1 - q.n) * (1 - q.n);
-      if (t + 1 < C && q.n > 0) {
-        const Row p = unpack_row(rec[t + 1]);
-        if (q.n <= kRowCells) {
-          hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c0);
-          if (q.n > 1) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c1);
-          if (q.n > 2) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c2);
-        } else {
-          for (int w = 0; w < Cw; ++w) {
-            uint32_t wd = bits_word<SB>(bits + t * Cw + w);
-            while (wd) {
-              hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, (w << 5) + __ffs(wd) - 1);
-              wd &= wd - 1;
-            }
-          }
-        }
-      }
-    }
-    for (int i = lane; i < C; i += 32) pen += (long long)(1 - (int)cc[i]) * (1 - (int)cc[i]);
-    const long long last = (long long)B * warp_sum64(hd) + (long long)a.A * warp_sum64(pen);
-    if (best != LLONG_MAX) best += last - E;
-    E = last;
-  }
   // ---- outputs: zeros in 16-byte stores, then the cells
   uint8_t *out = a.states_out + (size_t)rep * n;
   const int head = min(n, (int)((16 - (reinterpret_cast<uintptr_t>(out) & 15)) & 15));
