@@ -156,6 +156,104 @@ __device__ __forceinline__ int row_sum_d(const Row &q, int u, const uint32_t *bi
   return f;
 }
 
+// Sums of d over the cells of row t (their number n; more than three, so the
+// bits hold them), of the cells but `skip`, for this lane's columns i .. i + 3
+// (-4 < i; a multiple of 4 below Cp when ALIGNED): by the whole warp, from the
+// matrix in global memory, eight cells' rows in flight at a time.
+template <typename DT, bool SB, bool ALIGNED>
+__device__ __forceinline__ void add_cells(const DT *d, int Cp, int C, const uint32_t *bits, int Cw, int t, int n, int skip,
+                                          int i, int lane, int (&f)[4]) {
+  uint32_t word = 0, left = 0, wd = 0;
+  int w0 = -32, w = 0;
+  auto next = [&]() {  // the next cell, C (the row of zeros) after the last
+    while (wd == 0) {
+      if (left == 0) {
+        w0 += 32;
+        if (w0 >= Cw) return C;
+        word = w0 + lane < Cw ? bits_word<SB>(bits + QP_IX(t * Cw + w0 + lane, C * Cw, 3)) : 0u;
+        if ((skip >> 5) == w0 + lane) word &= ~(1u << (skip & 31));
+        left = __ballot_sync(kFull, word != 0);
+        continue;
+      }
+      w = w0 + __ffs(left) - 1;
+      left &= left - 1;
+      wd = __shfl_sync(kFull, word, w - w0);
+    }
+    const int h = (w << 5) + __ffs(wd) - 1;
+    wd &= wd - 1;
+    return h;
+  };
+  for (int k = 0; k < n; k += 8) {
+    const DT *p[8];
+#pragma unroll
+    for (int g = 0; g < 8; ++g) p[g] = d + (size_t)QP_IX(next(), C + 1, 2) * Cp + i;
+    DT v[8][4];
+#pragma unroll
+    for (int g = 0; g < 8; ++g) {
+      if (!ALIGNED) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[g][j] = __ldg(p[g] + j);
+      } else if (sizeof(DT) == 2) {
+        *reinterpret_cast<int2 *>(v[g]) = __ldg(reinterpret_cast<const int2 *>(p[g]));
+      } else {
+        *reinterpret_cast<int4 *>(v[g]) = __ldg(reinterpret_cast<const int4 *>(p[g]));
+      }
+    }
+#pragma unroll
+    for (int g = 0; g < 8; ++g)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) f[j] += (int)v[g][j];
+  }
+}
+
+// This lane's part of the sum of d over the pairs of a cell of row t and one of
+// row t + 1, by the whole warp.  (A lane per row, cell by cell, the energy of a state
+// with half its cells set was the larger part of a short anneal from it: 230 cells,
+// 256 chains, one sweep 31.0 -> 20.7 ms.)
+template <typename DT, bool SB>
+__device__ __forceinline__ long long pair_distance(const DT *d, int Cp, int C, const uint32_t *bits, int Cw, const uint2 *rec,
+                                                int t, int lane) {
+  const Row q = unpack_row(rec[t]), p = unpack_row(rec[t + 1]);
+  long long sum = 0;
+  for (int b = 0; b < Cp; b += 128) {
+    const int i = b + 4 * lane, i0 = min(i, Cp - 4);
+    int f[4] = {0, 0, 0, 0};
+    if (p.n <= kRowCells) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        f[j] = (int)__ldg(d + (size_t)p.c0 * Cp + i0 + j);
+        if (p.n > 1) f[j] += (int)__ldg(d + (size_t)p.c1 * Cp + i0 + j);
+        if (p.n > 2) f[j] += (int)__ldg(d + (size_t)p.c2 * Cp + i0 + j);
+      }
+    } else {
+      add_cells<DT, SB, true>(d, Cp, C, bits, Cw, t + 1, p.n, -1, i0, lane, f);
+    }
+    uint32_t x = 0;  // row t's cells among the four
+    if (q.n > kRowCells) {
+      x = bits_word<SB>(bits + QP_IX(t * Cw + (min(i0, C - 1) >> 5), C * Cw, 3)) >> (i0 & 31);
+    } else {
+      if ((unsigned)(q.c0 - i0) < 4u) x |= 1u << (q.c0 - i0);
+      if (q.n > 1 && (unsigned)(q.c1 - i0) < 4u) x |= 1u << (q.c1 - i0);
+      if (q.n > 2 && (unsigned)(q.c2 - i0) < 4u) x |= 1u << (q.c2 - i0);
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (i < Cp && i0 + j < C && ((x >> j) & 1u)) sum += f[j];
+  }
+  return sum;
+}
+
+// The same for every two rows whose numbers of cells multiply to more than `most`.
+template <typename DT, bool SB>
+__device__ __noinline__ long long pairs_distance(const DT *d, int Cp, int C, const uint32_t *bits, int Cw, const uint2 *rec,
+                                                 int most, int lane) {
+  long long sum = 0;
+  for (int t = 0; t + 1 < C; ++t)
+    if ((int)(rec[t].x & 0xFFFFu) * (int)(rec[t + 1].x & 0xFFFFu) > most)
+      sum += pair_distance<DT, SB>(d, Cp, C, bits, Cw, rec, t, lane);
+  return sum;
+}
+
 // Row t's record from its bits (r cells); of a row with more than three, one
 // of its cells.
 template <bool SB>
@@ -245,13 +343,19 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
   {
     long long hd = 0, pen = 0;
     int v = 0, z = 0;
+    // Rows t and t + 1 of many cells: their pairs by the whole warp (pair_distance), which for fewer takes longer.  Only
+    // where the bits are in shared memory: the others' sweeps lose 1% to it (893 cells 22.0 -> 22.2 ms).
+    const int most = (C + 127) / 128 * ((C + 127) / 128) * 144;
+    bool many = false;
     for (int t = lane; t < C; t += 32) {
       const Row q = unpack_row(rec[t]);
       pen += (long long)(1 - q.n) * (1 - q.n);
       v += q.n != 1;
       if (a.init && t + 1 < C && q.n > 0) {
         const Row p = unpack_row(rec[t + 1]);
-        if (q.n <= kRowCells) {
+        if (ROWS == kWide && SB && q.n * p.n > most) {
+          many = true;
+        } else if (q.n <= kRowCells) {
           hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c0);
           if (q.n > 1) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c1);
           if (q.n > 2) hd += row_sum_d<DT, DM, SB>(p, t + 1, bits, Cw, C, D, q.c2);
@@ -266,6 +370,8 @@ __device__ __forceinline__ void events_replica(const StructArgs &a, int rep, uin
         }
       }
     }
+    if (ROWS == kWide && SB && __any_sync(kFull, many))
+      hd += pairs_distance<DT, SB>(static_cast<const DT *>(a.d), a.Cp, C, bits, Cw, rec, most, lane);
     for (int i = lane; i < C; i += 32) {
       const int c = cc[i];
       pen += (long long)(1 - c) * (1 - c);
